@@ -19,8 +19,7 @@ memory (the kernel reads the queries and writes each converged row to host memor
 in place).
 
 Roofline: algorithmic bytes per launch come from the kernel's own per-query work
-counters (stops expanded, types examined, AP records read, relaxations), taken in an
-untimed pass over the same batches, times the fixed per-unit byte figures in BYTES
+counters (stops expanded, edges looked up, relaxations), taken in an untimed pass over the same batches, times the fixed per-unit byte figures in BYTES
 below.
 
 `--impl reference` times the CPU oracle (connection scan, Algorithm 1) on the host
@@ -49,12 +48,11 @@ BATCH = 256
 FLUSH_BYTES = 256 << 20
 FALLBACK_HBM_GBS = 6800.0
 
-# Per-unit algorithmic bytes of the method's data structures: per expanded stop 8 B frontier
-# entry + 4 B e[u] + 8 B row offsets; per examined type 16 B type record + 8 B pair of
-# cluster offsets + 4 B read of e[v] (charged on every examined type, also those that
-# stop early); per AP record examined 16 B; per relaxation 4 B atomic write + 8 B frontier
-# push; per query 4 B x V initialisation + 4 B x V result row.
-BYTES = {"vertices": 20, "types": 28, "aps": 16, "relaxed": 12}
+# Per-unit algorithmic bytes of the round kernel's data structures: per expanded stop 8 B
+# queue entry + 4 B e[u]; per looked-up edge 8 B record + 16 B slot entry + 4 B read of e[v];
+# per relaxation 4 B atomic write + 8 B queue entry; per query 4 B x V initialisation +
+# 4 B x V result row.
+BYTES = {"vertices": 12, "lookups": 28, "relaxed": 12}
 
 # DRAM bytes per query of the timed kernel, from the ncu captures summarised in profiles/
 # (the bench's own launches, dram__bytes_read.sum + dram__bytes_write.sum averaged over

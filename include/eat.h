@@ -151,12 +151,14 @@ typedef struct {
     int64_t vertices;  /* active stops expanded, summed over rounds (a stop with no
                           outgoing connection never needs expanding) */
     int64_t types;     /* connection types examined with an active tail: the
-                          "connections processed" of Section IV-C */
-    int64_t evals;     /* of the looked-up types, those with a departure at or after
-                          e[u] (their e[v] is read) */
-    int64_t lookups;   /* of the examined types, those whose cluster entry was read
-                          (Section II-D); types >= lookups >= evals */
-    int64_t aps;       /* AP records examined by the cluster lookup (Algorithm 6) */
+                          "connections processed" of Section IV-C (an edge entry of the
+                          round-based modes answers for all types of its edge) */
+    int64_t evals;     /* of the lookups, those that found a departure at or after e[u] */
+    int64_t lookups;   /* table entries read for the examined types: one per edge in the
+                          round-based modes (EAT_MODE_CTA, EAT_MODE_EDGE), one per type
+                          (Section II-D) in the others; types >= lookups >= evals */
+    int64_t aps;       /* departures (round-based modes) or AP records (Algorithm 6)
+                          examined by the lookups */
     int64_t relaxed;   /* relaxations that lowered e[v] (Algorithm 3): candidates below
                           the e[v] read just before the atomic min, so a candidate whose
                           atomic lost to a lower one made meanwhile is counted too */
@@ -173,7 +175,9 @@ typedef struct {
                                 paired mode or is on one network of 8,192 stops or more,
                                 else 512);
                                 else 64..1024, multiple of 32 */
-    int32_t vwarp;           /* lanes per active stop (1, 2, 4, 8, 16 or 32); 0 = automatic */
+    int32_t vwarp;           /* lanes per active stop (1, 2, 4, 8, 16 or 32), at most four of
+                                them in rounds with more stops than the block has
+                                sub-warps; 0 = automatic (8) */
     int32_t mode;            /* EAT_MODE_* */
     int32_t placement;       /* EAT_PLACE_*: where a query's arrivals and frontier
                                 bitmap live; 0 = automatic */
@@ -254,15 +258,9 @@ enum eat_mode {
                            takes the next query.  EAT_MODE_AUTO uses it only where
                            eat_autotune chose it; never in eat_query_batch_noalloc
                            unless requested */,
-    EAT_MODE_EDGE = 5   /* as EAT_MODE_CTA with two changes (the mapping chosen by degree
-                           and the warp min of Section II-F's warps): a stop with at least
-                           vwarp outgoing connection types is queued whole and expanded
-                           by a sub-warp of vwarp lanes (the whole warp for vwarp 32)
-                           instead of one item per type; and the lanes of a warp whose
-                           types share a head stop v reduce their candidates with a warp
-                           min, so that one lane per head stop reads e[v], lowers it and
-                           pushes v.  EAT_MODE_AUTO uses it only where eat_autotune
-                           chose it */
+    EAT_MODE_EDGE = 5   /* as EAT_MODE_CTA: a sub-warp of vwarp lanes per active stop and one
+                           relaxation per edge (Section II-E and II-F's warps), which is
+                           what the edge table gives every round-based launch */
 };
 
 /* Error message of the calling thread's last failed call ("" if none). */
@@ -624,7 +622,7 @@ void eat_server_destroy(eat_server *sv);
  *     (rounded up) for its frontier queue, plus n_stops / 4 bytes when the frontier
  *     bitmaps live in global memory (networks beyond about 900,000 stops), or
  *     16 * n_stops bytes in the paired mode (two queries per block); with a
- *     horizon, 16 * n_stops + n_stops / 8 bytes (the lists of waiting stops); the
+ *     horizon, 16 * n_stops bytes (the lists of waiting stops); the
  *     round-free mode needs none.  So the network may have at most 2,000,000 stops
  *     (about 1,000,000 with a horizon), and on large networks fewer blocks run at
  *     once while the other queries wait in the same launch.  Larger networks are

@@ -109,10 +109,9 @@ static int device_info(int dev, DeviceInfo &out) {
         DeviceGuard guard(dev);
         for (int nets : {1, EAT_MAX_NETS})
             for (int mem = 0; mem < 4; ++mem)
-                for (const void *k : {cta_kernel(nets, mem), cta_kernel(nets, mem, false, true),
-                                      async_kernel(nets, mem), cluster_kernel(), cta_kernel(1, 0, true),
-                                      cta_kernel(1, 0, true, true), cta_kernel(1, 0, true, false, true),
-                                      cta_kernel(1, 0, true, true, true), pair_kernel(false), pair_kernel(true),
+                for (const void *k : {cta_kernel(nets, mem), cta_kernel(nets, mem, true),
+                                      cta_kernel(nets, mem, false, true), async_kernel(nets, mem),
+                                      cluster_kernel(), pair_kernel(false), pair_kernel(true),
                                       ring_kernel(mem)}) {
                     e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)(d.smem_optin - d.reserve));
@@ -144,7 +143,6 @@ struct Plan {
     int nets = 1;
     bool async = false;           // round-free kernel (EAT_MODE_ASYNC)
     int cluster = 0;              // blocks per query in cluster mode (EAT_MODE_CLUSTER), else 0
-    bool pack = false;            // one int32 per queued item (small networks, shared arrivals)
     bool pair = false;            // two queries per block (EAT_MODE_PAIR)
     bool edge = false;            // warp min per head stop, degree-chosen mapping (EAT_MODE_EDGE)
     bool order = false;           // queries start by t_s (EAT_ORDER_BY_TIME): order array at off_order
@@ -154,7 +152,7 @@ struct Plan {
 
 static constexpr size_t kWsHeader = 256;   // work counter + internal status / counters
 static constexpr int32_t kDefaultIdleCap = 1 << 24;   // round-free mode's wait limit (full scans)
-static constexpr size_t kQueueEntryBytes = 16;  // (stop, type) item x 2 buffers
+static constexpr size_t kQueueEntryBytes = 16;  // 8-byte queue entry x 2 buffers
 
 // Default round cap: n_stops + 1 rounds always reach the fixpoint (every productive round
 // fixes one more stop); with a horizon, each move of the horizon can add one round in
@@ -283,7 +281,6 @@ static int make_pair_plan(int dev, const DeviceInfo &d, int32_t vmax, int32_t n,
     if (!net || vmax > 32767 || net->host.n_types > 65535)
         return fail(EAT_ERR_INVALID, "paired mode needs one network of at most 32,767 stops and 65,535 types");
     p.pair = true;
-    p.pack = true;
     p.mem = 0;
     p.async = false;
     p.nets = 1;
@@ -430,18 +427,15 @@ static int make_plan_core(int dev, int32_t vmax, int32_t n, int n_nets, const ea
     else if (place == EAT_PLACE_GLOBAL_ARR || (place == EAT_PLACE_AUTO && fits(1))) p.mem = 1;
     else p.mem = 2;
 
-    // Items take one int32 instead of two on one network small enough for the packed
-    // form (twice the queue in the same shared memory).
-    p.pack = p.mem == 0 && n_nets == 1 && tuned && vmax <= 32767 && tuned->host.n_types <= 65535;
     p.horizon = oh > 0 ? oh : (oh == 0 ? th : 0);
-    const size_t qbytes = p.pack ? kQueueEntryBytes / 2 : kQueueEntryBytes;
+    const size_t qbytes = kQueueEntryBytes;
     // Largest queue capacity that keeps the most blocks per SM the threads and the
     // registers allow (shared memory is the only other limit, and the one sized here).
     const size_t b0 = p.mem == 3 ? base(1) + (size_t)p.smem_arr_cap * 4 : base(p.mem);
     int reg_blocks = 0;
     {
         DeviceGuard guard(dev);
-        const void *k = cta_kernel(p.nets, p.mem, p.pack, false, p.horizon > 0);
+        const void *k = cta_kernel(p.nets, p.mem, false, p.horizon > 0);
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&reg_blocks, k, p.block, 0) != cudaSuccess) {
             cudaGetLastError();
             reg_blocks = 0;
@@ -467,13 +461,13 @@ static int make_plan_core(int dev, int32_t vmax, int32_t n, int n_nets, const ea
     {
         DeviceGuard guard(dev);
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-            &per_sm, cta_kernel(p.nets, p.mem, p.pack, false, p.horizon > 0), p.block, p.smem);
+            &per_sm, cta_kernel(p.nets, p.mem, false, p.horizon > 0), p.block, p.smem);
     }
     if (e != cudaSuccess) return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
     if (per_sm < 1) return fail(EAT_ERR_INVALID, "kernel does not fit on an SM with this block size");
     p.grid = (int)std::min<int64_t>((int64_t)std::max(n, 1), (int64_t)per_sm * d.sms);
-    // With a horizon a block also keeps two lists of waiting stops and their bitmap.
-    p.spill_stride = p.horizon > 0 ? (int64_t)align_up((size_t)vmax * 4 + (size_t)p.mask_words, 64)
+    // With a horizon a block also keeps two lists of waiting stops.
+    p.spill_stride = p.horizon > 0 ? (int64_t)align_up((size_t)vmax * 4, 64)
                                    : (int64_t)align_up((size_t)vmax * 2, 64);
     p.mask_stride = p.mem == 2 ? (int64_t)align_up(2 * (size_t)p.mask_words, 64) : 0;
     p.off_spill = kWsHeader;
@@ -540,7 +534,6 @@ static QueryArgs make_args(const Plan &p, int grid, char *ws, const int32_t *net
     qa.order = p.order ? (const int32_t *)(ws + p.off_order) : nullptr;
     qa.idle_cap = kDefaultIdleCap;
     qa.rg = RingArgs{};
-    qa.edge = p.edge ? 1 : 0;
     qa.horizon = p.horizon;
     return qa;
 }
@@ -603,11 +596,15 @@ static int run_batch(const eat_net *const *nets, int n_nets, const int32_t *net_
         if (e != cudaSuccess) return cuda_fail(e, "start-order kernel launch");
     }
     NetDev devs[EAT_MAX_NETS];
-    for (int i = 0; i < n_nets; ++i) devs[i] = nets[i]->dev;
+    EdgeDev edges[EAT_MAX_NETS];
+    for (int i = 0; i < n_nets; ++i) {
+        devs[i] = nets[i]->dev;
+        edges[i] = nets[i]->edev;
+    }
     e = p.cluster ? launch_cluster(devs[0], qa, p.cluster, p.grid, p.block, p.smem, st)
         : p.pair  ? launch_pair(devs[0], qa, p.grid, p.block, p.smem, st)
         : p.async ? launch_async(devs, n_nets, qa, p.mem, p.grid, p.block, p.smem, st)
-                  : launch_cta(devs, n_nets, qa, p.mem, p.grid, p.block, p.smem, st, p.pack);
+                  : launch_cta(edges, n_nets, qa, p.mem, p.grid, p.block, p.smem, st);
     if (e != cudaSuccess) return cuda_fail(e, "query kernel launch");
     return EAT_OK;
 }
@@ -679,8 +676,8 @@ int ring_launch(const eat_net *const *nets, int n_nets, const RingLaunch &rl, vo
         qa.arr_rows = arr_rows;
         qa.arr_rows_stride = rl.rows_stride;
     }
-    NetDev devs[EAT_MAX_NETS];
-    for (int i = 0; i < n_nets; ++i) devs[i] = nets[i]->dev;
+    EdgeDev devs[EAT_MAX_NETS];
+    for (int i = 0; i < n_nets; ++i) devs[i] = nets[i]->edev;
     DeviceGuard guard(nets[0]->device);
     cudaError_t e = launch_ring(devs, n_nets, qa, rl.mem, rl.grid, rl.block, rl.smem, st);
     if (e != cudaSuccess) return cuda_fail(e, "ring kernel launch");
@@ -712,12 +709,19 @@ static int upload(eat_net *net) {
         cudaGetLastError();
         return fail(EAT_ERR_NO_DEVICE, "no CUDA device " + std::to_string(net->device));
     }
-    const HostNet &h = net->host;
+    rc = build_edges(net->host);
+    if (rc) return rc;
+    HostNet &h = net->host;
     size_t off_row = 0;
     size_t off_tr = align_up(off_row + ((size_t)h.n_stops + 1) * 4, 256);
     size_t off_ce = align_up(off_tr + h.tr.size() * 4, 256);
     size_t off_apx = align_up(off_ce + h.ce.size() * 4, 256);
-    size_t total = align_up(off_apx + h.apx.size() * 4 + 16, 256);
+    size_t off_erow = align_up(off_apx + h.apx.size() * 4 + 16, 256);
+    size_t off_er = align_up(off_erow + h.erow.size() * 4, 256);
+    size_t off_ee = align_up(off_er + h.er.size() * 4, 256);
+    size_t off_ex = align_up(off_ee + h.ee.size() * 4, 256);
+    size_t off_et = align_up(off_ex + h.ex.size() * 4, 256);
+    size_t total = align_up(off_et + h.etypes.size() * 4 + 16, 256);
     DeviceGuard guard(net->device);
     if (!guard.ok) return fail(EAT_ERR_NO_DEVICE, "cudaSetDevice failed");
     e = cudaMalloc(&net->blob, total);
@@ -733,6 +737,11 @@ static int upload(eat_net *net) {
         {off_tr, h.tr.data(), h.tr.size() * 4},
         {off_ce, h.ce.data(), h.ce.size() * 4},
         {off_apx, h.apx.data(), h.apx.size() * 4},
+        {off_erow, h.erow.data(), h.erow.size() * 4},
+        {off_er, h.er.data(), h.er.size() * 4},
+        {off_ee, h.ee.data(), h.ee.size() * 4},
+        {off_ex, h.ex.data(), h.ex.size() * 4},
+        {off_et, h.etypes.data(), h.etypes.size() * 4},
     };
     for (const Piece &pc : pieces) {
         if (!pc.bytes) continue;
@@ -751,6 +760,20 @@ static int upload(eat_net *net) {
     d.inv_width = 1.0f / (float)h.width;
     d.k_min = h.k_min;
     d.y = h.y;
+    EdgeDev &x = net->edev;
+    x.erow = (const int32_t *)(b + off_erow);
+    x.er = (const int2 *)(b + off_er);
+    x.ee = (const int4 *)(b + off_ee);
+    x.ex = (const int2 *)(b + off_ex);
+    x.etypes = (const int32_t *)(b + off_et);
+    x.n_stops = h.n_stops;
+    x.n_edges = (int32_t)h.etypes.size();
+    x.base = h.e_base;
+    x.shift = h.e_shift;
+    x.y = h.e_y;
+    x.big = h.n_stops > kMaxPackedStops;
+    // No host view shows the edge table: its host copy goes.
+    for (std::vector<int32_t> *w : {&h.erow, &h.er, &h.ee, &h.ex, &h.etypes}) std::vector<int32_t>().swap(*w);
     return EAT_OK;
 }
 
@@ -1491,7 +1514,7 @@ extern "C" int eat_query_batch_noalloc(const eat_net *net, const int32_t *source
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync(no-allocation scratch)");
     e = p.pair    ? launch_pair(net->dev, qa, grid, p.block, p.smem, st)
         : p.async ? launch_async(&net->dev, 1, qa, p.mem, grid, p.block, p.smem, st)
-                  : launch_cta(&net->dev, 1, qa, p.mem, grid, p.block, p.smem, st, p.pack);
+                  : launch_cta(&net->edev, 1, qa, p.mem, grid, p.block, p.smem, st);
     if (e != cudaSuccess) return cuda_fail(e, "query kernel launch");
     return EAT_OK;
 }

@@ -608,4 +608,213 @@ int build_fused(HostNet &h) {
     return EAT_OK;
 }
 
+// Edge table (see EdgeDev in eat_internal.h): per edge the merged departures of all its
+// connection types without dominated ones, cut into time slots of 2^shift seconds.
+int build_edges(HostNet &h) {
+    const int32_t V = h.n_stops, W = h.width, t0 = h.t0;
+    struct Pair { int32_t dep, arr; };
+    struct Part {
+        int32_t u_begin = 0, u_end = 0;
+        std::vector<int32_t> per_u, head, types;      // edges per stop; head and types per edge
+        std::vector<int64_t> ptr;                     // first pair of each edge
+        std::vector<Pair> pairs;
+        std::vector<int32_t> ex;
+        int64_t quads = 0;
+        bool oom = false;
+    };
+    const unsigned hw = std::max(1u, std::min(32u, std::thread::hardware_concurrency()));
+    const int n_parts = (int)std::min<int64_t>((int64_t)hw * 4, V);
+    std::vector<Part> parts((size_t)n_parts);
+    {
+        int32_t u = 0;                                // about equal numbers of types
+        for (int k = 0; k < n_parts; ++k) {
+            const int64_t target = ((int64_t)h.n_types * (k + 1)) / n_parts;
+            parts[k].u_begin = u;
+            int32_t e = u;
+            if (k == n_parts - 1) e = V;
+            else while (e < V && h.row_ptr[e] < target) ++e;
+            parts[k].u_end = u = e;
+        }
+    }
+    auto run = [&](auto fn) {
+        std::atomic_int next{0};
+        auto work = [&] {
+            for (int k; (k = next.fetch_add(1)) < n_parts;) {
+                try {
+                    fn(parts[k]);
+                } catch (const std::bad_alloc &) {
+                    parts[k].oom = true;
+                }
+            }
+        };
+        std::vector<std::thread> th;
+        for (unsigned i = 1; i < hw; ++i) th.emplace_back(work);
+        work();
+        for (auto &t : th) t.join();
+        for (const Part &p : parts)
+            if (p.oom) return false;
+        return true;
+    };
+    // Per edge: every (departure, arrival), sorted; from the back, an arrival that is not
+    // below all later ones' is dominated.
+    const bool ok = run([&](Part &p) {
+        std::vector<int32_t> ts;
+        std::vector<Pair> all;
+        p.ptr.push_back(0);
+        for (int32_t u = p.u_begin; u < p.u_end; ++u) {
+            ts.resize((size_t)(h.row_ptr[u + 1] - h.row_ptr[u]));
+            for (size_t i = 0; i < ts.size(); ++i) ts[i] = h.row_ptr[u] + (int32_t)i;
+            auto head = [&](int32_t t) { return h.type_rec[4 * (size_t)t]; };
+            std::stable_sort(ts.begin(), ts.end(), [&](int32_t a, int32_t b) { return head(a) < head(b); });
+            int32_t n_edges = 0;
+            for (size_t i = 0, j; i < ts.size(); i = j) {
+                all.clear();
+                for (j = i; j < ts.size() && head(ts[j]) == head(ts[i]); ++j) {
+                    const int32_t *r = &h.type_rec[4 * (size_t)ts[j]];
+                    for (int32_t k = (r[2] - t0) / W; k <= (r[3] - t0) / W; ++k)
+                        for (int32_t a = h.cl[h.type_cl[ts[j]] + k]; a < h.cl[h.type_cl[ts[j]] + k + 1]; ++a) {
+                            const int32_t first = (int32_t)h.ap[2 * (size_t)a];
+                            const uint32_t sc = h.ap[2 * (size_t)a + 1];
+                            const int32_t n = (int32_t)(sc & 0xffffu), step = (int32_t)(sc >> 16);
+                            for (int32_t m = 0; m < n; ++m)
+                                all.push_back({first + m * step, first + m * step + r[1]});
+                        }
+                }
+                std::sort(all.begin(), all.end(), [](const Pair &a, const Pair &b) {
+                    return a.dep < b.dep || (a.dep == b.dep && a.arr < b.arr);
+                });
+                size_t keep = all.size();
+                int32_t best = EAT_INF;
+                for (size_t m = all.size(); m-- > 0;)
+                    if (all[m].arr < best) {
+                        best = all[m].arr;
+                        if (keep == all.size() || all[keep].dep != all[m].dep) --keep;
+                        all[keep] = all[m];
+                    }
+                p.pairs.insert(p.pairs.end(), all.begin() + (ptrdiff_t)keep, all.end());
+                p.ptr.push_back((int64_t)p.pairs.size());
+                p.head.push_back(head(ts[i]));
+                p.types.push_back((int32_t)(j - i));
+                ++n_edges;
+            }
+            p.per_u.push_back(n_edges);
+        }
+    });
+    if (!ok) return fail(EAT_ERR_OOM, "host allocation of the edge table failed");
+
+    int64_t E = 0, n_pairs = 0;
+    int32_t first = EAT_INF, last = INT32_MIN;
+    std::vector<int64_t> e_off((size_t)n_parts);
+    for (int k = 0; k < n_parts; ++k) {
+        e_off[k] = E;
+        E += (int64_t)parts[k].head.size();
+        n_pairs += (int64_t)parts[k].pairs.size();
+        for (size_t e = 0; e < parts[k].head.size(); ++e) {
+            first = std::min(first, parts[k].pairs[(size_t)parts[k].ptr[e]].dep);
+            last = std::max(last, parts[k].pairs[(size_t)parts[k].ptr[e + 1] - 1].dep);
+        }
+    }
+    h.e_base = E ? first : 0;
+    h.e_shift = 0;
+    h.e_y = 0;
+    if (E) {
+        // Slots of about one departure of an edge on average (the largest power of two up
+        // to the mean headway): an entry holds two inside the slot and the first one after
+        // it, so few lookups go on to the list.  Wider only to keep the table within 2 GB,
+        // or within the cluster table's size where that is larger.
+        const int64_t span = (int64_t)last - first + 1;
+        const double headway = (double)span * (double)E / (double)n_pairs;
+        auto slots = [&](int32_t s) { return ((int64_t)last - first) / ((int64_t)1 << s) + 1; };
+        int32_t s = 3;
+        while (s < 15 && (double)((int64_t)2 << s) <= headway) ++s;
+        const int64_t most = std::max((int64_t)2 << 30, (int64_t)h.n_types * h.y * 32);
+        while (s < 15 && E * slots(s) * 16 > most) ++s;
+        h.e_shift = s;
+        h.e_y = (int32_t)slots(s);
+    }
+    try {
+        h.erow.assign((size_t)V + 1, 0);
+        h.er.assign((size_t)E * 2, 0);
+        h.etypes.assign((size_t)E, 0);
+        h.ee.assign((size_t)E * (size_t)h.e_y * 4, 0);
+    } catch (const std::bad_alloc &) {
+        return fail(EAT_ERR_OOM, "host allocation of the edge table failed");
+    }
+    {
+        int32_t r = 0;
+        for (const Part &p : parts)
+            for (size_t i = 0; i < p.per_u.size(); ++i) {
+                h.erow[(size_t)p.u_begin + i] = r;
+                r += p.per_u[i];
+            }
+        h.erow[V] = r;
+    }
+    // Entries, with list offsets local to the part; the lists' places follow from their sizes.
+    const bool big = V > kMaxPackedStops;
+    auto fill = [&](Part &p) {
+        const int64_t e0 = e_off[&p - parts.data()];
+        for (size_t e = 0; e < p.head.size(); ++e) {
+            const int32_t v = p.head[e], d = std::min(h.erow[v + 1] - h.erow[v], kCountOverflow);
+            int32_t *r = &h.er[2 * (size_t)(e0 + (int64_t)e)];
+            r[0] = big ? v : (int32_t)((uint32_t)v | (uint32_t)d << 24);
+            r[1] = h.erow[v];
+            h.etypes[(size_t)(e0 + (int64_t)e)] = p.types[e];
+            const Pair *q = p.pairs.data() + p.ptr[e], *const end = p.pairs.data() + p.ptr[e + 1];
+            for (int32_t k = 0; k < h.e_y; ++k) {
+                const int64_t lo = (int64_t)h.e_base + ((int64_t)k << h.e_shift);
+                const int64_t hi = lo + ((int64_t)1 << h.e_shift);
+                while (q < end && q->dep < lo) ++q;
+                const Pair *z = q;
+                while (z < end && z->dep < hi) ++z;
+                if (z < end) ++z;                     // the first departure after the slot
+                uint32_t dep[3], dur[3] = {0, 0, 0};
+                const Pair *m = q;
+                for (int j = 0; j < 3; ++j) {
+                    dep[j] = (uint32_t)kNoDeparture;
+                    if (m == q + j && m < z && m->dep - lo < kNoDeparture && m->arr - m->dep <= 0xffff) {
+                        dep[j] = (uint32_t)(m->dep - lo);
+                        dur[j] = (uint32_t)(m->arr - m->dep);
+                        ++m;
+                    }
+                }
+                int32_t *w = &h.ee[((size_t)k * (size_t)E + (size_t)(e0 + (int64_t)e)) * 4];
+                for (int j = 0; j < 3; ++j) w[j] = (int32_t)(dep[j] | dur[j] << 16);
+                w[3] = 0;
+                if (m == z) continue;
+                w[3] = (int32_t)(p.quads + 1);
+                const bool open = z == end && z[-1].dep < hi;   // nothing after the slot
+                for (; m < z; ++m) p.ex.insert(p.ex.end(), {m->dep, m->arr});
+                if (open) p.ex.insert(p.ex.end(), {EAT_INF, EAT_INF});
+                while (p.ex.size() % 8) p.ex.push_back(EAT_INF);
+                p.quads = (int64_t)p.ex.size() / 8;
+            }
+        }
+        std::vector<Pair>().swap(p.pairs);
+    };
+    if (!run(fill)) return fail(EAT_ERR_OOM, "host allocation of the edge table failed");
+    std::vector<int64_t> q_off((size_t)n_parts);
+    int64_t quads = 0;
+    for (int k = 0; k < n_parts; ++k) {
+        q_off[k] = quads;
+        quads += parts[k].quads;
+    }
+    if (quads >= INT32_MAX) return fail(EAT_ERR_INVALID, "edge lists too large for 32-bit indices");
+    try {
+        h.ex.resize((size_t)quads * 8);
+    } catch (const std::bad_alloc &) {
+        return fail(EAT_ERR_OOM, "host allocation of the edge table failed");
+    }
+    run([&](Part &p) {
+        const size_t k = (size_t)(&p - parts.data());
+        std::copy(p.ex.begin(), p.ex.end(), h.ex.begin() + q_off[k] * 8);
+        if (!q_off[k]) return;
+        for (int32_t s = 0; s < h.e_y; ++s)
+            for (size_t e = 0; e < p.head.size(); ++e) {
+                int32_t &x = h.ee[((size_t)s * (size_t)E + (size_t)e_off[k] + e) * 4 + 3];
+                if (x) x += (int32_t)q_off[k];
+            }
+    });
+    return EAT_OK;
+}
+
 }  // namespace eat

@@ -13,6 +13,13 @@
 
 #include "eat.h"
 
+// Functions that the kernels and the host (tests of the layouts) share.
+#ifdef __CUDACC__
+#define EAT_HD __host__ __device__
+#else
+#define EAT_HD
+#endif
+
 namespace eat {
 
 // Device-side descriptor of one resident network (plain pointers into one blob).
@@ -34,9 +41,48 @@ namespace eat {
 //                 next = first departure of the next non-empty cluster (INF if none)
 //   apx[]         uint2 {first term, sc} of the fifth and later APs of a cluster
 //   row_ptr[V+1]  types leaving stop u are row_ptr[u] .. row_ptr[u+1]-1
+// and the edge table that the round kernel reads (see EdgeDev; build_edges).
 constexpr int32_t kCountOverflow = 255;
 constexpr int32_t kMaxDuration = 1 << 24;
 constexpr int32_t kInlineAps = 4;
+
+// The network by edges (u, v) and time slots of 2^shift seconds.  An edge's connections of
+// every duration are merged into one list ordered by departure, without those that another
+// one dominates (departs no earlier, arrives no later): the earliest arrival over the edge
+// for a tail reached at e is then the arrival of the first listed departure >= e, one
+// relaxation for the edge instead of one per connection type (Section II-E).
+//   er[i]        8-byte record of edge i: {v | d << 24, erow[v]}: head stop, edges leaving
+//                it (255 = read erow), its first edge; networks of more than 2^24 stops:
+//                {v, erow[v]}, d always read from erow
+//   ee[k*E + i]  16-byte entry of edge i for slot k, slot-major (a round's lookups are at
+//                nearby times and fall in few slabs): the listed departures inside the slot
+//                and the first one after it, the first three as 16-bit numbers
+//                {d0 | l0 << 16, d1 | l1 << 16, d2 | l2 << 16, x}: departure d (relative to
+//                the slot's start, 0xffff = none), duration l; the others (or values that
+//                do not fit 16 bits) from ex[4 * (x - 1)] on, x = 0 if there are none
+//   ex[]         {departure, arrival} pairs, each list a multiple of four pairs (32 bytes)
+//                ended by the first departure after the slot or by {INF, INF}
+//   erow[V+1]    edges leaving stop u are erow[u] .. erow[u+1]-1
+// Against one 16-byte record and one 32-byte entry per (type, cluster) this reads 24 bytes
+// per edge, where an edge has two (city) or three (large) types of which half have no
+// departure left: a large query of a 1,024-query step looks up 65,000 edges instead of
+// 194,000 types, and the table takes 0.7 GB instead of 5.1 GB.
+constexpr int32_t kNoDeparture = 0xffff;
+constexpr int32_t kMaxPackedStops = 1 << 24;
+
+struct EdgeDev {
+    const int32_t *erow;      // [V + 1]
+    const int2 *er;           // [E]
+    const int4 *ee;           // [y * E], slot-major
+    const int2 *ex;
+    const int32_t *etypes;    // [E] connection types of each edge (work counters only)
+    int32_t n_stops;
+    int32_t n_edges;
+    int32_t base;             // start of slot 0 (the network's first departure)
+    int32_t shift;            // slots of 2^shift seconds
+    int32_t y;                // slots
+    int32_t big;              // more than 2^24 stops: er holds no degree
+};
 
 struct NetDev {
     const int32_t *row_ptr;   // [V + 1] types by tail stop
@@ -52,10 +98,38 @@ struct NetDev {
     int32_t y;                // clusters stored per type
 };
 
+// Slot of time e and e relative to the slot's start; e before the first slot counts as its
+// start (every departure is then >= e).  A slot >= E.y: no departure at or after e.
+EAT_HD inline uint32_t edge_slot(int32_t base, int32_t shift, int32_t e, uint32_t &rel) {
+    const uint32_t d = e > base ? (uint32_t)e - (uint32_t)base : 0u;
+    rel = d & ((1u << shift) - 1u);
+    return d >> shift;
+}
+
+// Start time of slot k.
+EAT_HD inline int32_t edge_slot_start(int32_t base, int32_t shift, uint32_t k) {
+    return (int32_t)((uint32_t)base + (k << shift));
+}
+
+// Earliest arrival over an edge from its entry c for a tail reached at `rel` in the slot that
+// starts at `start`, from the three inline departures; EAT_INF if none of them is at or after
+// it (the list, if c.w is set, has the others).
+EAT_HD inline int32_t edge_inline(const int4 c, uint32_t rel, int32_t start) {
+    const uint32_t x = (uint32_t)c.x, y = (uint32_t)c.y, z = (uint32_t)c.z;
+    const uint32_t p = rel <= (x & 0xffffu) ? x : rel <= (y & 0xffffu) ? y : z;
+    const uint32_t d = p & 0xffffu;
+    return rel <= d && d != (uint32_t)kNoDeparture ? (int32_t)((uint32_t)start + d + (p >> 16)) : EAT_INF;
+}
+
 // Up to NETS networks passed by value as a kernel parameter.
 template <int NETS>
 struct NetTable {
     NetDev net[NETS];
+};
+
+template <int NETS>
+struct EdgeTable {
+    EdgeDev net[NETS];
 };
 
 // Host copy of the built arrays (kept for eat_net_host_view).
@@ -74,6 +148,13 @@ struct HostNet {
     std::vector<int32_t> tr;         // 4 T
     std::vector<int32_t> ce;         // 8 T y
     std::vector<uint32_t> apx;       // 2 n_apx
+    // Edge table (see EdgeDev).
+    int32_t e_base = 0, e_shift = 0, e_y = 0;
+    std::vector<int32_t> erow;       // V + 1
+    std::vector<int32_t> er;         // 2 E
+    std::vector<int32_t> ee;         // 4 E e_y
+    std::vector<int32_t> ex;         // 2 per pair
+    std::vector<int32_t> etypes;     // E
 };
 
 }  // namespace eat
@@ -84,6 +165,7 @@ struct eat_net {
     void *blob = nullptr;            // one cudaMalloc holding every array
     int64_t blob_bytes = 0;
     eat::NetDev dev{};
+    eat::EdgeDev edev{};
     // Internal workspace and staging buffers (eat_query, NULL-workspace batches).
     mutable std::mutex ws_lock;
     mutable void *ws = nullptr;
@@ -116,6 +198,9 @@ int build_host_csr(const eat_csr_input *in, int32_t width, int32_t t0, HostNet &
 
 // Device layout from the logical arrays (eat_build.cpp).
 int build_fused(HostNet &h);
+
+// Edge table from the logical arrays (eat_build.cpp).
+int build_edges(HostNet &h);
 
 // Greedy AP cover of sorted unique values (eat_build.cpp); appends (first, step, terms).
 void ap_cover(const int32_t *vals, int32_t n, int32_t width_hint,

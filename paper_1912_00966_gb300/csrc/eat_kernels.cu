@@ -19,24 +19,24 @@
 // mode (eat_async_kernel) and the cluster mode (eat_cluster_kernel) are
 // described at their kernels below.
 //
-// Work items: when a stop v joins the next frontier, the thread that lowered e[v]
-// writes one (v, type) item per connection type leaving v into shared memory (one
-// 32- or 64-bit store each), so the next round hands every thread one (stop, type)
-// pair: the paper's one thread per connection type (Algorithm 5), restricted to the
-// active tails.  Per item, the type's 16-byte record (head, duration, head row, last
-// departure) and e[u] are loaded together, then the 32-byte cluster entry of e[u]'s
-// cluster, then e[v] beside any further APs.  Stops whose items do not fit spill to a
-// global queue and are expanded by `vwarp`-lane sub-warps (Section II-F's virtual
-// warps).
+// The round kernel (eat_cta_kernel) reads the network by edges (EdgeDev in
+// eat_internal.h): all connection types of an edge (u, v) are merged, per time slot, into one
+// 16-byte entry, so that an edge is one lookup and one relaxation (Section II-E).  The
+// frontier is a queue of stops in shared memory: the thread that lowers e[v] stores
+// {v, degree, first edge} (8 bytes, taken from the edge's record), and the next round
+// gives each queued stop a sub-warp (Section II-F's virtual warps) whose lanes take its
+// edges.  Per lane: the queue entry and e[u] (the same for the sub-warp), the edge's 8-byte
+// record, then the 16-byte entry of e[u]'s slot beside e[v].  Queue entries past the shared
+// buffer spill to global memory.
 //
 // Horizon (qa.horizon > 0, an option; not in the paper): Algorithms 4-5 expand every
 // improved stop in the next round, so a stop first reached late by a path of few
 // connections is expanded, and its successors with it, again each time a later round
 // improves it.  With a horizon H a stop lowered to an arrival >= H is not queued but
-// waits (once, in a per-block list with a bitmap); when no stop below H is left to
-// expand, waiting stops whose arrival has since dropped below H are dropped (they
-// were queued by that lowering), H moves to the earliest remaining arrival + horizon,
-// and the stops below the new H become the next round's spilled stops.  Every
+// waits (once, in a per-block list: the thread whose atomic min found it unreached adds
+// it); when no stop below H is left to expand, H moves to the least arrival given to a
+// waiting stop + horizon, waiting stops below the new H are queued, and those whose arrival
+// had dropped below the old H are dropped (they were queued by that lowering).  Every
 // lowered stop is still expanded with its arrival at some round after the lowering,
 // so the fixpoint is the same; only the order of relaxations changes (as
 // delta-stepping orders Bellman-Ford's).
@@ -136,52 +136,62 @@ __device__ __forceinline__ void ring_done(const RingArgs &R, int32_t slot, int32
 constexpr int32_t kNullItem = -1;           // hole left by a stop that spilled
 constexpr int32_t kFirstItem = INT32_MIN;    // flag on the first item of a stop
 
-// Items are (stop, type) pairs in two int32 arrays per buffer, or, with PACK (networks
-// of at most 32,767 stops and 65,535 types), one word per item: first-item flag << 31 |
-// stop << 16 | type, which doubles the items a buffer holds in the same shared memory
-// (kNullItem is then no valid item: it would be stop 32,767, type 65,535).
+// `n` words of `p` (any 4-byte alignment) set to kInf by the block's threads, 16 bytes a
+// store between the first and the last 16-byte boundary.
+__device__ __forceinline__ void fill_inf(int32_t *p, int32_t n, int tid, int nthr) {
+    const int32_t head = min(n, (int32_t)((4 - ((reinterpret_cast<uintptr_t>(p) >> 2) & 3)) & 3));
+    const int32_t n4 = (n - head) >> 2;
+    if (tid < head) p[tid] = kInf;
+    int4 *const q = reinterpret_cast<int4 *>(p + head);
+    for (int32_t i = tid; i < n4; i += nthr) q[i] = make_int4(kInf, kInf, kInf, kInf);
+    const int32_t done = head + 4 * n4;
+    if (tid < n - done) p[done + tid] = kInf;
+}
+
+// Bound by the chain of dependent loads of a round (queue entry and e[u], then the edge's
+// record and entry, then e[v] and the atomics on the queue) times the rounds of the deepest
+// query, not by bandwidth.  Against one thread per (stop, connection type) item with the
+// 32-byte cluster entries (us per step, the same shapes): grid 256 queries 117 -> 69, city
+// 256 queries 531 -> 353, city 37 queries on hourly clusters 690 -> 290, 60,000 stops 300
+// queries 3,766 -> 2,019, large 96 queries 4,353 -> 2,889 and 1,024 queries with a horizon of
+// one hour 6,452 -> 4,230, 64 ragged networks 4,096 queries 1,979 -> 1,505.
 // COUNT: the build that fills qa.counters; without it the per-thread work counters are
 // dead code and compiled away (the timed launches pass no counters).  HZ: the build that
-// honours qa.horizon (the packed build also comes without, for launches with none).
-template <int NETS, int ARR, bool SMEM_MASK, bool PACK = false, bool RING = false, bool COUNT = false,
-          bool HZ = true>
+// honours qa.horizon.
+template <int NETS, int ARR, bool SMEM_MASK, bool RING = false, bool COUNT = false, bool HZ = true>
 __global__ void __launch_bounds__(1024, 1)
-eat_cta_kernel(const __grid_constant__ NetTable<NETS> nets, const QueryArgs qa) {
+eat_cta_kernel(const __grid_constant__ EdgeTable<NETS> nets, const QueryArgs qa) {
     extern __shared__ __align__(16) int32_t smem[];
     __shared__ int32_t s_q;
     __shared__ int32_t s_ring[4];     // ring mode: net, source, t_s, row of the request
-    __shared__ int32_t s_items[3];    // items reserved per round (rotating)
-    __shared__ int32_t s_spill[3];    // stops spilled per round (rotating)
+    __shared__ int32_t s_n[3];        // stops queued per round (rotating)
+    __shared__ int32_t s_wait[2];     // stops in either waiting list
+    __shared__ int32_t s_min[2];      // least arrival given to a stop waiting in it
+    __shared__ int32_t s_rel[2];      // stops released from it
     __shared__ unsigned long long s_cnt[6];
-    __shared__ int32_t s_def[4];      // waiting stops: count, kept, released, least arrival
 
     const int tid = threadIdx.x;
     const int nthr = blockDim.x;
-    const int vw = 1 << qa.vw_log2;
-    const int lane = tid & (vw - 1);
-    const int sub = tid >> qa.vw_log2;
-    const int nsub = nthr >> qa.vw_log2;
-    const int32_t icap = qa.qcap;
+    const int32_t qcap = qa.qcap;
 
-    // Item buffers (stop, type) and spill queues; round r writes buffer r & 1.
-    int32_t *const item_base = smem + qa.smem_q_off;
+    // Stop queues and spilled stops; round r writes buffer r & 1.
+    int2 *const queue = reinterpret_cast<int2 *>(smem + qa.smem_q_off);
     int32_t *const spill_base = qa.spill + (int64_t)blockIdx.x * qa.spill_stride;
     uint32_t *const mask_base = SMEM_MASK ? (uint32_t *)(smem + qa.smem_mask_off)
                                           : qa.gmask + (int64_t)blockIdx.x * qa.mask_stride;
-    // Stops waiting beyond the horizon: two lists of vmax stops and their bitmap.
-    int32_t *const def_base = spill_base + 2 * (int64_t)qa.vmax;
-    uint32_t *const dmask = (uint32_t *)(spill_base + 4 * (int64_t)qa.vmax);
+    // Stops waiting beyond the horizon: two lists of vmax stops.
+    int32_t *const wait_base = spill_base + 2 * (int64_t)qa.vmax;
 
     for (;;) {
         if (tid == 0) s_q = RING ? ring_next(qa.rg, s_ring) : next_query(qa);
-        if (tid < 6) s_cnt[tid] = 0;
+        if (COUNT && tid < 6) s_cnt[tid] = 0;
         __syncthreads();
         const int q = s_q;
         if (RING ? q < 0 : q >= qa.n) break;
 
         const int ni = RING ? s_ring[0] : qa.net_idx == nullptr ? 0 : __ldg(qa.net_idx + q);
         const bool net_ok = (unsigned)ni < (unsigned)qa.n_nets;
-        const NetDev &N = nets.net[net_ok ? ni : 0];
+        const EdgeDev &N = nets.net[net_ok ? ni : 0];
         const int32_t V = N.n_stops;
         const int64_t off = RING         ? (int64_t)s_ring[3] * qa.rg.row_stride
                             : qa.arr_off ? __ldg(qa.arr_off + q)
@@ -198,258 +208,176 @@ eat_cta_kernel(const __grid_constant__ NetTable<NETS> nets, const QueryArgs qa) 
         uint32_t *const mask1 = mask_base + qa.mask_words;
 
         // Algorithm 2: every stop passive at infinity.
-        for (int32_t i = tid; i < V; i += nthr) arr[i] = kInf;
+        fill_inf(arr, V, tid, nthr);
         for (int32_t i = tid; i < nwords; i += nthr) {
             mask0[i] = 0u;
             mask1[i] = 0u;
         }
         const bool hz_on = HZ && qa.horizon > 0;
-        if (hz_on)
-            for (int32_t i = tid; i < nwords; i += nthr) dmask[i] = 0u;
-        if (tid < 3) {
-            s_items[tid] = 0;
-            s_spill[tid] = 0;
+        if (tid < 3) s_n[tid] = 0;
+        if (HZ && tid < 2) {
+            s_wait[tid] = 0;
+            s_min[tid] = kInf;
+            s_rel[tid] = 0;
         }
-        if (tid == 0) s_def[0] = 0;
         const int32_t s = RING ? s_ring[1] : __ldg(qa.src + q);
         const int32_t t_s = RING ? s_ring[2] : __ldg(qa.ts + q);
         const bool valid = net_ok && (unsigned)s < (unsigned)V;
         __syncthreads();
-        // The source is the frontier of "round -1": spill queue of buffer 1, counter slot 2.
+        // The source is the frontier of "round -1": buffer 1.
         if (tid == 0 && valid) {
             arr[s] = t_s;
-            spill_base[qa.vmax] = s;
-            s_spill[2] = 1;
+            const int32_t row = __ldg(N.erow + s);
+            const int32_t d = min(__ldg(N.erow + s + 1) - row, kCountOverflow);
+            queue[qcap] = make_int2(N.big ? s : (int32_t)((uint32_t)s | (uint32_t)d << 24), row);
         }
         __syncthreads();
 
-        int32_t n_items = 0, n_spill = valid ? 1 : 0;
+        int32_t n = valid ? 1 : 0;
         int32_t rounds = 0;
         // Horizon H (kInf when there is none): a stop lowered to an arrival at or after
         // H waits until no stop below H is left to expand.
         int32_t H = hz_on && t_s < kInf - qa.horizon ? t_s + qa.horizon : kInf;
-        int dl = 0;                                       // list that new waiting stops join
+        int wl = 0;                                       // list that new waiting stops join
         int cs = 0;                                       // counter slot written this round
         int32_t c_vert = 0, c_types = 0, c_evals = 0, c_lookups = 0, c_aps = 0, c_relax = 0;
-        while (n_items + n_spill > 0 && rounds < qa.max_rounds) {
+        while (n > 0 && rounds < qa.max_rounds) {
             const int wr = rounds & 1, rd = wr ^ 1;
-            // One-word items (PACK) or two-word items {stop | first flag, type}.
-            int32_t *const iu_rd = item_base + (PACK ? rd : 2 * rd) * icap;
-            int32_t *const iu_wr = item_base + (PACK ? wr : 2 * wr) * icap;
-            const int2 *const i2_rd = reinterpret_cast<const int2 *>(iu_rd);
-            int2 *const i2_wr = reinterpret_cast<int2 *>(iu_wr);
+            const int2 *const q_rd = queue + rd * qcap;
+            int2 *const q_wr = queue + wr * qcap;
             const int32_t *const sp_rd = spill_base + (int64_t)rd * qa.vmax;
             int32_t *const sp_wr = spill_base + (int64_t)wr * qa.vmax;
-            uint32_t *const pmask = wr ? mask1 : mask0;    // stops pushed this round
-            uint32_t *const cmask = wr ? mask0 : mask1;    // stops pushed last round
+            uint32_t *const pmask = wr ? mask1 : mask0;    // stops queued this round
+            uint32_t *const cmask = wr ? mask0 : mask1;    // stops queued last round
             // The slot used next round was last read two barriers ago.
-            if (tid == 0) {
-                const int nx = cs == 2 ? 0 : cs + 1;
-                s_items[nx] = 0;
-                s_spill[nx] = 0;
-            }
+            if (tid == 0) s_n[cs == 2 ? 0 : cs + 1] = 0;
 
-            // Relaxation (Algorithm 3 with getConnection, Algorithm 6) in two steps.
-            // lookup: t_c + lambda of one type of tail u from its cluster entry and type
-            // record, for e[u] at or before the type's last departure (so that some
-            // departure is at or after e[u]).  lower: when that candidate is below the
-            // e[v] read beside the lookup, e[v] is lowered with an atomic min whose result
-            // is not waited for and v goes on the next frontier as items or as a spilled
-            // stop: every lowering is made by a thread whose candidate was below its read,
-            // so every lowering pushes v (at most once a round: the bitmap); a push whose
-            // min lost to a lower one made meanwhile only repeats work.  In EAT_MODE_EDGE
-            // a stop with at least vwarp types is queued whole for a vwarp-lane sub-warp
-            // (the mapping chosen by degree).
-            auto lookup = [&](int32_t e_u, int32_t k, const int4 ca, const int4 cb,
-                              const int4 tr) -> int32_t {  // tr = {v, lambda|d, row of v, last}
-                ++c_lookups;
-                ++c_evals;
-                int32_t n, x;
-                entry_aps(cb, n, x);
-                return cluster_lookup(ca, cb, n, x, cluster_base(N, k), e_u, N.apx, c_aps) +
-                       (tr.y & 0xffffff);
-            };
-            auto lower = [&](const int4 tr, int32_t cand, int32_t ev) {
+            // Relaxation (Algorithm 3): when the candidate is below the e[v] read beside the
+            // lookup, e[v] is lowered with an atomic min whose result is not waited for and
+            // v goes on the next frontier: every lowering is made by a thread whose
+            // candidate was below its read, so every lowering queues v (at most once a
+            // round: the bitmap); a stop queued by a min that lost to a lower one made
+            // meanwhile only repeats work.  Beyond the horizon the result is waited for
+            // when e[v] was read as infinite: a stop with an arrival at or after H waits in
+            // the list already, so the one thread that finds it unreached adds it.
+            auto lower = [&](const int2 h, int32_t v, int32_t cand, int32_t ev) {
                 if (cand >= ev) return;
-                const int32_t v = tr.x;
-                atomicMin(arr + v, cand);
                 ++c_relax;
-                int32_t d = (int32_t)((uint32_t)tr.y >> 24);  // types leaving v
-                if (d == kCountOverflow) d = __ldg(N.row_ptr + v + 1) - tr.z;
-                if (d <= 0) return;
+                const bool out_edges = N.big ? __ldg(N.erow + v + 1) > h.y : (uint32_t)h.x >> 24;
+                if (HZ && cand >= H) {
+                    if (ev != kInf) atomicMin(arr + v, cand);
+                    else if (atomicMin(arr + v, cand) == kInf && out_edges)
+                        wait_base[(int64_t)wl * qa.vmax + atomicAdd(&s_wait[wl], 1)] = v;
+                    atomicMin(&s_min[wl], cand);
+                    return;
+                }
+                atomicMin(arr + v, cand);
+                if (!out_edges) return;
                 const uint32_t bit = 1u << (v & 31);
-                if (HZ && cand >= H) {                      // beyond the horizon: wait
-                    if (!(atomicOr(dmask + (v >> 5), bit) & bit))
-                        def_base[(int64_t)dl * qa.vmax + atomicAdd(&s_def[0], 1)] = v;
-                    return;
-                }
                 if (atomicOr(pmask + (v >> 5), bit) & bit) return;   // already queued
-                if (qa.edge && d >= vw) {                   // a sub-warp expands v whole
-                    sp_wr[atomicAdd(&s_spill[cs], 1)] = v;
-                    return;
-                }
-                const int32_t base = atomicAdd(&s_items[cs], d);
-                if (base + d > icap) {
-                    for (int32_t j = base; j < icap; ++j) {
-                        if (PACK) iu_wr[j] = kNullItem;
-                        else i2_wr[j].x = kNullItem;
-                    }
-                    sp_wr[atomicAdd(&s_spill[cs], 1)] = v;
-                    return;
-                }
-                if (PACK) {
-                    const int32_t hv = (v << 16) | tr.z;
-                    iu_wr[base] = hv | kFirstItem;
-                    for (int32_t j = 1; j < d; ++j) iu_wr[base + j] = hv + j;
-                } else {
-                    i2_wr[base] = make_int2(v | kFirstItem, tr.z);
-                    for (int32_t j = 1; j < d; ++j) i2_wr[base + j] = make_int2(v, tr.z + j);
-                }
-            };
-            // Item i: its stop u and type t (clearing u's bit in last round's bitmap at
-            // u's first item); loads the type record and e[u], then the cluster entry of
-            // e[u]'s cluster.  Returns whether the type has a departure at or after e[u]
-            // (else it stops here, Section III-D).
-            auto load_item = [&](int32_t i, int32_t &e_u, int32_t &k, int4 &ca, int4 &cb,
-                                 int4 &tr) -> bool {
-                int32_t u, t;
-                if (PACK) {
-                    const int32_t raw = iu_rd[i];
-                    if (raw == kNullItem) return false;
-                    u = (raw >> 16) & 0x7fff;
-                    t = raw & 0xffff;
-                    if (raw < 0) {
-                        atomicAnd(cmask + (u >> 5), ~(1u << (u & 31)));
-                        ++c_vert;
-                    }
-                } else {
-                    const int2 it = i2_rd[i];
-                    if (it.x == kNullItem) return false;
-                    u = it.x & 0x7fffffff;
-                    t = it.y;
-                    if (it.x < 0) {
-                        atomicAnd(cmask + (u >> 5), ~(1u << (u & 31)));
-                        ++c_vert;
-                    }
-                }
-                ++c_types;
-                tr = __ldg(N.tr + t);
-                e_u = load_arr(arr, u, arr_shared);
-                k = cluster_slot(N, e_u);
-                if (k < N.y) load_entry(entry_at(N, k, t), ca, cb);
-                return e_u <= tr.w;
+                const int32_t pos = atomicAdd(&s_n[cs], 1);
+                if (pos < qcap) q_wr[pos] = h;
+                else sp_wr[pos - qcap] = v;
             };
 
-            if (!qa.edge) {
-                // One thread per (stop, type) item.
-                for (int32_t i = tid; i < n_items; i += nthr) {
-                    int32_t e_u, k;
-                    int4 ca = make_int4(0, 0, 0, 0), cb = ca, tr;
-                    if (!load_item(i, e_u, k, ca, cb, tr)) continue;
-                    const int32_t ev = load_arr(arr, tr.x, arr_shared);
-                    lower(tr, lookup(e_u, k, ca, cb, tr), ev);
-                }
-            } else {
-                // EAT_MODE_EDGE: a warp's lanes take consecutive items and every lane runs
-                // every pass (lanes past the end carry none); lanes whose types share a head
-                // stop v (the types of one edge, or of edges into one stop) reduce their
-                // candidates with a warp min, and one lane per head stop lowers e[v].
-                for (int32_t ib = tid & ~31; ib < n_items; ib += nthr) {
-                    const int32_t i = ib + (tid & 31);
-                    int32_t e_u = 0, k = 0, ev = kInf, cand = kInf;
-                    int4 ca = make_int4(0, 0, 0, 0), cb = ca, tr = ca;
-                    bool live = i < n_items && load_item(i, e_u, k, ca, cb, tr);
-                    if (live) {
-                        ev = load_arr(arr, tr.x, arr_shared);
-                        cand = lookup(e_u, k, ca, cb, tr);
-                    }
-                    const unsigned grp = __match_any_sync(0xffffffffu, live ? tr.x : -1 - (tid & 31));
-                    const int32_t m = __reduce_min_sync(grp, cand);
-                    const unsigned first = __ballot_sync(0xffffffffu, cand == m) & grp;
-                    if (live && (tid & 31) == __ffs(first) - 1) lower(tr, cand, ev);
-                }
-            }
-            // Spilled stops: `vw` lanes per stop stride over its types.
-            for (int32_t i = sub; i < n_spill; i += nsub) {
-                const int32_t u = __ldcg(sp_rd + i);
-                const int32_t beg = __ldg(N.row_ptr + u);
-                const int32_t end = __ldg(N.row_ptr + u + 1);
-                if (lane == 0) {
-                    atomicAnd(cmask + (u >> 5), ~(1u << (u & 31)));
-                    ++c_vert;
+            // A sub-warp of 2^pl lanes per stop: `vwarp` lanes while that keeps every stop of
+            // the round in one pass, else four.
+            const int pl = (n << qa.vw_log2) <= nthr ? qa.vw_log2 : min(qa.vw_log2, 2);
+            const int lane = tid & ((1 << pl) - 1);
+            const int nsub = nthr >> pl;
+            for (int32_t i = tid >> pl; i < n; i += nsub) {
+                int32_t u, row, d;
+                if (i < qcap) {
+                    const int2 e = q_rd[i];
+                    row = e.y;
+                    u = N.big ? e.x : e.x & 0xffffff;
+                    d = N.big ? kCountOverflow : (int32_t)((uint32_t)e.x >> 24);
+                } else {
+                    u = __ldcg(sp_rd + (i - qcap));
+                    row = __ldg(N.erow + u);
+                    d = kCountOverflow;
                 }
                 const int32_t e_u = load_arr(arr, u, arr_shared);
-                const int32_t k = cluster_slot(N, e_u);
-                if (k >= N.y) {                             // no departure left anywhere
-                    if (lane == 0) c_types += end - beg;
+                if (d == kCountOverflow) d = __ldg(N.erow + u + 1) - row;
+                if (lane == 0) {
+                    cmask[u >> 5] = 0u;                     // every stop of the word is in this queue
+                    ++c_vert;
+                }
+                uint32_t rel;
+                const uint32_t k = edge_slot(N.base, N.shift, e_u, rel);
+                if (k >= (uint32_t)N.y) {                   // no departure left anywhere
+                    if (COUNT)
+                        for (int32_t t = row + lane; t < row + d; t += 1 << pl) c_types += __ldg(N.etypes + t);
                     continue;
                 }
-                for (int32_t t = beg + lane; t < end; t += vw) {
-                    ++c_types;
-                    int4 ca, cb;
-                    load_entry(entry_at(N, k, t), ca, cb);
-                    const int4 tr = __ldg(N.tr + t);
-                    if (e_u > tr.w) continue;
-                    const int32_t ev = load_arr(arr, tr.x, arr_shared);
-                    lower(tr, lookup(e_u, k, ca, cb, tr), ev);
+                const int32_t start = edge_slot_start(N.base, N.shift, k);
+                const int4 *const slab = N.ee + (int64_t)k * N.n_edges;
+                for (int32_t t = row + lane; t < row + d; t += 1 << pl) {
+                    const int2 h = __ldg(N.er + t);
+                    const int4 c = __ldg(slab + t);
+                    const int32_t v = N.big ? h.x : h.x & 0xffffff;
+                    const int32_t ev = load_arr(arr, v, arr_shared);
+                    int32_t seen = 3;
+                    const int32_t cand = edge_lookup(N, c, rel, start, e_u, seen);
+                    if (COUNT) {
+                        c_types += __ldg(N.etypes + t);
+                        ++c_lookups;
+                        c_evals += cand != kInf;
+                        c_aps += seen;
+                    }
+                    lower(h, v, cand, ev);
                 }
             }
             __syncthreads();
-            n_items = min(s_items[cs], icap);
-            n_spill = s_spill[cs];
+            n = s_n[cs];
+            // No stop below H is left: H moves on, in one pass over the waiting list.  The
+            // least arrival may be that of a stop since lowered below H, so that a pass
+            // can release none; the kept ones then give the exact least arrival.
+            while (HZ && hz_on && n == 0 && s_wait[wl] > 0) {
+                const int32_t nd = s_wait[wl], least = s_min[wl];
+                const int32_t Hn = least < kInf - qa.horizon ? least + qa.horizon : kInf;
+                const int32_t *const L = wait_base + (int64_t)wl * qa.vmax;
+                int32_t *const K = wait_base + (int64_t)(wl ^ 1) * qa.vmax;
+                int32_t m = kInf;
+                for (int32_t i = tid; i < nd; i += nthr) {
+                    const int32_t v = __ldcg(L + i);
+                    const int32_t e = load_arr(arr, v, arr_shared);
+                    if (e < H) continue;
+                    if (e >= Hn) {
+                        m = min(m, e);
+                        K[atomicAdd(&s_wait[wl ^ 1], 1)] = v;
+                        continue;
+                    }
+                    const int32_t pos = atomicAdd(&s_rel[wl], 1);
+                    if (pos < qcap) {
+                        const int32_t row = __ldg(N.erow + v);
+                        const int32_t d = min(__ldg(N.erow + v + 1) - row, kCountOverflow);
+                        q_wr[pos] = make_int2(N.big ? v : (int32_t)((uint32_t)v | (uint32_t)d << 24), row);
+                    } else {
+                        sp_wr[pos - qcap] = v;
+                    }
+                }
+                if (m < kInf) atomicMin(&s_min[wl ^ 1], m);
+                __syncthreads();
+                n = s_rel[wl];
+                H = Hn;
+                if (tid == 0) {
+                    s_wait[wl] = 0;
+                    s_min[wl] = kInf;
+                    s_rel[wl ^ 1] = 0;
+                }
+                wl ^= 1;
+                if (n == 0) __syncthreads();              // the list freed above is written next
+            }
             cs = cs == 2 ? 0 : cs + 1;
             ++rounds;
-            if (hz_on && n_items + n_spill == 0) {
-                // No stop below H is left: waiting stops since lowered below H were queued
-                // by that lowering and drop out; H moves to the earliest remaining arrival
-                // + horizon and the stops below it become next round's spilled stops, the
-                // others wait on (in the other list).  (Releasing while a few stops below
-                // H are still queued moves H every round and loses the horizon.)  The
-                // waiting count is read before a barrier that no change to it precedes.
-                const int32_t nd = s_def[0];
-                if (tid == 0) {
-                    s_def[1] = 0;
-                    s_def[2] = 0;
-                    s_def[3] = kInf;
-                }
-                __syncthreads();
-                if (nd > 0) {
-                    const int32_t *const L = def_base + (int64_t)dl * qa.vmax;
-                    int32_t *const K = def_base + (int64_t)(dl ^ 1) * qa.vmax;
-                    int32_t *const sp_next = spill_base + (int64_t)((rounds & 1) ^ 1) * qa.vmax;
-                    int32_t m = kInf;
-                    for (int32_t i = tid; i < nd; i += nthr) {
-                        const int32_t e = load_arr(arr, __ldcg(L + i), arr_shared);
-                        if (e >= H) m = min(m, e);
-                    }
-                    m = __reduce_min_sync(0xffffffffu, m);
-                    if ((tid & 31) == 0 && m < kInf) atomicMin(&s_def[3], m);
-                    __syncthreads();
-                    const int32_t lo = s_def[3];
-                    const int32_t Hn = lo < kInf - qa.horizon ? lo + qa.horizon : kInf;
-                    for (int32_t i = tid; i < nd; i += nthr) {
-                        const int32_t v = __ldcg(L + i);
-                        const int32_t e = load_arr(arr, v, arr_shared);
-                        if (e < H) continue;
-                        if (e < Hn) sp_next[atomicAdd(&s_def[2], 1)] = v;
-                        else K[atomicAdd(&s_def[1], 1)] = v;
-                    }
-                    __syncthreads();
-                    n_spill = s_def[2];
-                    H = Hn;
-                    dl ^= 1;
-                    if (tid == 0) s_def[0] = s_def[1];   // no thread reads [0] or [1] before this
-                    __syncthreads();
-                }
-            }
         }
-        const int32_t F = n_items + n_spill;
 
         if (arr_shared || qa.arr_rows) {
             __syncthreads();
             copy_row(out, arr, V, arr_shared, tid, nthr);
         }
-        const int32_t q_status = !valid ? EAT_ERR_INVALID : (F > 0 ? EAT_ERR_NO_CONVERGENCE : EAT_OK);
+        const int32_t q_status = !valid ? EAT_ERR_INVALID : (n > 0 ? EAT_ERR_NO_CONVERGENCE : EAT_OK);
         if (RING) {
             __syncthreads();                              // the whole row is written
             if (tid == 0) ring_done(qa.rg, q, q_status);
@@ -1241,26 +1169,24 @@ eat_cluster_kernel(const __grid_constant__ NetTable<NETS> nets, const QueryArgs 
     cluster.sync();                                   // block 0 is done reading the others
 }
 
-template <int NETS, bool COUNT>
+template <int NETS, bool COUNT, bool HZ>
 static const void *cta_kernel_ptr(int mem) {
     switch (mem) {
-    case 0: return (const void *)eat_cta_kernel<NETS, kArrShared, true, false, false, COUNT>;
-    case 1: return (const void *)eat_cta_kernel<NETS, kArrGlobal, true, false, false, COUNT>;
-    case 3: return (const void *)eat_cta_kernel<NETS, kArrPerQuery, true, false, false, COUNT>;
-    default: return (const void *)eat_cta_kernel<NETS, kArrGlobal, false, false, false, COUNT>;
+    case 0: return (const void *)eat_cta_kernel<NETS, kArrShared, true, false, COUNT, HZ>;
+    case 1: return (const void *)eat_cta_kernel<NETS, kArrGlobal, true, false, COUNT, HZ>;
+    case 3: return (const void *)eat_cta_kernel<NETS, kArrPerQuery, true, false, COUNT, HZ>;
+    default: return (const void *)eat_cta_kernel<NETS, kArrGlobal, false, false, COUNT, HZ>;
     }
 }
 
-const void *cta_kernel(int nets, int mem, bool pack, bool count, bool hz) {
-    if (pack) {
-        if (hz)
-            return count ? (const void *)eat_cta_kernel<1, kArrShared, true, true, false, true, true>
-                         : (const void *)eat_cta_kernel<1, kArrShared, true, true, false, false, true>;
-        return count ? (const void *)eat_cta_kernel<1, kArrShared, true, true, false, true, false>
-                     : (const void *)eat_cta_kernel<1, kArrShared, true, true, false, false, false>;
-    }
-    if (count) return nets == 1 ? cta_kernel_ptr<1, true>(mem) : cta_kernel_ptr<EAT_MAX_NETS, true>(mem);
-    return nets == 1 ? cta_kernel_ptr<1, false>(mem) : cta_kernel_ptr<EAT_MAX_NETS, false>(mem);
+template <int NETS>
+static const void *cta_kernel_for(int mem, bool count, bool hz) {
+    if (count) return cta_kernel_ptr<NETS, true, true>(mem);   // honours a horizon, if there is one
+    return hz ? cta_kernel_ptr<NETS, false, true>(mem) : cta_kernel_ptr<NETS, false, false>(mem);
+}
+
+const void *cta_kernel(int nets, int mem, bool count, bool hz) {
+    return nets == 1 ? cta_kernel_for<1>(mem, count, hz) : cta_kernel_for<EAT_MAX_NETS>(mem, count, hz);
 }
 
 template <int NETS>
@@ -1296,60 +1222,35 @@ cudaError_t launch_async(const NetDev *nets, int n_nets, const QueryArgs &qa, in
     return launch_async_t<EAT_MAX_NETS>(nets, n_nets, qa, mem, grid, block, smem, st);
 }
 
-template <int NETS, bool COUNT>
-static cudaError_t launch_cta_t(const NetDev *nets, int n_nets, const QueryArgs &qa, int mem,
-                                int grid, int block, size_t smem, cudaStream_t st) {
-    NetTable<NETS> tab;
+template <int NETS>
+static cudaError_t launch_cta_t(const void *kernel, const EdgeDev *nets, int n_nets,
+                                const QueryArgs &qa, int grid, int block, size_t smem,
+                                cudaStream_t st) {
+    EdgeTable<NETS> tab;
     for (int i = 0; i < n_nets && i < NETS; ++i) tab.net[i] = nets[i];
-    for (int i = n_nets; i < NETS; ++i) tab.net[i] = NetDev{};
-    switch (mem) {
-    case 0: eat_cta_kernel<NETS, kArrShared, true, false, false, COUNT><<<grid, block, smem, st>>>(tab, qa); break;
-    case 1: eat_cta_kernel<NETS, kArrGlobal, true, false, false, COUNT><<<grid, block, smem, st>>>(tab, qa); break;
-    case 3: eat_cta_kernel<NETS, kArrPerQuery, true, false, false, COUNT><<<grid, block, smem, st>>>(tab, qa); break;
-    default: eat_cta_kernel<NETS, kArrGlobal, false, false, false, COUNT><<<grid, block, smem, st>>>(tab, qa); break;
-    }
-    return cudaGetLastError();
+    for (int i = n_nets; i < NETS; ++i) tab.net[i] = EdgeDev{};
+    void *args[2] = {&tab, const_cast<QueryArgs *>(&qa)};
+    return cudaLaunchKernel(kernel, dim3((unsigned)grid), dim3((unsigned)block), args, smem, st);
 }
 
-cudaError_t launch_cta(const NetDev *nets, int n_nets, const QueryArgs &qa, int mem, int grid,
-                       int block, size_t smem, cudaStream_t st, bool pack) {
-    const bool count = qa.counters != nullptr;
-    if (pack) {
-        NetTable<1> tab;
-        tab.net[0] = nets[0];
-        const bool hz = qa.horizon > 0;
-        if (count && hz) eat_cta_kernel<1, kArrShared, true, true, false, true, true><<<grid, block, smem, st>>>(tab, qa);
-        else if (count) eat_cta_kernel<1, kArrShared, true, true, false, true, false><<<grid, block, smem, st>>>(tab, qa);
-        else if (hz) eat_cta_kernel<1, kArrShared, true, true, false, false, true><<<grid, block, smem, st>>>(tab, qa);
-        else eat_cta_kernel<1, kArrShared, true, true, false, false, false><<<grid, block, smem, st>>>(tab, qa);
-        return cudaGetLastError();
-    }
-    if (n_nets == 1)
-        return count ? launch_cta_t<1, true>(nets, n_nets, qa, mem, grid, block, smem, st)
-                     : launch_cta_t<1, false>(nets, n_nets, qa, mem, grid, block, smem, st);
-    return count ? launch_cta_t<EAT_MAX_NETS, true>(nets, n_nets, qa, mem, grid, block, smem, st)
-                 : launch_cta_t<EAT_MAX_NETS, false>(nets, n_nets, qa, mem, grid, block, smem, st);
+cudaError_t launch_cta(const EdgeDev *nets, int n_nets, const QueryArgs &qa, int mem, int grid,
+                       int block, size_t smem, cudaStream_t st) {
+    const void *k = cta_kernel(n_nets == 1 ? 1 : EAT_MAX_NETS, mem, qa.counters != nullptr, qa.horizon > 0);
+    return n_nets == 1 ? launch_cta_t<1>(k, nets, n_nets, qa, grid, block, smem, st)
+                       : launch_cta_t<EAT_MAX_NETS>(k, nets, n_nets, qa, grid, block, smem, st);
 }
 
 const void *ring_kernel(int mem) {
     switch (mem) {
-    case 0: return (const void *)eat_cta_kernel<EAT_MAX_NETS, kArrShared, true, false, true>;
-    case 3: return (const void *)eat_cta_kernel<EAT_MAX_NETS, kArrPerQuery, true, false, true>;
-    default: return (const void *)eat_cta_kernel<EAT_MAX_NETS, kArrGlobal, true, false, true>;
+    case 0: return (const void *)eat_cta_kernel<EAT_MAX_NETS, kArrShared, true, true, false, false>;
+    case 3: return (const void *)eat_cta_kernel<EAT_MAX_NETS, kArrPerQuery, true, true, false, false>;
+    default: return (const void *)eat_cta_kernel<EAT_MAX_NETS, kArrGlobal, true, true, false, false>;
     }
 }
 
-cudaError_t launch_ring(const NetDev *nets, int n_nets, const QueryArgs &qa, int mem, int grid,
+cudaError_t launch_ring(const EdgeDev *nets, int n_nets, const QueryArgs &qa, int mem, int grid,
                         int block, size_t smem, cudaStream_t st) {
-    NetTable<EAT_MAX_NETS> tab;
-    for (int i = 0; i < n_nets && i < EAT_MAX_NETS; ++i) tab.net[i] = nets[i];
-    for (int i = n_nets; i < EAT_MAX_NETS; ++i) tab.net[i] = NetDev{};
-    switch (mem) {
-    case 0: eat_cta_kernel<EAT_MAX_NETS, kArrShared, true, false, true><<<grid, block, smem, st>>>(tab, qa); break;
-    case 3: eat_cta_kernel<EAT_MAX_NETS, kArrPerQuery, true, false, true><<<grid, block, smem, st>>>(tab, qa); break;
-    default: eat_cta_kernel<EAT_MAX_NETS, kArrGlobal, true, false, true><<<grid, block, smem, st>>>(tab, qa); break;
-    }
-    return cudaGetLastError();
+    return launch_cta_t<EAT_MAX_NETS>(ring_kernel(mem), nets, n_nets, qa, grid, block, smem, st);
 }
 
 const void *pair_kernel(bool count) {

@@ -48,7 +48,8 @@ struct QueryArgs {
     int32_t max_rounds;
     int32_t vw_log2;           // lanes per active stop = 1 << vw_log2
     int32_t vmax;              // largest n_stops in the launch
-    int32_t qcap;              // shared-memory (stop, type) items per buffer
+    int32_t qcap;              // queue entries per buffer in shared memory (stops; paired
+                               // and cluster mode: (stop, type) items)
     int32_t mask_words;        // words per bitmap (padded)
     int32_t smem_mask_off;     // int offset of the bitmaps in dynamic shared memory
     int32_t smem_q_off;        // int offset of the item buffers in dynamic shared memory
@@ -59,30 +60,25 @@ struct QueryArgs {
     const int32_t *order;      // [n]: the i-th query handed out is order[i], or nullptr (i)
     int32_t idle_cap;          // round-free mode: empty 32-word bitmap scans in a row per warp
     RingArgs rg;               // ring mode only
-    int32_t edge;              // EAT_MODE_EDGE: warp min per head stop, stops with >= vwarp
-                               // types expanded whole by a sub-warp
     int32_t horizon;           // seconds, 0 = none: stops lowered to an arrival at or after
                                // the horizon wait (per-query kernel); with one,
-                               // spill_stride >= 4 * vmax + mask_words
+                               // spill_stride >= 4 * vmax
 };
 
 // mem: 0 = arrivals and bitmaps in shared memory, 1 = arrivals global / bitmaps
 // shared, 2 = both global, 3 = bitmaps shared and arrivals shared per query when
 // the query's network fits.  nets: 1 or EAT_MAX_NETS (kernel table size).
-// pack: one int32 per item (one network of at most 32,767 stops and 65,535 types,
-// arrivals and bitmaps in shared memory).
 // count: the instantiation that fills qa.counters (launch_cta picks it when counters are
-// given); hz: with pack, the instantiation that honours qa.horizon (launch_cta picks it
-// when qa.horizon > 0; the others always honour it).
-const void *cta_kernel(int nets, int mem, bool pack = false, bool count = false, bool hz = false);
-cudaError_t launch_cta(const NetDev *nets, int n_nets, const QueryArgs &qa, int mem, int grid,
-                       int block, size_t smem, cudaStream_t st, bool pack = false);
+// given); hz: the one that honours qa.horizon (launch_cta picks it when qa.horizon > 0).
+const void *cta_kernel(int nets, int mem, bool count = false, bool hz = false);
+cudaError_t launch_cta(const EdgeDev *nets, int n_nets, const QueryArgs &qa, int mem, int grid,
+                       int block, size_t smem, cudaStream_t st);
 // Ring mode of the per-query kernel (serving): persistent blocks take requests from
 // qa.rg until the host's stop flag is set and no request is left, or until they find
 // none for rg.idle_iters polls; mem 0, 1 or 3; rows go to arr_out + row * row_stride,
 // arrivals not in shared memory live in the block's arr_rows row meanwhile.
 const void *ring_kernel(int mem);
-cudaError_t launch_ring(const NetDev *nets, int n_nets, const QueryArgs &qa, int mem, int grid,
+cudaError_t launch_ring(const EdgeDev *nets, int n_nets, const QueryArgs &qa, int mem, int grid,
                         int block, size_t smem, cudaStream_t st);
 // Asynchronous (round-free) kernel; mem 0, 1 or 3 as above (bitmap always shared).
 const void *async_kernel(int nets, int mem);

@@ -1,0 +1,71 @@
+"""The round kernel on networks at the edges of its layout: more stops than a packed record
+holds, stops of more than 255 edges, frontiers larger than the shared-memory queue, slots
+with departures beyond the inline ones.  Rows equal the oracle's exactly."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+
+torch = pytest.importorskip("torch")
+pytestmark = [pytest.mark.gpu, pytest.mark.skipif(not torch.cuda.is_available(), reason="no CUDA device")]
+
+
+def _timetable(n, u, v, dep, dur):
+    c = [np.asarray(a, dtype=np.int32) for a in (u, v, dep, dur)]
+    z = np.zeros(c[0].shape[0], np.int32)
+    return synth.Timetable("edges", n, *c, z, z)
+
+
+def _many_stops():
+    """2^24 + 9 stops, connections between a few of them at both ends of the range."""
+    rng = np.random.default_rng(1)
+    ids = np.concatenate([np.arange(12), 2**24 + np.arange(-4, 9)])
+    u, v = rng.choice(ids, 900), rng.choice(ids, 900)
+    return _timetable(2**24 + 9, u, v, rng.integers(0, 5000, 900), rng.integers(1, 300, 900)), ids
+
+
+def _star(n_spokes, n_stops):
+    """A hub with an edge to every spoke, each spoke with two edges onward, some back."""
+    rng = np.random.default_rng(n_spokes)
+    spokes = 1 + np.arange(n_spokes)
+    u = np.concatenate([np.zeros(n_spokes, int), spokes, spokes])
+    v = np.concatenate([spokes, rng.integers(0, n_stops, n_spokes), rng.integers(0, n_stops, n_spokes)])
+    m = u.shape[0]
+    k = 3
+    return _timetable(n_stops, np.tile(u, k), np.tile(v, k), rng.integers(0, 4000, k * m),
+                      rng.integers(1, 500, k * m)), np.concatenate([[0], spokes[:6]])
+
+
+def _dense():
+    """Every second a departure of some duration on a few edges."""
+    rng = np.random.default_rng(5)
+    m = 20000
+    u = rng.integers(0, 6, m)
+    return _timetable(6, u, (u + rng.integers(1, 6, m)) % 6, rng.integers(0, 30000, m),
+                      rng.integers(1, 8, m) ** 4), np.arange(6)
+
+
+CASES = {"many_stops": _many_stops, "star_300": lambda: _star(300, 800),
+         "star_queue_spills": lambda: _star(20000, 50000), "star_global": lambda: _star(30000, 400000),
+         "dense": _dense}
+
+
+@pytest.mark.parametrize("which", CASES)
+def test_rows(which):
+    from paper_1912_00966_gb300 import eat
+    tt, ids = CASES[which]()
+    sc = oracle.SortedConnections(tt)
+    net = eat.eat_build(tt.n_stops, tt.u, tt.v, tt.dep, tt.dur, device=0, cluster_width=300)
+    rng = np.random.default_rng(2)
+    src = np.concatenate([[ids[0], ids[0]], rng.choice(ids, 2)]).astype(np.int32)
+    ts = np.array([0, 1000, 2000, 29990], np.int32)
+    want = np.stack([oracle.csa(sc, int(s), int(t)) for s, t in zip(src, ts)])
+    out = torch.empty((4, tt.n_stops), dtype=torch.int32, device="cuda")
+    for opts in ({}, {"horizon": 200}, {"block": 64, "horizon": 1500}, {"block": 256, "vwarp": 1}):
+        out.fill_(-7)
+        eat.eat_query_batch(net, torch.as_tensor(src).cuda(), torch.as_tensor(ts).cuda(), out, **opts)
+        assert np.array_equal(out.cpu().numpy(), want), opts
+    got = eat.eat_query(net, int(src[3]), int(ts[3]))
+    assert np.array_equal(got, want[3])
+    net.close()
