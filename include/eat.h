@@ -171,10 +171,13 @@ typedef struct {
                                 2 * n_stops + 2 with a horizon (each horizon step adds at
                                 most one round to the n_stops + 1) */
     int32_t block;           /* threads per CTA: 0 = automatic (the tuned shape, else 1024
-                                when the batch has at most one query per SM, runs in the
-                                paired mode or is on one network of 8,192 stops or more,
-                                else 512);
-                                else 64..1024, multiple of 32 */
+                                when the batch has at most one query per SM or runs in the
+                                paired mode; on one network up to 1.5 queries per SM 1024
+                                from 8,192 stops on, else 512, and for fuller batches 128
+                                to 1024 by the network's size; 384 over several networks);
+                                else 64..1024, multiple of 32.  In an automatic block on a
+                                small network the threads that its rounds cannot fill leave
+                                at once */
     int32_t vwarp;           /* lanes per active stop (1, 2, 4, 8, 16 or 32), at most four of
                                 them in rounds with more stops than the block has
                                 sub-warps; 0 = automatic (8) */
@@ -202,7 +205,12 @@ typedef struct {
                                 later round improves them (Algorithms 4-5 expand every
                                 improved stop in the next round).
                                 0 = automatic (the value eat_autotune chose for this
-                                batch size, else none); < 0 = none; > 0 with
+                                batch size, else, for a call without a round cap on one
+                                network whose stops have two or more edges on average,
+                                two hours when the arrivals are in global memory and four
+                                hours in shared memory for 2 queries up to half the SM
+                                count and for more than 1.5 queries per SM; none otherwise
+                                and in eat_query_batch_noalloc); < 0 = none; > 0 with
                                 EAT_MODE_PAIR, EAT_MODE_ASYNC or EAT_MODE_CLUSTER is
                                 EAT_ERR_INVALID */
     int32_t *status;         /* optional [n] per-query eat_status, device memory */
@@ -220,8 +228,10 @@ enum eat_placement {
 enum eat_order {
     EAT_ORDER_AUTO = 0,      /* on one network: EAT_ORDER_BY_TIME when the batch has more
                                 queries than the launch runs at once (some wait for a
-                                free block) or runs in EAT_MODE_PAIR; otherwise, and for
-                                batches over several networks, EAT_ORDER_AS_GIVEN */
+                                free block), has more queries than the GPU has SMs on a
+                                network of 8,192 stops or more, or runs in EAT_MODE_PAIR;
+                                otherwise, and for batches over several networks,
+                                EAT_ORDER_AS_GIVEN */
     EAT_ORDER_BY_TIME = 1,   /* queries start in order of departure time t_s (15-minute
                                 buckets, earliest first; a one-block device counting sort
                                 before the launch, n int32 of workspace): the longest
@@ -449,14 +459,13 @@ int eat_next_departure(const eat_net *net, const int32_t *types, const int32_t *
  * eat_autotune -- choose the launch shape for this network by measurement (no
  * counterpart in the paper, which fixes one thread per type or per edge and
  * sweeps the virtual-warp size by hand, Section IV-B).  Candidates, in this
- * order: block sizes 512, 1024 and 256 threads, each with the round-based mode
- * and vwarp 8, 4, 16, 2, 32 lanes per spilled stop, then with the asynchronous
- * mode, then with EAT_MODE_EDGE and vwarp 8 and 32, as far as they fit the device
- * (1024 threads first on networks of 8,192 stops or more and for batches of at most
- * one query per SM, where it is the default); when n exceeds the SM count, then the
- * paired mode with vwarp 8, 4 and 16; then the round-based mode with the first two
- * block sizes, vwarp 8 and horizons of 1, 2, 4 and 12 hours (the other candidates run
- * with none).  They are run on the sample batch
+ * order: the automatic shape's block size first if it is one of 1024, 512 and 256
+ * threads, then the others of these, each with the round-based mode and vwarp 8, 4
+ * and 16 lanes per stop and with the asynchronous mode, without a horizon; when n
+ * exceeds the SM count, the paired mode with vwarp 8, 4 and 16; and the round-based
+ * mode with each block size, vwarp 8 and horizons of 1, 2, 4 and 12 hours, which come
+ * first on networks where the automatic shape has a horizon; as far as they fit the
+ * device.  They are run on the sample batch
  * sources/times (n queries, device memory) in nine rounds over all candidates:
  * the first warms up, the other eight are timed with CUDA events on `stream`,
  * each after a write of twice the L2 size so that every timing starts with the
@@ -479,8 +488,8 @@ int eat_autotune(eat_net *net, const int32_t *sources, const int32_t *times, int
  * networks of uneven size (eat_query_batch_multi) by measurement; no counterpart in the
  * paper, as for eat_autotune.  Candidates, in this order: start order as given, then by
  * t_s (EAT_ORDER_AS_GIVEN, EAT_ORDER_BY_TIME); for each, block sizes 512, 1024 and 256
- * threads, each with the round-based mode and vwarp 8, 4, 16, 2, 32, then the
- * asynchronous mode, then EAT_MODE_EDGE with vwarp 8; then the round-based mode with 512
+ * threads, each with the round-based mode and vwarp 8, 4, 16, then the
+ * asynchronous mode; then the round-based mode with 512
  * threads, vwarp 8, start by t_s and horizons of 2 and 12 hours (the others run with
  * none); shapes without a plan for these networks are skipped.  They run on
  * the sample batch (net_idx, sources, times: [n] int32 device memory; rows packed in
@@ -622,7 +631,7 @@ void eat_server_destroy(eat_server *sv);
  *     (rounded up) for its frontier queue, plus n_stops / 4 bytes when the frontier
  *     bitmaps live in global memory (networks beyond about 900,000 stops), or
  *     16 * n_stops bytes in the paired mode (two queries per block); with a
- *     horizon, 16 * n_stops bytes (the lists of waiting stops); the
+ *     horizon, 16 * n_stops + n_stops / 8 bytes; the
  *     round-free mode needs none.  So the network may have at most 2,000,000 stops
  *     (about 1,000,000 with a horizon), and on large networks fewer blocks run at
  *     once while the other queries wait in the same launch.  Larger networks are

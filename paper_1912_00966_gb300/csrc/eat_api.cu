@@ -109,8 +109,9 @@ static int device_info(int dev, DeviceInfo &out) {
         DeviceGuard guard(dev);
         for (int nets : {1, EAT_MAX_NETS})
             for (int mem = 0; mem < 4; ++mem)
-                for (const void *k : {cta_kernel(nets, mem), cta_kernel(nets, mem, true),
-                                      cta_kernel(nets, mem, false, true), async_kernel(nets, mem),
+                for (const void *k : {cta_kernel(nets, mem, 1024), cta_kernel(nets, mem, 1024, true),
+                                      cta_kernel(nets, mem, 1024, false, true), cta_kernel(nets, mem, 512),
+                                      cta_kernel(nets, mem, 512, false, true), async_kernel(nets, mem),
                                       cluster_kernel(), pair_kernel(false), pair_kernel(true),
                                       ring_kernel(mem)}) {
                     e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -135,6 +136,7 @@ struct Plan {
     int32_t mask_words = 0;       // words per bitmap
     int32_t smem_mask_off = 0;    // int offsets into dynamic shared memory
     int32_t smem_q_off = 0;
+    int32_t smem_wait_off = 0;    // bitmap of waiting stops (horizon), 0 = global memory
     int32_t smem_arr_cap = 0;     // mem 3: arrivals shared for networks up to this size
     int64_t spill_stride = 0;     // ints per persistent block
     int64_t mask_stride = 0;      // words per persistent block (global bitmaps only)
@@ -148,11 +150,19 @@ struct Plan {
     bool order = false;           // queries start by t_s (EAT_ORDER_BY_TIME): order array at off_order
     size_t off_order = 0;
     int32_t horizon = 0;          // seconds (eat_query_opts.horizon resolved), 0 = none
+    int active = 0;               // threads of a block that work, 0 = all
 };
 
 static constexpr size_t kWsHeader = 256;   // work counter + internal status / counters
 static constexpr int32_t kDefaultIdleCap = 1 << 24;   // round-free mode's wait limit (full scans)
 static constexpr size_t kQueueEntryBytes = 16;  // 8-byte queue entry x 2 buffers
+// Shared memory that an SM's blocks take together where that can be had: the 196 KB step of
+// the SM's division leaves 60 KB of the 256 to L1, in which every load in flight holds a
+// line.  A queue that took all there was left L1 28 KB: large network, 1,024 queries, three
+// 512-thread blocks per SM, horizon one hour 3,556 us against 2,595; 96 queries, one
+// 1,024-thread block 1,452 against 1,103; 60,000 stops, 300 queries 1,177 against 1,007.
+static constexpr size_t kSmemBesideL1 = 196 << 10;
+static constexpr size_t kQueueMost = 1024;      // stops queued in shared memory per buffer
 
 // Default round cap: n_stops + 1 rounds always reach the fixpoint (every productive round
 // fixes one more stop); with a horizon, each move of the horizon can add one round in
@@ -271,7 +281,9 @@ static int make_cluster_plan(int dev, const DeviceInfo &d, int32_t vmax, int32_t
     return EAT_OK;
 }
 
-static constexpr int32_t kWideMinStops = 8192;   // 1,024-thread blocks for any batch from this size
+static constexpr int32_t kWideMinStops = 8192;   // start by t_s, 1,024-thread blocks for small batches
+// Stops whose arrivals, bitmaps and queue fit an SM's shared memory once and twice.
+static constexpr int32_t kOneSharedStops = 52000, kTwoSharedStops = 24000;
 
 // Plan of the paired kernel: two arrival rows, four bitmaps (two per query) and the
 // shared item buffers (one int32 per item) in one block's shared memory.  Returns
@@ -315,8 +327,15 @@ static int make_pair_plan(int dev, const DeviceInfo &d, int32_t vmax, int32_t n,
     return EAT_OK;
 }
 
+// Batch-size class of n queries (log2).
+static int log2_class(int32_t n) {
+    int c = 0;
+    while (c < 31 && ((int64_t)1 << (c + 1)) <= n) ++c;
+    return c;
+}
+
 static int make_plan_core(int dev, int32_t vmax, int32_t n, int n_nets, const eat_query_opts *o,
-                          Plan &p, int32_t vmin, const eat_net *tuned, bool own_workspace) {
+                          Plan &p, int32_t vmin, const eat_net *tuned, bool own_workspace, bool use_tuned) {
     if (vmin < 0) vmin = vmax;
     DeviceInfo d;
     int rc = device_info(dev, d);
@@ -324,26 +343,35 @@ static int make_plan_core(int dev, int32_t vmax, int32_t n, int n_nets, const ea
     p.nets = n_nets == 1 ? 1 : EAT_MAX_NETS;
     p.vmax = vmax;
     int tb = 0, tv = 0, tm = 0, th = 0;
-    if (tuned && n > 0) {
-        int cls = 0;
-        while (cls < 31 && (1 << (cls + 1)) <= n) ++cls;
-        const uint64_t sh = tuned->tuned[cls].load(std::memory_order_relaxed);
+    if (tuned && use_tuned && n > 0) {
+        const uint64_t sh = tuned->tuned[log2_class(n)].load(std::memory_order_relaxed);
         tb = (int)(sh & 0xffffu);
         tv = (int)((sh >> 16) & 0xffu);
         tm = (int)((sh >> 24) & 0xffu);
         th = (int)(uint32_t)(sh >> 32);
     }
-    // Default shape: a 1,024-thread block per query when the batch has at most one query
-    // per SM, or on one network of 8,192 stops or more (there the batch starts in order
-    // of t_s, so the longest queries run first and the later ones fill the blocks that
-    // free up: city 0.70 ms per 256-query step against 0.88 ms for two 512-thread
-    // blocks per SM); fuller batches on small networks, and batches over several
-    // networks (mostly small ones: the ragged batch of 64 networks took 4.59 ms with
-    // 1,024 threads against 2.71 ms with 512), run two 512-thread blocks per SM.
-    // A tuned shape or opts->block overrides.
-    p.block = (o && o->block) ? o->block
-              : (tb ? tb
-                    : (n >= 1 && (n <= d.sms || (n_nets == 1 && vmax >= kWideMinStops)) ? 1024 : 512));
+    // Default shape (a tuned shape or opts->block overrides).  Up to 1.5 queries per SM: one
+    // 1,024-thread block per SM (512 threads on networks below 8,192 stops once some queries
+    // wait).  Fuller batches on one network: as many threads as its rounds fill, several
+    // blocks per SM (us for 300 / 1,024 queries: 3,000-stop grid 96 / 114 with 128 threads
+    // against 105 / 160 with 512; 10,000-stop city 215 / 322 with 256 against 225 / 402;
+    // 20,000-stop city, 256 queries, 287 with 512 against 319 with 1,024), with arrivals in
+    // global memory 1,024 threads up to 2.5 queries per SM (100,000 stops, 300 / 600
+    // queries: 1,410 / 2,596 against 1,790 / 2,341 with 512).  Batches over several networks:
+    // 384 threads (4,096 queries on 64 ragged grids 824 us; 256: 901, 512: 911).
+    const bool wide = vmax >= kWideMinStops;
+    const bool full = 2 * (int64_t)n > 3 * (int64_t)d.sms;
+    const bool one_shared = vmax <= kOneSharedStops, two_shared = vmax <= kTwoSharedStops;
+    const bool rounds = !o || o->mode == EAT_MODE_AUTO || o->mode == EAT_MODE_CTA || o->mode == EAT_MODE_EDGE;
+    int block = 512;
+    if ((n >= 1 && n <= d.sms) || (!rounds && n_nets == 1 && wide)) block = 1024;
+    else if (!rounds) block = 512;
+    else if (n_nets > 1) block = 384;
+    else if (!full) block = wide ? 1024 : 512;
+    else if (vmax < 4096) block = 128;
+    else if (vmax < 12288) block = 256;
+    else if (!two_shared && (one_shared ? n <= 4 * d.sms : 2 * (int64_t)n <= 5 * (int64_t)d.sms)) block = 1024;
+    p.block = (o && o->block) ? o->block : (tb ? tb : block);
     if (p.block < 64 || p.block > 1024 || p.block % 32)
         return fail(EAT_ERR_INVALID, "block must be a multiple of 32 in 64..1024");
     int vw = (o && o->vwarp) ? o->vwarp : (tv ? tv : 8);
@@ -408,34 +436,63 @@ static int make_plan_core(int dev, int32_t vmax, int32_t n, int n_nets, const ea
         return fail(EAT_ERR_INVALID, "arrivals do not fit in shared memory");
     if (place == EAT_PLACE_GLOBAL_ARR && !fits(1))
         return fail(EAT_ERR_INVALID, "bitmaps do not fit in shared memory");
-    // A batch over networks of uneven size whose largest arrival row would cost
-    // more than half an SM's shared memory keeps arrivals in shared memory only
-    // for the networks that fit half an SM (two blocks per SM stay resident).
-    const size_t half = d.smem_per_sm / 2 - d.reserve;
+    // A batch over networks of uneven size whose largest arrival row does not fit the share
+    // of an SM's shared memory that as many blocks leave each other as it can have queries
+    // there (up to four) keeps arrivals in shared memory only for the networks that do (64
+    // grids of 1,000 to 50,000 stops, 4,096 queries: a quarter of an SM 824 us, a third
+    // 1,005, half 1,265, a sixth 834).  The ring kernel, which serves single requests as they
+    // come, is sized for two blocks.
+    const bool ring = n_nets > 1 && !own_workspace;
+    const int parts = ring ? 2 : (int)std::min<int64_t>(4, (std::max(n, 1) + d.sms - 1) / d.sms);
+    const size_t share = (parts <= 2 ? d.smem_per_sm : kSmemBesideL1) / (size_t)parts - d.reserve;
     p.smem_arr_cap = 0;
-    if (place == EAT_PLACE_AUTO && vmin < vmax && base(0) + kQueueEntryBytes * qmin > half &&
-        fits(1)) {
-        const size_t room = half - base(1) - kQueueEntryBytes * 1024;
-        const int32_t cap = (int32_t)std::min<size_t>(room / 4 & ~(size_t)3, (size_t)vmax);
+    if (place == EAT_PLACE_AUTO && vmin < vmax && base(0) + kQueueEntryBytes * qmin > share && fits(1)) {
+        const int64_t room = (int64_t)share - (int64_t)base(1) - (int64_t)(kQueueEntryBytes * 512);
+        const int32_t cap = (int32_t)std::min<int64_t>(room / 4 & ~(int64_t)3, (int64_t)vmax);
         if (cap >= vmin) {
             p.mem = 3;
             p.smem_arr_cap = cap;
         }
     }
+    // One network whose arrivals fit an SM only once: with more than four queries per SM three
+    // blocks with their rows in global memory do more (30,000 stops, 1,024 queries 471 us
+    // against 603; 50,000: 570 against 701).
+    const bool spread = n_nets == 1 && !two_shared && n > 4 * d.sms && p.block <= 512 && fits(1) && rounds;
     if (p.mem == 3) {
-    } else if (place == EAT_PLACE_SHARED || (place == EAT_PLACE_AUTO && fits(0))) p.mem = 0;
+    } else if (place == EAT_PLACE_SHARED || (place == EAT_PLACE_AUTO && fits(0) && !spread)) p.mem = 0;
     else if (place == EAT_PLACE_GLOBAL_ARR || (place == EAT_PLACE_AUTO && fits(1))) p.mem = 1;
     else p.mem = 2;
 
-    p.horizon = oh > 0 ? oh : (oh == 0 ? th : 0);
+    // The tuned horizon, else on one network where stops have two or more edges on average
+    // (where they have fewer, a stop is seldom improved again and a horizon only adds rounds:
+    // 3,000-stop grid, 300 queries 105 -> 119 us with four hours): two hours with arrivals in
+    // global memory (200,000 stops, 96 queries 2,960 -> 1,600; one hour and four hours within
+    // 7 %), four hours in shared memory for full batches (20,000-stop city, 256 queries
+    // 390 -> 287) and for a few queries (37: 268 -> 224; a single one gains nothing).
+    int32_t automatic = 0;
+    if (own_workspace && n_nets == 1 && tuned && tuned->branching && !(o && o->max_rounds > 0))
+        automatic = p.mem != 0 ? 7200 : full || (n > 1 && 2 * (int64_t)n <= d.sms) ? 14400 : 0;
+    p.horizon = oh > 0 ? oh : oh < 0 ? 0 : tb ? th : automatic;
+    // Threads at work in a default-shaped block (the others leave): no more than the rounds
+    // of a small network fill (1,024 stops, 256 queries: 128 of 512 threads 62 us, all 69;
+    // 16,000 stops, 100 queries: 512 157, 1,024 187).
+    p.active = p.block;
+    if (!(o && o->block) && !tb && p.mem == 0)
+        p.active = std::min(p.block, vmax < 2048 ? 128 : vmax < 6144 ? 256 : vmax <= 32768 ? 512 : 1024);
     const size_t qbytes = kQueueEntryBytes;
-    // Largest queue capacity that keeps the most blocks per SM the threads and the
-    // registers allow (shared memory is the only other limit, and the one sized here).
-    const size_t b0 = p.mem == 3 ? base(1) + (size_t)p.smem_arr_cap * 4 : base(p.mem);
+    // As many blocks per SM as the threads and the registers allow (shared memory is the only
+    // other limit, and the one sized here), and the largest queue, up to kQueueMost stops,
+    // that keeps them and leaves L1 its share.
+    const size_t bm = p.mem == 3 ? base(1) + (size_t)p.smem_arr_cap * 4 : base(p.mem);
+    // The bitmap of waiting stops beside shared arrivals, where that leaves room for a queue.
+    const size_t wait_bytes = (size_t)p.mask_words * 4;
+    const bool wait_shared = p.mem == 0 && p.horizon > 0 && bm + wait_bytes + qbytes * qmin <= limit;
+    p.smem_wait_off = wait_shared ? (int32_t)(bm / 4) : 0;
+    const size_t b0 = bm + (wait_shared ? wait_bytes : 0);
     int reg_blocks = 0;
     {
         DeviceGuard guard(dev);
-        const void *k = cta_kernel(p.nets, p.mem, false, p.horizon > 0);
+        const void *k = cta_kernel(p.nets, p.mem, p.block, false, p.horizon > 0);
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&reg_blocks, k, p.block, 0) != cudaSuccess) {
             cudaGetLastError();
             reg_blocks = 0;
@@ -446,14 +503,15 @@ static int make_plan_core(int dev, int32_t vmax, int32_t n, int n_nets, const ea
     for (int b = max_blocks; b >= 1; --b) {
         const size_t budget = std::min(limit, d.smem_per_sm / (size_t)b - d.reserve);
         if (d.smem_per_sm / (size_t)b < d.reserve || b0 + qbytes * qmin > budget) continue;
-        size_t cap = (budget - b0) / qbytes;
-        cap = std::min(cap, (size_t)std::max(vmax, 1));
+        const size_t beside = kSmemBesideL1 / (size_t)b - 1024;   // 1 KB of each block is the driver's
+        const size_t room = b0 + qbytes * qmin <= beside ? std::min(budget, beside) : budget;
+        size_t cap = std::min({(room - b0) / qbytes, (size_t)std::max(vmax, 1), kQueueMost});
         if (cap >= 64) cap &= ~(size_t)31;
         p.qcap = (int32_t)std::max(cap, qmin);
         break;
     }
     p.smem_mask_off = p.mem == 0 ? (int32_t)(arr_bytes / 4) : p.mem == 3 ? p.smem_arr_cap : 0;
-    p.smem_q_off = p.smem_mask_off + (p.mem != 2 ? 2 * p.mask_words : 0);
+    p.smem_q_off = (int32_t)(b0 / 4);
     p.smem = b0 + qbytes * (size_t)p.qcap;
 
     int per_sm = 0;
@@ -461,13 +519,13 @@ static int make_plan_core(int dev, int32_t vmax, int32_t n, int n_nets, const ea
     {
         DeviceGuard guard(dev);
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-            &per_sm, cta_kernel(p.nets, p.mem, false, p.horizon > 0), p.block, p.smem);
+            &per_sm, cta_kernel(p.nets, p.mem, p.block, false, p.horizon > 0), p.block, p.smem);
     }
     if (e != cudaSuccess) return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
     if (per_sm < 1) return fail(EAT_ERR_INVALID, "kernel does not fit on an SM with this block size");
     p.grid = (int)std::min<int64_t>((int64_t)std::max(n, 1), (int64_t)per_sm * d.sms);
-    // With a horizon a block also keeps two lists of waiting stops.
-    p.spill_stride = p.horizon > 0 ? (int64_t)align_up((size_t)vmax * 4, 64)
+    // With a horizon a block also keeps the bitmap of waiting stops.
+    p.spill_stride = p.horizon > 0 ? (int64_t)align_up((size_t)vmax * 2 + (size_t)p.mask_words, 64)
                                    : (int64_t)align_up((size_t)vmax * 2, 64);
     p.mask_stride = p.mem == 2 ? (int64_t)align_up(2 * (size_t)p.mask_words, 64) : 0;
     p.off_spill = kWsHeader;
@@ -480,17 +538,21 @@ static int make_plan_core(int dev, int32_t vmax, int32_t n, int n_nets, const ea
 // also gets its start order (EAT_ORDER_BY_TIME) at the end of the workspace.
 static int make_plan(int dev, int32_t vmax, int32_t n, int n_nets, const eat_query_opts *o,
                      Plan &p, int32_t vmin = -1, const eat_net *tuned = nullptr,
-                     bool own_workspace = true) {
+                     bool own_workspace = true, bool use_tuned = true) {
     const int order = o ? o->order : EAT_ORDER_AUTO;
     if (order < EAT_ORDER_AUTO || order > EAT_ORDER_AS_GIVEN)
         return fail(EAT_ERR_INVALID, "order must be one of EAT_ORDER_*");
-    int rc = make_plan_core(dev, vmax, n, n_nets, o, p, vmin < 0 ? vmax : vmin, tuned, own_workspace);
+    int rc = make_plan_core(dev, vmax, n, n_nets, o, p, vmin < 0 ? vmax : vmin, tuned, own_workspace, use_tuned);
     if (rc) return rc;
-    // Automatic, on one network: sorted when some queries must wait for a free block
-    // (they then start longest first) and in the paired mode (an early query shares its
-    // block with a late one); a batch that starts all at once gains nothing for the
-    // sort's launch.  Batches over several networks keep index order (measured only so).
-    const bool waits = p.cluster == 0 && !p.pair && n > p.grid;
+    // Automatic, on one network: sorted when some queries must wait for a free block or share
+    // an SM of a network of 8,192 stops or more (they then start longest first) and in the
+    // paired mode (an early query shares its block with a late one); a batch that starts
+    // all at once gains nothing for the sort's launch.  Batches over several networks keep
+    // index order (measured only so).
+    DeviceInfo d;
+    rc = device_info(dev, d);
+    if (rc) return rc;
+    const bool waits = p.cluster == 0 && !p.pair && (n > p.grid || (vmax >= kWideMinStops && n > d.sms));
     if (own_workspace && n > 1 &&
         (order == EAT_ORDER_BY_TIME ||
          (order == EAT_ORDER_AUTO && n_nets == 1 && (waits || p.pair)))) {
@@ -499,6 +561,22 @@ static int make_plan(int dev, int32_t vmax, int32_t n, int n_nets, const eat_que
         p.ws_bytes = p.off_order + align_up((size_t)n * 4, 256);
     }
     return EAT_OK;
+}
+
+// Whether the round kernel prefetches: the edge tables of a launch's networks together do not
+// stay in L2.  (Large network, 1.1 GB, 96 queries 1,526 -> 1,426 us; 60,000 stops, 218 MB, 300
+// queries 1,210 -> 1,164; 64 ragged networks, 700 MB, 1,700 -> 1,538; but the city's 62 MB
+// stay in L2, and its 256 queries took 302 us with the prefetches against 287.)
+static constexpr int64_t kPrefetchBytes = (int64_t)96 << 20;
+
+static int32_t prefetch_wanted(const eat_net *const *nets, int n_nets) {
+    int64_t bytes = 0;
+    for (int i = 0; i < n_nets; ++i) {
+        const EdgeDev &e = nets[i]->edev;
+        if (e.big) return 0;
+        bytes += (int64_t)e.n_edges * e.y * 16;
+    }
+    return bytes > kPrefetchBytes;
 }
 
 // Kernel arguments for a plan; `grid` persistent blocks share the scratch at `ws`.
@@ -528,6 +606,7 @@ static QueryArgs make_args(const Plan &p, int grid, char *ws, const int32_t *net
     qa.mask_words = p.mask_words;
     qa.smem_mask_off = p.smem_mask_off;
     qa.smem_q_off = p.smem_q_off;
+    qa.smem_wait_off = p.smem_wait_off;
     qa.smem_arr_cap = p.smem_arr_cap;
     qa.arr_rows = nullptr;
     qa.arr_rows_stride = 0;
@@ -535,7 +614,15 @@ static QueryArgs make_args(const Plan &p, int grid, char *ws, const int32_t *net
     qa.idle_cap = kDefaultIdleCap;
     qa.rg = RingArgs{};
     qa.horizon = p.horizon;
+    qa.active = p.active ? p.active : p.block;
+    qa.prefetch = 0;
     return qa;
+}
+
+// Whether a launch's blocks take queries from the counter (zeroed before the launch): in the
+// round kernel and cluster mode a block's first query is its own index.
+static bool takes_counter(const Plan &p, int32_t n, int grid) {
+    return p.pair || p.async || (!p.cluster && n > grid);
 }
 
 // Per-block arrival rows needed when a plan keeps some arrivals out of shared memory
@@ -583,13 +670,15 @@ static int run_batch(const eat_net *const *nets, int n_nets, const int32_t *net_
                              cap, status_override ? status_override : (o ? o->status : nullptr),
                              counters_override ? counters_override : (o ? o->counters : nullptr));
     if (o && o->idle_cap > 0) qa.idle_cap = o->idle_cap;
+    qa.prefetch = prefetch_wanted(nets, n_nets);
     if (arr_rows && p.mem != 0) {
         if (arr_rows_size < arr_rows_bytes(p)) return fail(EAT_ERR_INVALID, "arrival rows too small");
         qa.arr_rows = arr_rows;
         qa.arr_rows_stride = (int64_t)align_up((size_t)p.vmax, 64);
     }
     DeviceGuard guard(dev);
-    cudaError_t e = cudaMemsetAsync(qa.work, 0, sizeof(int32_t), st);
+    cudaError_t e = cudaSuccess;
+    if (takes_counter(p, n, p.grid)) e = cudaMemsetAsync(qa.work, 0, sizeof(int32_t), st);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync");
     if (p.order) {
         e = launch_order(ts, n, (int32_t *)((char *)ws + p.off_order), st);
@@ -623,6 +712,7 @@ int ring_setup(const eat_net *const *nets, int n_nets, RingLaunch &rl) {
     if (rc) return rc;
     eat_query_opts o{};
     o.mode = EAT_MODE_CTA;
+    o.block = 512;
     Plan p;
     rc = make_plan(nets[0]->device, vmax, 4 * d.sms, n_nets, &o, p, vmin, nullptr, false);
     if (rc) return rc;
@@ -672,6 +762,7 @@ int ring_launch(const eat_net *const *nets, int n_nets, const RingLaunch &rl, vo
     QueryArgs qa = make_args(p, rl.grid, (char *)ws, nullptr, nullptr, nullptr, 0, n_nets, pool,
                              nullptr, default_round_cap(rl.vmax, p.horizon), nullptr, nullptr);
     qa.rg = rg;
+    qa.prefetch = prefetch_wanted(nets, n_nets);
     if (rl.mem != 0) {
         qa.arr_rows = arr_rows;
         qa.arr_rows_stride = rl.rows_stride;
@@ -772,6 +863,9 @@ static int upload(eat_net *net) {
     x.shift = h.e_shift;
     x.y = h.e_y;
     x.big = h.n_stops > kMaxPackedStops;
+    int64_t tails = 0;
+    for (int32_t u = 0; u < h.n_stops; ++u) tails += h.erow[u + 1] > h.erow[u];
+    net->branching = tails > 0 && x.n_edges >= 2 * tails;
     // No host view shows the edge table: its host copy goes.
     for (std::vector<int32_t> *w : {&h.erow, &h.er, &h.ee, &h.ex, &h.etypes}) std::vector<int32_t>().swap(*w);
     return EAT_OK;
@@ -1317,8 +1411,7 @@ extern "C" int eat_autotune(eat_net *net, const int32_t *sources, const int32_t 
     cudaStream_t st = (cudaStream_t)stream;
     const eat_net *nets[1] = {net};
     std::vector<TuneCand> cands;
-    // Fixed order, the library's default shape first (rounds, vwarp 8, 1,024 threads on
-    // networks of 8,192 stops or more, else 512): ties go to the earliest.
+    // Fixed order, the library's default block size first: ties go to the earliest.
     DeviceInfo dinfo;
     int drc = device_info(net->device, dinfo);
     if (drc) return drc;
@@ -1330,17 +1423,29 @@ extern "C" int eat_autotune(eat_net *net, const int32_t *sources, const int32_t 
             for (int v : {8, 4, 16}) pairs.push_back({EAT_MODE_PAIR, 1024, v, EAT_ORDER_AUTO, 0, {}});
         else clear_error();                  // network too large for two rows per block
     }
-    const bool wide = net->host.n_stops >= kWideMinStops || n <= dinfo.sms;
-    for (int b : {wide ? 1024 : 512, wide ? 512 : 1024, 256}) {
-        for (int v : {8, 4, 16, 2, 32}) cands.push_back({EAT_MODE_CTA, b, v, EAT_ORDER_AUTO, 0, {}});
+    // The automatic shape's block and horizon first, then the three block sizes.
+    eat_query_opts plain{};
+    plain.mode = EAT_MODE_CTA;
+    Plan first;
+    const int frc = make_plan(net->device, net->host.n_stops, n, 1, &plain, first, -1, net, true, false);
+    if (frc) return frc;
+    std::vector<int> blocks;
+    for (int b : {first.block, 1024, 512, 256})
+        if ((b == 256 || b == 512 || b == 1024) && std::find(blocks.begin(), blocks.end(), b) == blocks.end())
+            blocks.push_back(b);
+    const bool hours = first.horizon > 0;
+    auto with_horizons = [&](int b) {
+        for (int h : {3600, 7200, 14400, 43200}) cands.push_back({EAT_MODE_CTA, b, 8, EAT_ORDER_AUTO, h, {}});
+    };
+    if (hours)
+        for (int b : blocks) with_horizons(b);
+    for (int b : blocks) {
+        for (int v : {8, 4, 16}) cands.push_back({EAT_MODE_CTA, b, v, EAT_ORDER_AUTO, 0, {}});
         cands.push_back({EAT_MODE_ASYNC, b, 8, EAT_ORDER_AUTO, 0, {}});
-        for (int v : {8, 32}) cands.push_back({EAT_MODE_EDGE, b, v, EAT_ORDER_AUTO, 0, {}});
     }
     cands.insert(cands.end(), pairs.begin(), pairs.end());
-    // Horizons (1, 2, 4 and 12 hours) with the first two block sizes and vwarp 8.
-    for (int b : {wide ? 1024 : 512, wide ? 512 : 1024})
-        for (int h : {3600, 7200, 14400, 43200})
-            cands.push_back({EAT_MODE_CTA, b, 8, EAT_ORDER_AUTO, h, {}});
+    if (!hours)
+        for (int b : blocks) with_horizons(b);
     size_t ws_need = 0;
     int rc = usable_candidates(nets, 1, n, cands, ws_need);
     if (rc) return rc;
@@ -1352,9 +1457,7 @@ extern "C" int eat_autotune(eat_net *net, const int32_t *sources, const int32_t 
                          },
                          win);
     if (rc) return rc;
-    int cls = 0;
-    while (cls < 31 && (1 << (cls + 1)) <= n) ++cls;
-    net->tuned[cls].store((uint64_t)win.b | (uint64_t)win.v << 16 | (uint64_t)win.m << 24 |
+    net->tuned[log2_class(n)].store((uint64_t)win.b | (uint64_t)win.v << 16 | (uint64_t)win.m << 24 |
                               (uint64_t)(uint32_t)win.h << 32,
                           std::memory_order_relaxed);
     if (best) {
@@ -1411,15 +1514,14 @@ extern "C" int eat_autotune_multi(const eat_net *const *nets, int32_t n_nets, co
     }
     // Candidates in a fixed order, the library's default for a batch over several
     // networks first (512 threads, vwarp 8, index order): block sizes 512, 1,024 and
-    // 256, each with vwarp 8, 4, 16, 2, 32, the round-free mode and the edge mode, each
-    // in index order and then in order of t_s; then horizons of 2 and 12 hours (512
-    // threads, vwarp 8, in order of t_s).
+    // 256, each with vwarp 8, 4, 16 and the round-free mode, each in index order and then
+    // in order of t_s; then horizons of 2 and 12 hours (512 threads, vwarp 8, in order of
+    // t_s).
     std::vector<TuneCand> cands;
     for (int ord : {EAT_ORDER_AS_GIVEN, EAT_ORDER_BY_TIME})
         for (int b : {512, 1024, 256}) {
-            for (int v : {8, 4, 16, 2, 32}) cands.push_back({EAT_MODE_CTA, b, v, ord, 0, {}});
+            for (int v : {8, 4, 16}) cands.push_back({EAT_MODE_CTA, b, v, ord, 0, {}});
             cands.push_back({EAT_MODE_ASYNC, b, 8, ord, 0, {}});
-            cands.push_back({EAT_MODE_EDGE, b, 8, ord, 0, {}});
         }
     for (int h : {7200, 43200}) cands.push_back({EAT_MODE_CTA, 512, 8, EAT_ORDER_BY_TIME, h, {}});
     size_t ws_need = 0;
@@ -1493,8 +1595,11 @@ extern "C" int eat_query_batch_noalloc(const eat_net *net, const int32_t *source
     Plan p;
     int rc = make_plan(net->device, net->host.n_stops, n, 1, opts, p, -1, net, false);
     if (rc) return rc;
-    // Fewer persistent blocks so that their queue spill fits the fixed scratch.
-    const size_t per_block = (size_t)p.spill_stride * 4 + (size_t)p.mask_stride * 4;
+    // Fewer persistent blocks so that their queue spill fits the fixed scratch (with a horizon
+    // the documented 16 bytes a stop are asked for, though the bitmap takes less).
+    const size_t per_block =
+        std::max((size_t)p.spill_stride, p.horizon > 0 ? align_up((size_t)p.vmax * 4 + (size_t)p.mask_words, 64) : 0) * 4 +
+        (size_t)p.mask_stride * 4;
     const size_t fit = per_block ? (EAT_NOALLOC_SCRATCH_BYTES - kWsHeader) / per_block : (size_t)p.grid;
     if (fit < 1)
         return fail(EAT_ERR_INVALID, "network too large for the no-allocation scratch");
@@ -1508,9 +1613,11 @@ extern "C" int eat_query_batch_noalloc(const eat_net *net, const int32_t *source
                              nullptr, cap, opts ? opts->status : nullptr,
                              opts ? opts->counters : nullptr);
     if (opts && opts->idle_cap > 0) qa.idle_cap = opts->idle_cap;
+    qa.prefetch = prefetch_wanted(&net, 1);
     cudaStream_t st = (cudaStream_t)stream;
     // The query counter must start at zero; the queues need no clearing.
-    cudaError_t e = cudaMemsetAsync(qa.work, 0, sizeof(int32_t), st);
+    cudaError_t e = cudaSuccess;
+    if (takes_counter(p, n, grid)) e = cudaMemsetAsync(qa.work, 0, sizeof(int32_t), st);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync(no-allocation scratch)");
     e = p.pair    ? launch_pair(net->dev, qa, grid, p.block, p.smem, st)
         : p.async ? launch_async(&net->dev, 1, qa, p.mem, grid, p.block, p.smem, st)

@@ -736,7 +736,9 @@ int build_edges(HostNet &h) {
         h.erow.assign((size_t)V + 1, 0);
         h.er.assign((size_t)E * 2, 0);
         h.etypes.assign((size_t)E, 0);
+        // and one slot without departures, for tails reached after the last slot
         h.ee.assign((size_t)E * (size_t)h.e_y * 4, 0);
+        for (int64_t e = 0; e < E; ++e) h.ee.insert(h.ee.end(), {-1, -1, -1, 0});
     } catch (const std::bad_alloc &) {
         return fail(EAT_ERR_OOM, "host allocation of the edge table failed");
     }

@@ -134,20 +134,18 @@ __device__ __forceinline__ const int4 *entry_at(const NetDev &N, int32_t k, int3
     return N.ce + 2 * ((int64_t)k * N.n_types + t);
 }
 
-// Edge lookup with the list: four {departure, arrival} pairs (32 bytes) a load; a list ends
-// with a departure at or after every time of its slot, or with {kInf, kInf}.
-__device__ __forceinline__ int32_t edge_lookup(const EdgeDev &E, const int4 c, uint32_t rel,
-                                               int32_t start, int32_t e, int32_t &seen) {
-    int32_t a = edge_inline(c, rel, start);
-    if (a != kInf || c.w == 0) return a;
-    const int4 *p = reinterpret_cast<const int4 *>(E.ex + 4 * ((int64_t)c.w - 1));
+// Earliest arrival for a tail reached at e from the list x of an edge's entry: four
+// {departure, arrival} pairs (32 bytes) a load; a list ends with a departure at or after
+// every time of its slot, or with {kInf, kInf}.
+__device__ __forceinline__ int32_t edge_list(const EdgeDev &E, int32_t x, int32_t e, int32_t &seen) {
+    const int4 *p = reinterpret_cast<const int4 *>(E.ex + 4 * ((int64_t)x - 1));
+    int4 a, b;
     for (;; p += 2) {
-        int4 x, y;
-        load_entry(p, x, y);
+        load_entry(p, a, b);
         seen += 4;
-        if (y.z < e) continue;
-        return x.x >= e ? x.y : x.z >= e ? x.w : y.x >= e ? y.y : y.w;
+        if (b.z >= e) break;
     }
+    return a.x >= e ? a.y : a.z >= e ? a.w : b.x >= e ? b.y : b.w;
 }
 
 // getConnection of type t at time e: least departure >= e, or kInf (none after the

@@ -98,17 +98,14 @@ struct NetDev {
     int32_t y;                // clusters stored per type
 };
 
-// Slot of time e and e relative to the slot's start; e before the first slot counts as its
+// Slot of time e, its start, and e relative to that; e before the first slot counts as its
 // start (every departure is then >= e).  A slot >= E.y: no departure at or after e.
-EAT_HD inline uint32_t edge_slot(int32_t base, int32_t shift, int32_t e, uint32_t &rel) {
-    const uint32_t d = e > base ? (uint32_t)e - (uint32_t)base : 0u;
+EAT_HD inline uint32_t edge_slot(int32_t base, int32_t shift, int32_t e, uint32_t &rel, int32_t &start) {
+    const int32_t t = e > base ? e : base;
+    const uint32_t d = (uint32_t)t - (uint32_t)base;
     rel = d & ((1u << shift) - 1u);
+    start = (int32_t)((uint32_t)t - rel);
     return d >> shift;
-}
-
-// Start time of slot k.
-EAT_HD inline int32_t edge_slot_start(int32_t base, int32_t shift, uint32_t k) {
-    return (int32_t)((uint32_t)base + (k << shift));
 }
 
 // Earliest arrival over an edge from its entry c for a tail reached at `rel` in the slot that
@@ -166,6 +163,7 @@ struct eat_net {
     int64_t blob_bytes = 0;
     eat::NetDev dev{};
     eat::EdgeDev edev{};
+    bool branching = false;          // two or more edges per stop that has any
     // Internal workspace and staging buffers (eat_query, NULL-workspace batches).
     mutable std::mutex ws_lock;
     mutable void *ws = nullptr;

@@ -33,10 +33,10 @@
 // improved stop in the next round, so a stop first reached late by a path of few
 // connections is expanded, and its successors with it, again each time a later round
 // improves it.  With a horizon H a stop lowered to an arrival >= H is not queued but
-// waits (once, in a per-block list: the thread whose atomic min found it unreached adds
-// it); when no stop below H is left to expand, H moves to the least arrival given to a
-// waiting stop + horizon, waiting stops below the new H are queued, and those whose arrival
-// had dropped below the old H are dropped (they were queued by that lowering).  Every
+// waits (a bit in a per-block bitmap); when no stop below H is left to expand, H moves to
+// the least arrival given to a waiting stop + horizon, waiting stops below the new H are
+// queued, and those whose arrival had dropped below the old H are dropped (they were queued
+// by that lowering).  Every
 // lowered stop is still expanded with its arrival at some round after the lowering,
 // so the fixpoint is the same; only the order of relaxations changes (as
 // delta-stepping orders Bellman-Ford's).
@@ -136,6 +136,18 @@ __device__ __forceinline__ void ring_done(const RingArgs &R, int32_t slot, int32
 constexpr int32_t kNullItem = -1;           // hole left by a stop that spilled
 constexpr int32_t kFirstItem = INT32_MIN;    // flag on the first item of a stop
 
+// An edge's entry.  Beside a row in global memory L1 is left to the loads in flight (large
+// network, 1,024 queries 2,620 -> 2,566 us); with arrivals in shared memory a stop expanded
+// again in the next rounds finds its entries there (city 302 us with, 361 without).
+template <bool KEEP>
+__device__ __forceinline__ int4 load_slot(const int4 *p) {
+    if (KEEP) return __ldg(p);
+    int4 v;
+    asm("ld.global.nc.L1::no_allocate.v4.b32 {%0,%1,%2,%3}, [%4];"
+        : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
+}
+
 // `n` words of `p` (any 4-byte alignment) set to kInf by the block's threads, 16 bytes a
 // store between the first and the last 16-byte boundary.
 __device__ __forceinline__ void fill_inf(int32_t *p, int32_t n, int tid, int nthr) {
@@ -150,28 +162,34 @@ __device__ __forceinline__ void fill_inf(int32_t *p, int32_t n, int tid, int nth
 
 // Bound by the chain of dependent loads of a round (queue entry and e[u], then the edge's
 // record and entry, then e[v] and the atomics on the queue) times the rounds of the deepest
-// query, not by bandwidth.  Against one thread per (stop, connection type) item with the
-// 32-byte cluster entries (us per step, the same shapes): grid 256 queries 117 -> 69, city
-// 256 queries 531 -> 353, city 37 queries on hourly clusters 690 -> 290, 60,000 stops 300
-// queries 3,766 -> 2,019, large 96 queries 4,353 -> 2,889 and 1,024 queries with a horizon of
-// one hour 6,452 -> 4,230, 64 ragged networks 4,096 queries 1,979 -> 1,505.
+// query, not by bandwidth: each load in flight holds a 128-byte line of L1, which is why the
+// launch leaves L1 its share (kSmemBesideL1 in eat_api.cu).  So a round is kept short: one pass
+// over the stops, no branch that the common stop takes (a slot without departures instead
+// of a test for the last one, spilled stops in a loop of their own), counters that are never
+// reset, two barriers only where the horizon moves.  us per step, against one thread per
+// (stop, connection type) item with 32-byte cluster entries and no room for L1: grid 256
+// queries 117 -> 58, city 37 queries 690 -> 233, 256 queries 527 -> 305, 60,000 stops 300
+// queries 3,753 -> 954, large 96 queries 4,296 -> 1,041, 1,024 queries 6,325 -> 2,453, 64
+// ragged networks 4,096 queries 1,959 -> 868.
+// Blocks of up to 512 threads are built for three a SM (at most 40 registers): large network,
+// 1,024 queries 3,414 us against 3,787 for two.
 // COUNT: the build that fills qa.counters; without it the per-thread work counters are
 // dead code and compiled away (the timed launches pass no counters).  HZ: the build that
 // honours qa.horizon.
-template <int NETS, int ARR, bool SMEM_MASK, bool RING = false, bool COUNT = false, bool HZ = true>
-__global__ void __launch_bounds__(1024, 1)
+template <int NETS, int ARR, bool SMEM_MASK, int MAXT = 1024, bool RING = false, bool COUNT = false, bool HZ = true>
+__global__ void __launch_bounds__(MAXT, MAXT == 512 ? 3 : 1)
 eat_cta_kernel(const __grid_constant__ EdgeTable<NETS> nets, const QueryArgs qa) {
     extern __shared__ __align__(16) int32_t smem[];
     __shared__ int32_t s_q;
     __shared__ int32_t s_ring[4];     // ring mode: net, source, t_s, row of the request
-    __shared__ int32_t s_n[3];        // stops queued per round (rotating)
-    __shared__ int32_t s_wait[2];     // stops in either waiting list
-    __shared__ int32_t s_min[2];      // least arrival given to a stop waiting in it
-    __shared__ int32_t s_rel[2];      // stops released from it
+    __shared__ int32_t s_n[2];        // stops queued so far in even and in odd rounds
+    __shared__ int32_t s_min[2];      // least arrival given to a waiting stop (alternating)
+    __shared__ int32_t s_rel[2];      // stops released (alternating)
     __shared__ unsigned long long s_cnt[6];
 
     const int tid = threadIdx.x;
-    const int nthr = blockDim.x;
+    const int nthr = qa.active;        // threads that work
+    if (tid >= nthr) return;           // the barriers below wait for those that have not left
     const int32_t qcap = qa.qcap;
 
     // Stop queues and spilled stops; round r writes buffer r & 1.
@@ -179,11 +197,24 @@ eat_cta_kernel(const __grid_constant__ EdgeTable<NETS> nets, const QueryArgs qa)
     int32_t *const spill_base = qa.spill + (int64_t)blockIdx.x * qa.spill_stride;
     uint32_t *const mask_base = SMEM_MASK ? (uint32_t *)(smem + qa.smem_mask_off)
                                           : qa.gmask + (int64_t)blockIdx.x * qa.mask_stride;
-    // Stops waiting beyond the horizon: two lists of vmax stops.
-    int32_t *const wait_base = spill_base + 2 * (int64_t)qa.vmax;
+    // Stops waiting beyond the horizon: a bitmap, in shared memory where that has room.
+    const bool wait_shared = ARR == kArrShared && qa.smem_wait_off > 0;
+    uint32_t *const wait = wait_shared ? (uint32_t *)(smem + qa.smem_wait_off)
+                                       : (uint32_t *)(spill_base + 2 * (int64_t)qa.vmax);
+    bool clear_wait = true;           // the workspace holds anything, or a capped query's bits
 
-    for (;;) {
-        if (tid == 0) s_q = RING ? ring_next(qa.rg, s_ring) : next_query(qa);
+    for (bool first = true;; first = false) {
+        // A block's first query is its own index; the counter (zeroed before a launch with
+        // more queries than blocks) gives the others.
+        if (!first && !RING && qa.n <= (int32_t)gridDim.x) break;
+        if (tid == 0) {
+            if (RING) {
+                s_q = ring_next(qa.rg, s_ring);
+            } else {
+                const int32_t w = first ? (int32_t)blockIdx.x : (int32_t)gridDim.x + atomicAdd(qa.work, 1);
+                s_q = (qa.order && w < qa.n) ? __ldg(qa.order + w) : w;
+            }
+        }
         if (COUNT && tid < 6) s_cnt[tid] = 0;
         __syncthreads();
         const int q = s_q;
@@ -191,7 +222,9 @@ eat_cta_kernel(const __grid_constant__ EdgeTable<NETS> nets, const QueryArgs qa)
 
         const int ni = RING ? s_ring[0] : qa.net_idx == nullptr ? 0 : __ldg(qa.net_idx + q);
         const bool net_ok = (unsigned)ni < (unsigned)qa.n_nets;
-        const EdgeDev &N = nets.net[net_ok ? ni : 0];
+        const EdgeDev N = nets.net[net_ok ? ni : 0];
+        // Only networks too large for bitmaps in shared memory can be too large for packed records.
+        const bool big = !SMEM_MASK && N.big;
         const int32_t V = N.n_stops;
         const int64_t off = RING         ? (int64_t)s_ring[3] * qa.rg.row_stride
                             : qa.arr_off ? __ldg(qa.arr_off + q)
@@ -214,9 +247,10 @@ eat_cta_kernel(const __grid_constant__ EdgeTable<NETS> nets, const QueryArgs qa)
             mask1[i] = 0u;
         }
         const bool hz_on = HZ && qa.horizon > 0;
-        if (tid < 3) s_n[tid] = 0;
+        if (tid < 2) s_n[tid] = 0;
+        if (hz_on && clear_wait)
+            for (int32_t i = tid; i < qa.mask_words; i += nthr) wait[i] = 0u;
         if (HZ && tid < 2) {
-            s_wait[tid] = 0;
             s_min[tid] = kInf;
             s_rel[tid] = 0;
         }
@@ -229,7 +263,7 @@ eat_cta_kernel(const __grid_constant__ EdgeTable<NETS> nets, const QueryArgs qa)
             arr[s] = t_s;
             const int32_t row = __ldg(N.erow + s);
             const int32_t d = min(__ldg(N.erow + s + 1) - row, kCountOverflow);
-            queue[qcap] = make_int2(N.big ? s : (int32_t)((uint32_t)s | (uint32_t)d << 24), row);
+            queue[qcap] = make_int2(big ? s : (int32_t)((uint32_t)s | (uint32_t)d << 24), row);
         }
         __syncthreads();
 
@@ -238,87 +272,77 @@ eat_cta_kernel(const __grid_constant__ EdgeTable<NETS> nets, const QueryArgs qa)
         // Horizon H (kInf when there is none): a stop lowered to an arrival at or after
         // H waits until no stop below H is left to expand.
         int32_t H = hz_on && t_s < kInf - qa.horizon ? t_s + qa.horizon : kInf;
-        int wl = 0;                                       // list that new waiting stops join
-        int cs = 0;                                       // counter slot written this round
+        int wl = 0;                                       // counters that new waiting stops use
+        int32_t seen_wr = 0, seen_rd = 0;                 // s_n of either parity before the round
         int32_t c_vert = 0, c_types = 0, c_evals = 0, c_lookups = 0, c_aps = 0, c_relax = 0;
+        int2 *q_rd = queue + qcap, *q_wr = queue;         // stops queued last round, this round
+        int32_t *sp_rd = spill_base + qa.vmax, *sp_wr = spill_base;
+        uint32_t *cmask = mask1, *pmask = mask0;
+        int32_t *n_rd = s_n + 1, *n_wr = s_n;
+        auto swap = [](auto &a, auto &b) {
+            const auto x = a;
+            a = b;
+            b = x;
+        };
         while (n > 0 && rounds < qa.max_rounds) {
-            const int wr = rounds & 1, rd = wr ^ 1;
-            const int2 *const q_rd = queue + rd * qcap;
-            int2 *const q_wr = queue + wr * qcap;
-            const int32_t *const sp_rd = spill_base + (int64_t)rd * qa.vmax;
-            int32_t *const sp_wr = spill_base + (int64_t)wr * qa.vmax;
-            uint32_t *const pmask = wr ? mask1 : mask0;    // stops queued this round
-            uint32_t *const cmask = wr ? mask0 : mask1;    // stops queued last round
-            // The slot used next round was last read two barriers ago.
-            if (tid == 0) s_n[cs == 2 ? 0 : cs + 1] = 0;
-
             // Relaxation (Algorithm 3): when the candidate is below the e[v] read beside the
             // lookup, e[v] is lowered with an atomic min whose result is not waited for and
             // v goes on the next frontier: every lowering is made by a thread whose
             // candidate was below its read, so every lowering queues v (at most once a
             // round: the bitmap); a stop queued by a min that lost to a lower one made
-            // meanwhile only repeats work.  Beyond the horizon the result is waited for
-            // when e[v] was read as infinite: a stop with an arrival at or after H waits in
-            // the list already, so the one thread that finds it unreached adds it.
+            // meanwhile only repeats work.  Beyond the horizon a stop read as infinite gets
+            // its bit; one with an arrival at or after H has it already.  (An atomic min on
+            // a row in global memory whose result is waited for costs far more than the
+            // read and the two unwaited ones: queueing by its result took 1,529 against
+            // 1,411 us per 300 queries on 60,000 stops, 4,927 against 3,738 per 1,024 on
+            // the large network.)
             auto lower = [&](const int2 h, int32_t v, int32_t cand, int32_t ev) {
                 if (cand >= ev) return;
                 ++c_relax;
-                const bool out_edges = N.big ? __ldg(N.erow + v + 1) > h.y : (uint32_t)h.x >> 24;
+                atomicMin(arr + v, cand);
+                const bool leaf = big ? __ldg(N.erow + v + 1) == h.y : (uint32_t)h.x < 1u << 24;
+                const uint32_t bit = 1u << (v & 31);
                 if (HZ && cand >= H) {
-                    if (ev != kInf) atomicMin(arr + v, cand);
-                    else if (atomicMin(arr + v, cand) == kInf && out_edges)
-                        wait_base[(int64_t)wl * qa.vmax + atomicAdd(&s_wait[wl], 1)] = v;
+                    if (leaf) return;
+                    if (ev == kInf) atomicOr(wait + (v >> 5), bit);
                     atomicMin(&s_min[wl], cand);
                     return;
                 }
-                atomicMin(arr + v, cand);
-                if (!out_edges) return;
-                const uint32_t bit = 1u << (v & 31);
-                if (atomicOr(pmask + (v >> 5), bit) & bit) return;   // already queued
-                const int32_t pos = atomicAdd(&s_n[cs], 1);
-                if (pos < qcap) q_wr[pos] = h;
+                if ((atomicOr(pmask + (v >> 5), bit) & bit) != 0 || leaf) return;   // queued, or no edges
+                const int32_t pos = atomicAdd(n_wr, 1) - seen_wr;
+                if (qa.prefetch) {
+                    // The entries of v's edges start for L2 now; v is expanded next round.
+                    uint32_t rel;
+                    int32_t start;
+                    const uint32_t k = min(edge_slot(N.base, N.shift, cand, rel, start), (uint32_t)N.y);
+                    const int4 *const p = N.ee + (uint64_t)k * (uint32_t)N.n_edges + h.y;
+                    const uint32_t d = (uint32_t)h.x >> 24;
+                    asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
+                    if (d > 1) asm volatile("prefetch.global.L2 [%0];" ::"l"(p + (d - 1)));
+                }
+                if (__builtin_expect(pos < qcap, 1)) q_wr[pos] = h;
                 else sp_wr[pos - qcap] = v;
             };
-
-            // A sub-warp of 2^pl lanes per stop: `vwarp` lanes while that keeps every stop of
-            // the round in one pass, else four.
-            const int pl = (n << qa.vw_log2) <= nthr ? qa.vw_log2 : min(qa.vw_log2, 2);
-            const int lane = tid & ((1 << pl) - 1);
-            const int nsub = nthr >> pl;
-            for (int32_t i = tid >> pl; i < n; i += nsub) {
-                int32_t u, row, d;
-                if (i < qcap) {
-                    const int2 e = q_rd[i];
-                    row = e.y;
-                    u = N.big ? e.x : e.x & 0xffffff;
-                    d = N.big ? kCountOverflow : (int32_t)((uint32_t)e.x >> 24);
-                } else {
-                    u = __ldcg(sp_rd + (i - qcap));
-                    row = __ldg(N.erow + u);
-                    d = kCountOverflow;
-                }
+            // Stop u's edges t, t + P, ... of its d by the lanes of a sub-warp.
+            auto expand = [&](int32_t u, int32_t t, int32_t d, int P, int lane) {
                 const int32_t e_u = load_arr(arr, u, arr_shared);
-                if (d == kCountOverflow) d = __ldg(N.erow + u + 1) - row;
-                if (lane == 0) {
-                    cmask[u >> 5] = 0u;                     // every stop of the word is in this queue
-                    ++c_vert;
-                }
+                cmask[u >> 5] = 0u;                         // every stop of the word is in this queue
+                if (d == kCountOverflow) d = __ldg(N.erow + u + 1) - t;
                 uint32_t rel;
-                const uint32_t k = edge_slot(N.base, N.shift, e_u, rel);
-                if (k >= (uint32_t)N.y) {                   // no departure left anywhere
-                    if (COUNT)
-                        for (int32_t t = row + lane; t < row + d; t += 1 << pl) c_types += __ldg(N.etypes + t);
-                    continue;
-                }
-                const int32_t start = edge_slot_start(N.base, N.shift, k);
-                const int4 *const slab = N.ee + (int64_t)k * N.n_edges;
-                for (int32_t t = row + lane; t < row + d; t += 1 << pl) {
+                int32_t start;
+                // slot y holds no departures
+                const uint32_t k = min(edge_slot(N.base, N.shift, e_u, rel, start), (uint32_t)N.y);
+                const int4 *const slab = N.ee + (uint64_t)k * (uint32_t)N.n_edges;
+                if (COUNT) c_vert += lane == 0;
+                const int32_t end = t + d;
+#pragma unroll 1
+                for (t += lane; t < end; t += P) {
                     const int2 h = __ldg(N.er + t);
-                    const int4 c = __ldg(slab + t);
-                    const int32_t v = N.big ? h.x : h.x & 0xffffff;
+                    const int4 c = load_slot<ARR == kArrShared>(slab + t);
+                    const int32_t v = big ? h.x : h.x & 0xffffff;
                     const int32_t ev = load_arr(arr, v, arr_shared);
-                    int32_t seen = 3;
-                    const int32_t cand = edge_lookup(N, c, rel, start, e_u, seen);
+                    int32_t cand = edge_inline(c, rel, start), seen = 3;
+                    if (__builtin_expect(cand == kInf && c.w != 0, 0)) cand = edge_list(N, c.w, e_u, seen);
                     if (COUNT) {
                         c_types += __ldg(N.etypes + t);
                         ++c_lookups;
@@ -327,50 +351,98 @@ eat_cta_kernel(const __grid_constant__ EdgeTable<NETS> nets, const QueryArgs qa)
                     }
                     lower(h, v, cand, ev);
                 }
+            };
+
+            // A sub-warp of 2^pl lanes per stop: `vwarp` lanes while that keeps every stop of
+            // the round in one pass, else four.
+            const int pl = (n << qa.vw_log2) <= nthr ? qa.vw_log2 : min(qa.vw_log2, 2);
+            const int lane = tid & ((1 << pl) - 1);
+            const int nsub = nthr >> pl;
+            const int32_t nq = min(n, qcap);
+#pragma unroll 1
+            for (int32_t i = tid >> pl; i < nq; i += nsub) {
+                const int2 e = q_rd[i];
+                expand(big ? e.x : e.x & 0xffffff, e.y, big ? kCountOverflow : (int32_t)((uint32_t)e.x >> 24),
+                       1 << pl, lane);
+            }
+            if (n > qcap) {                                 // spilled stops
+#pragma unroll 1
+                for (int32_t i = tid >> 3; i < n - qcap; i += nthr >> 3) {
+                    const int32_t u = __ldcg(sp_rd + i);
+                    expand(u, __ldg(N.erow + u), kCountOverflow, 8, tid & 7);
+                }
             }
             __syncthreads();
-            n = s_n[cs];
-            // No stop below H is left: H moves on, in one pass over the waiting list.  The
-            // least arrival may be that of a stop since lowered below H, so that a pass
-            // can release none; the kept ones then give the exact least arrival.
-            while (HZ && hz_on && n == 0 && s_wait[wl] > 0) {
-                const int32_t nd = s_wait[wl], least = s_min[wl];
+            n = *n_wr - seen_wr;
+            seen_wr += n;
+            // No stop below H is left: H moves on, in one pass over the waiting bitmap (a word
+            // per thread, four in flight).  The least arrival may be that of a stop since
+            // lowered below H, so that a pass can release none; the kept ones then give the
+            // exact least arrival.
+            while (HZ && hz_on && n == 0 && s_min[wl] < kInf) {
+                const int32_t least = s_min[wl];
                 const int32_t Hn = least < kInf - qa.horizon ? least + qa.horizon : kInf;
-                const int32_t *const L = wait_base + (int64_t)wl * qa.vmax;
-                int32_t *const K = wait_base + (int64_t)(wl ^ 1) * qa.vmax;
                 int32_t m = kInf;
-                for (int32_t i = tid; i < nd; i += nthr) {
-                    const int32_t v = __ldcg(L + i);
-                    const int32_t e = load_arr(arr, v, arr_shared);
-                    if (e < H) continue;
-                    if (e >= Hn) {
-                        m = min(m, e);
-                        K[atomicAdd(&s_wait[wl ^ 1], 1)] = v;
-                        continue;
+                auto word = [&](int32_t w, const uint32_t x) {
+                    uint32_t keep = x;
+                    for (uint32_t left = x; left;) {
+                        int32_t v[2], e[2];
+#pragma unroll
+                        for (int j = 0; j < 2; ++j) {
+                            v[j] = left ? w * 32 + __ffs((int)left) - 1 : -1;
+                            left &= left - 1;
+                            e[j] = v[j] >= 0 ? load_arr(arr, v[j], arr_shared) : kInf;
+                        }
+#pragma unroll
+                        for (int j = 0; j < 2; ++j) {
+                            if (v[j] < 0) continue;
+                            if (e[j] >= Hn) {
+                                m = min(m, e[j]);
+                                continue;
+                            }
+                            keep &= ~(1u << (v[j] & 31));
+                            if (e[j] < H) continue;
+                            const int32_t pos = atomicAdd(&s_rel[wl], 1);
+                            if (pos < qcap) {
+                                const int32_t row = __ldg(N.erow + v[j]);
+                                const int32_t d = min(__ldg(N.erow + v[j] + 1) - row, kCountOverflow);
+                                q_wr[pos] = make_int2(
+                                    big ? v[j] : (int32_t)((uint32_t)v[j] | (uint32_t)d << 24), row);
+                            } else {
+                                sp_wr[pos - qcap] = v[j];
+                            }
+                        }
                     }
-                    const int32_t pos = atomicAdd(&s_rel[wl], 1);
-                    if (pos < qcap) {
-                        const int32_t row = __ldg(N.erow + v);
-                        const int32_t d = min(__ldg(N.erow + v + 1) - row, kCountOverflow);
-                        q_wr[pos] = make_int2(N.big ? v : (int32_t)((uint32_t)v | (uint32_t)d << 24), row);
-                    } else {
-                        sp_wr[pos - qcap] = v;
+                    if (keep != x) wait[w] = keep;
+                };
+                for (int32_t w = tid; w < nwords; w += 4 * nthr) {
+                    uint32_t x[4];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const int32_t i = w + j * nthr;
+                        x[j] = i >= nwords ? 0u : wait_shared ? wait[i] : __ldcg(wait + i);
                     }
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        if (x[j]) word(w + j * nthr, x[j]);
                 }
                 if (m < kInf) atomicMin(&s_min[wl ^ 1], m);
                 __syncthreads();
                 n = s_rel[wl];
                 H = Hn;
                 if (tid == 0) {
-                    s_wait[wl] = 0;
                     s_min[wl] = kInf;
                     s_rel[wl ^ 1] = 0;
                 }
                 wl ^= 1;
-                if (n == 0) __syncthreads();              // the list freed above is written next
+                if (n == 0) __syncthreads();              // the counters freed above are next
             }
-            cs = cs == 2 ? 0 : cs + 1;
             ++rounds;
+            swap(q_rd, q_wr);
+            swap(sp_rd, sp_wr);
+            swap(cmask, pmask);
+            swap(n_rd, n_wr);
+            swap(seen_rd, seen_wr);
         }
 
         if (arr_shared || qa.arr_rows) {
@@ -378,6 +450,7 @@ eat_cta_kernel(const __grid_constant__ EdgeTable<NETS> nets, const QueryArgs qa)
             copy_row(out, arr, V, arr_shared, tid, nthr);
         }
         const int32_t q_status = !valid ? EAT_ERR_INVALID : (n > 0 ? EAT_ERR_NO_CONVERGENCE : EAT_OK);
+        clear_wait = n > 0;
         if (RING) {
             __syncthreads();                              // the whole row is written
             if (tid == 0) ring_done(qa.rg, q, q_status);
@@ -1169,24 +1242,27 @@ eat_cluster_kernel(const __grid_constant__ NetTable<NETS> nets, const QueryArgs 
     cluster.sync();                                   // block 0 is done reading the others
 }
 
-template <int NETS, bool COUNT, bool HZ>
+template <int NETS, int MAXT, bool COUNT, bool HZ>
 static const void *cta_kernel_ptr(int mem) {
     switch (mem) {
-    case 0: return (const void *)eat_cta_kernel<NETS, kArrShared, true, false, COUNT, HZ>;
-    case 1: return (const void *)eat_cta_kernel<NETS, kArrGlobal, true, false, COUNT, HZ>;
-    case 3: return (const void *)eat_cta_kernel<NETS, kArrPerQuery, true, false, COUNT, HZ>;
-    default: return (const void *)eat_cta_kernel<NETS, kArrGlobal, false, false, COUNT, HZ>;
+    case 0: return (const void *)eat_cta_kernel<NETS, kArrShared, true, MAXT, false, COUNT, HZ>;
+    case 1: return (const void *)eat_cta_kernel<NETS, kArrGlobal, true, MAXT, false, COUNT, HZ>;
+    case 3: return (const void *)eat_cta_kernel<NETS, kArrPerQuery, true, MAXT, false, COUNT, HZ>;
+    default: return (const void *)eat_cta_kernel<NETS, kArrGlobal, false, MAXT, false, COUNT, HZ>;
     }
 }
 
 template <int NETS>
-static const void *cta_kernel_for(int mem, bool count, bool hz) {
-    if (count) return cta_kernel_ptr<NETS, true, true>(mem);   // honours a horizon, if there is one
-    return hz ? cta_kernel_ptr<NETS, false, true>(mem) : cta_kernel_ptr<NETS, false, false>(mem);
+static const void *cta_kernel_for(int mem, int block, bool count, bool hz) {
+    if (count) return cta_kernel_ptr<NETS, 1024, true, true>(mem);   // honours a horizon, if there is one
+    if (block > 512)
+        return hz ? cta_kernel_ptr<NETS, 1024, false, true>(mem) : cta_kernel_ptr<NETS, 1024, false, false>(mem);
+    return hz ? cta_kernel_ptr<NETS, 512, false, true>(mem) : cta_kernel_ptr<NETS, 512, false, false>(mem);
 }
 
-const void *cta_kernel(int nets, int mem, bool count, bool hz) {
-    return nets == 1 ? cta_kernel_for<1>(mem, count, hz) : cta_kernel_for<EAT_MAX_NETS>(mem, count, hz);
+const void *cta_kernel(int nets, int mem, int block, bool count, bool hz) {
+    return nets == 1 ? cta_kernel_for<1>(mem, block, count, hz)
+                     : cta_kernel_for<EAT_MAX_NETS>(mem, block, count, hz);
 }
 
 template <int NETS>
@@ -1235,16 +1311,17 @@ static cudaError_t launch_cta_t(const void *kernel, const EdgeDev *nets, int n_n
 
 cudaError_t launch_cta(const EdgeDev *nets, int n_nets, const QueryArgs &qa, int mem, int grid,
                        int block, size_t smem, cudaStream_t st) {
-    const void *k = cta_kernel(n_nets == 1 ? 1 : EAT_MAX_NETS, mem, qa.counters != nullptr, qa.horizon > 0);
+    const void *k = cta_kernel(n_nets == 1 ? 1 : EAT_MAX_NETS, mem, block, qa.counters != nullptr,
+                               qa.horizon > 0);
     return n_nets == 1 ? launch_cta_t<1>(k, nets, n_nets, qa, grid, block, smem, st)
                        : launch_cta_t<EAT_MAX_NETS>(k, nets, n_nets, qa, grid, block, smem, st);
 }
 
 const void *ring_kernel(int mem) {
     switch (mem) {
-    case 0: return (const void *)eat_cta_kernel<EAT_MAX_NETS, kArrShared, true, true, false, false>;
-    case 3: return (const void *)eat_cta_kernel<EAT_MAX_NETS, kArrPerQuery, true, true, false, false>;
-    default: return (const void *)eat_cta_kernel<EAT_MAX_NETS, kArrGlobal, true, true, false, false>;
+    case 0: return (const void *)eat_cta_kernel<EAT_MAX_NETS, kArrShared, true, 512, true, false, false>;
+    case 3: return (const void *)eat_cta_kernel<EAT_MAX_NETS, kArrPerQuery, true, 512, true, false, false>;
+    default: return (const void *)eat_cta_kernel<EAT_MAX_NETS, kArrGlobal, true, 512, true, false, false>;
     }
 }
 

@@ -53,6 +53,7 @@ struct QueryArgs {
     int32_t mask_words;        // words per bitmap (padded)
     int32_t smem_mask_off;     // int offset of the bitmaps in dynamic shared memory
     int32_t smem_q_off;        // int offset of the item buffers in dynamic shared memory
+    int32_t smem_wait_off;     // int offset of the waiting stops' bitmap, 0 = after the spilled stops
     int32_t smem_arr_cap;      // per-query placement: arrivals shared when n_stops <= this
     int32_t *arr_rows;         // [grid][arr_rows_stride]: a block's arrivals when they are not
                                // in shared memory and arr_out is host memory, or nullptr
@@ -60,9 +61,11 @@ struct QueryArgs {
     const int32_t *order;      // [n]: the i-th query handed out is order[i], or nullptr (i)
     int32_t idle_cap;          // round-free mode: empty 32-word bitmap scans in a row per warp
     RingArgs rg;               // ring mode only
+    int32_t prefetch;          // round kernel: a queued stop's entries are prefetched into L2
+    int32_t active;            // round kernel: threads of a block that work (a multiple of 32)
     int32_t horizon;           // seconds, 0 = none: stops lowered to an arrival at or after
                                // the horizon wait (per-query kernel); with one,
-                               // spill_stride >= 4 * vmax
+                               // spill_stride >= 2 * vmax + mask_words
 };
 
 // mem: 0 = arrivals and bitmaps in shared memory, 1 = arrivals global / bitmaps
@@ -70,7 +73,7 @@ struct QueryArgs {
 // the query's network fits.  nets: 1 or EAT_MAX_NETS (kernel table size).
 // count: the instantiation that fills qa.counters (launch_cta picks it when counters are
 // given); hz: the one that honours qa.horizon (launch_cta picks it when qa.horizon > 0).
-const void *cta_kernel(int nets, int mem, bool count = false, bool hz = false);
+const void *cta_kernel(int nets, int mem, int block, bool count = false, bool hz = false);
 cudaError_t launch_cta(const EdgeDev *nets, int n_nets, const QueryArgs &qa, int mem, int grid,
                        int block, size_t smem, cudaStream_t st);
 // Ring mode of the per-query kernel (serving): persistent blocks take requests from

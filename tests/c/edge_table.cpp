@@ -22,11 +22,12 @@ using namespace eat;
 
 static int32_t lookup(const HostNet &h, int64_t i, int32_t e) {
     uint32_t rel;
-    const uint32_t k = edge_slot(h.e_base, h.e_shift, e, rel);
+    int32_t start;
+    const uint32_t k = edge_slot(h.e_base, h.e_shift, e, rel, start);
     if (k >= (uint32_t)h.e_y) return EAT_INF;
     const int32_t *w = &h.ee[((size_t)k * h.etypes.size() + (size_t)i) * 4];
     const int4 c = {w[0], w[1], w[2], w[3]};
-    const int32_t a = edge_inline(c, rel, edge_slot_start(h.e_base, h.e_shift, k));
+    const int32_t a = edge_inline(c, rel, start);
     if (a != EAT_INF || c.w == 0) return a;
     for (size_t p = 8 * ((size_t)c.w - 1);; p += 8) {
         if (p + 8 > h.ex.size()) {

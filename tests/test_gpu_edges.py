@@ -69,3 +69,32 @@ def test_rows(which):
     got = eat.eat_query(net, int(src[3]), int(ts[3]))
     assert np.array_equal(got, want[3])
     net.close()
+
+
+@pytest.mark.parametrize("family,stops", [("grid", 1500), ("grid", 5000), ("grid", 13000), ("grid", 30000),
+                                          ("city", 3000), ("city", 21000), ("city", 60000)])
+def test_automatic_shapes(family, stops):
+    """Every automatic launch shape (block size, threads at work, placement, horizon) by batch
+    size on networks with and without a branching frontier, with and without counters."""
+    import os
+    from paper_1912_00966_gb300 import eat
+    if family == "grid":
+        tt = synth.grid_timetable(stops, max(2, stops // 25), 700 + stops, force_stop0=False)
+    else:
+        tt = synth.transit.geometric_timetable(stops, 4, stops // 60, (20, 40), (15, 40), 0.2,
+                                               synth.transit.PEAK_BANDS, 700 + stops)
+    net = eat.eat_build(tt.n_stops, tt.u, tt.v, tt.dep, tt.dur, device=0)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    most = 4 * sms + 40
+    q = synth.random_queries(tt, most, 71)
+    src, ts = torch.as_tensor(q.source).cuda(), torch.as_tensor(q.t_s).cuda()
+    want = torch.as_tensor(oracle.csa_many(oracle.SortedConnections(tt), q.source, q.t_s,
+                                           os.cpu_count() or 8)[0]).cuda()
+    out = torch.empty((most, stops), dtype=torch.int32, device="cuda")
+    counters = torch.zeros((most, 7), dtype=torch.int64, device="cuda")
+    for n in (1, 2, sms // 2, sms // 2 + 1, sms + 1, 3 * sms // 2 + 1, 2 * sms + 77, most):
+        for more in ({}, {"counters": counters}, {"max_rounds": 2 * stops + 2}):
+            out.fill_(-7)
+            eat.eat_query_batch(net, src[:n], ts[:n], out[:n], **more)
+            assert torch.equal(out[:n], want[:n]), (n, list(more))
+    net.close()
