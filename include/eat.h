@@ -174,7 +174,8 @@ typedef struct {
                                 when the batch has at most one query per SM or runs in the
                                 paired mode; on one network up to 1.5 queries per SM 1024
                                 from 8,192 stops on, else 512, and for fuller batches 128
-                                to 1024 by the network's size; 384 over several networks);
+                                to 1024 by the network's size and the batch's; 384 to 1024
+                                over several networks);
                                 else 64..1024, multiple of 32.  In an automatic block on a
                                 small network the threads that its rounds cannot fill leave
                                 at once */
@@ -208,9 +209,10 @@ typedef struct {
                                 batch size, else, for a call without a round cap on one
                                 network whose stops have two or more edges on average,
                                 two hours when the arrivals are in global memory and four
-                                hours in shared memory for 2 queries up to half the SM
-                                count and for more than 1.5 queries per SM; none otherwise
-                                and in eat_query_batch_noalloc); < 0 = none; > 0 with
+                                hours in shared memory for batches of two queries or more
+                                (from one to 1.125 queries per SM only where stops have 2.6
+                                edges or more); none otherwise and in
+                                eat_query_batch_noalloc); < 0 = none; > 0 with
                                 EAT_MODE_PAIR, EAT_MODE_ASYNC or EAT_MODE_CLUSTER is
                                 EAT_ERR_INVALID */
     int32_t *status;         /* optional [n] per-query eat_status, device memory */
@@ -228,9 +230,9 @@ enum eat_placement {
 enum eat_order {
     EAT_ORDER_AUTO = 0,      /* on one network: EAT_ORDER_BY_TIME when the batch has more
                                 queries than the launch runs at once (some wait for a
-                                free block), has more queries than the GPU has SMs on a
-                                network of 8,192 stops or more, or runs in EAT_MODE_PAIR;
-                                otherwise, and for batches over several networks,
+                                free block) or runs in EAT_MODE_PAIR; on one or several
+                                networks with one of 8,192 stops or more when it has more
+                                queries than the GPU has SMs; otherwise
                                 EAT_ORDER_AS_GIVEN */
     EAT_ORDER_BY_TIME = 1,   /* queries start in order of departure time t_s (15-minute
                                 buckets, earliest first; a one-block device counting sort
@@ -464,8 +466,8 @@ int eat_next_departure(const eat_net *net, const int32_t *types, const int32_t *
  * and 16 lanes per stop and with the asynchronous mode, without a horizon; when n
  * exceeds the SM count, the paired mode with vwarp 8, 4 and 16; and the round-based
  * mode with each block size, vwarp 8 and horizons of 1, 2, 4 and 12 hours, which come
- * first on networks where the automatic shape has a horizon; as far as they fit the
- * device.  They are run on the sample batch
+ * first on networks where the automatic shape has a horizon (with that one first); as far
+ * as they fit the device.  They are run on the sample batch
  * sources/times (n queries, device memory) in nine rounds over all candidates:
  * the first warms up, the other eight are timed with CUDA events on `stream`,
  * each after a write of twice the L2 size so that every timing starts with the
@@ -487,8 +489,9 @@ int eat_autotune(eat_net *net, const int32_t *sources, const int32_t *times, int
  * eat_autotune_multi -- choose the launch shape and start order of a batch over several
  * networks of uneven size (eat_query_batch_multi) by measurement; no counterpart in the
  * paper, as for eat_autotune.  Candidates, in this order: start order as given, then by
- * t_s (EAT_ORDER_AS_GIVEN, EAT_ORDER_BY_TIME); for each, block sizes 512, 1024 and 256
- * threads, each with the round-based mode and vwarp 8, 4, 16, then the
+ * t_s (EAT_ORDER_AS_GIVEN, EAT_ORDER_BY_TIME; the automatic one first); for each, block
+ * sizes 512, 1024 and 256 threads (the one nearest the automatic shape's first), each with
+ * the round-based mode and vwarp 8, 4, 16, then the
  * asynchronous mode; then the round-based mode with 512
  * threads, vwarp 8, start by t_s and horizons of 2 and 12 hours (the others run with
  * none); shapes without a plan for these networks are skipped.  They run on

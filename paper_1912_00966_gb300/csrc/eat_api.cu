@@ -109,9 +109,11 @@ static int device_info(int dev, DeviceInfo &out) {
         DeviceGuard guard(dev);
         for (int nets : {1, EAT_MAX_NETS})
             for (int mem = 0; mem < 4; ++mem)
-                for (const void *k : {cta_kernel(nets, mem, 1024), cta_kernel(nets, mem, 1024, true),
-                                      cta_kernel(nets, mem, 1024, false, true), cta_kernel(nets, mem, 512),
-                                      cta_kernel(nets, mem, 512, false, true), async_kernel(nets, mem),
+                for (const void *k : {cta_kernel(nets, mem, kOne1024), cta_kernel(nets, mem, kOne1024, true),
+                                      cta_kernel(nets, mem, kOne1024, false, true), cta_kernel(nets, mem, kTwo1024),
+                                      cta_kernel(nets, mem, kTwo1024, false, true), cta_kernel(nets, mem, kThree512),
+                                      cta_kernel(nets, mem, kThree512, false, true),
+                                      async_kernel(nets, mem),
                                       cluster_kernel(), pair_kernel(false), pair_kernel(true),
                                       ring_kernel(mem)}) {
                     e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -150,6 +152,7 @@ struct Plan {
     bool order = false;           // queries start by t_s (EAT_ORDER_BY_TIME): order array at off_order
     size_t off_order = 0;
     int32_t horizon = 0;          // seconds (eat_query_opts.horizon resolved), 0 = none
+    int build = kOne1024;         // registers of the round kernel
     int active = 0;               // threads of a block that work, 0 = all
 };
 
@@ -351,26 +354,37 @@ static int make_plan_core(int dev, int32_t vmax, int32_t n, int n_nets, const ea
         th = (int)(uint32_t)(sh >> 32);
     }
     // Default shape (a tuned shape or opts->block overrides).  Up to 1.5 queries per SM: one
-    // 1,024-thread block per SM (512 threads on networks below 8,192 stops once some queries
-    // wait).  Fuller batches on one network: as many threads as its rounds fill, several
+    // 1,024-thread block per query (512 threads on networks below 8,192 stops once some
+    // queries wait).  Fuller batches on one network: as many threads as its rounds fill, several
     // blocks per SM (us for 300 / 1,024 queries: 3,000-stop grid 96 / 114 with 128 threads
-    // against 105 / 160 with 512; 10,000-stop city 215 / 322 with 256 against 225 / 402;
-    // 20,000-stop city, 256 queries, 287 with 512 against 319 with 1,024), with arrivals in
-    // global memory 1,024 threads up to 2.5 queries per SM (100,000 stops, 300 / 600
-    // queries: 1,410 / 2,596 against 1,790 / 2,341 with 512).  Batches over several networks:
-    // 384 threads (4,096 queries on 64 ragged grids 824 us; 256: 901, 512: 911).
+    // against 105 / 160 with 512; 10,000-stop city 212 / 363 with 256 against 210 / 408;
+    // 20,000-stop city 293 / 637 with 512 against 309 / 736 with 1,024).  With arrivals in
+    // global memory two 1,024-thread blocks per SM, until there are enough queries to keep
+    // three of 512 threads busy (us for 512 / 1,024 queries: 60,000 stops 1,031 / 1,929
+    // against 1,224 / 1,468; 200,000 stops 1,478 / 2,594 against 1,976 / 2,472).  Batches over
+    // several networks: 384 threads (64 grids of up to 50,000 stops, 4,096 queries 709 us, 512
+    // 835, 256 801), and with large networks among them fewer and larger blocks for fewer
+    // queries (1,024 queries on the 64: 512 threads 524, 384 586, 1,024 614; 512 queries on
+    // 20: 1,024 threads 345, 512 414, 384 469).
     const bool wide = vmax >= kWideMinStops;
     const bool full = 2 * (int64_t)n > 3 * (int64_t)d.sms;
-    const bool one_shared = vmax <= kOneSharedStops, two_shared = vmax <= kTwoSharedStops;
+    const bool two_shared = vmax <= kTwoSharedStops, one_shared = vmax <= kOneSharedStops;
     const bool rounds = !o || o->mode == EAT_MODE_AUTO || o->mode == EAT_MODE_CTA || o->mode == EAT_MODE_EDGE;
+    const bool branching = n_nets == 1 && tuned && tuned->branching > 0;
+    // One network whose arrivals fit an SM only once: from two queries per SM on where stops
+    // branch, else from four, rows in global memory do more (us in shared / global memory:
+    // 35,000-stop city, 400 queries 568 / 507, 512 707 / 565; 30,000-stop grid, 512 queries
+    // 326 / 350, 1,024 queries 603 / 490).
+    const bool spread = n_nets == 1 && !two_shared && rounds && n > (branching ? 2 : 4) * d.sms;
     int block = 512;
     if ((n >= 1 && n <= d.sms) || (!rounds && n_nets == 1 && wide)) block = 1024;
     else if (!rounds) block = 512;
-    else if (n_nets > 1) block = 384;
+    else if (n_nets > 1) block = vmax < 16384 || n > 16 * d.sms ? 384 : n > 4 * d.sms ? 512 : 1024;
     else if (!full) block = wide ? 1024 : 512;
     else if (vmax < 4096) block = 128;
     else if (vmax < 12288) block = 256;
-    else if (!two_shared && (one_shared ? n <= 4 * d.sms : 2 * (int64_t)n <= 5 * (int64_t)d.sms)) block = 1024;
+    else if (!two_shared && n <= (one_shared ? 3 : vmax < 80000 ? 4 : 5) * d.sms && (branching || !one_shared))
+        block = 1024;
     p.block = (o && o->block) ? o->block : (tb ? tb : block);
     if (p.block < 64 || p.block > 1024 || p.block % 32)
         return fail(EAT_ERR_INVALID, "block must be a multiple of 32 in 64..1024");
@@ -438,28 +452,26 @@ static int make_plan_core(int dev, int32_t vmax, int32_t n, int n_nets, const ea
         return fail(EAT_ERR_INVALID, "bitmaps do not fit in shared memory");
     // A batch over networks of uneven size whose largest arrival row does not fit the share
     // of an SM's shared memory that as many blocks leave each other as it can have queries
-    // there (up to four) keeps arrivals in shared memory only for the networks that do (64
-    // grids of 1,000 to 50,000 stops, 4,096 queries: a quarter of an SM 824 us, a third
-    // 1,005, half 1,265, a sixth 834).  The ring kernel, which serves single requests as they
-    // come, is sized for two blocks.
+    // there (up to five) keeps arrivals in shared memory only for the networks that do (64
+    // grids of 1,000 to 50,000 stops, 4,096 queries in 384-thread blocks: a fifth of an SM
+    // 709 us, a quarter 805; in 512-thread blocks a quarter 833, a third 1,005, half 1,265).
+    // The ring kernel, which serves single requests as they come, is sized for two blocks.
     const bool ring = n_nets > 1 && !own_workspace;
-    const int parts = ring ? 2 : (int)std::min<int64_t>(4, (std::max(n, 1) + d.sms - 1) / d.sms);
+    const int parts = ring ? 2 : std::max(1, std::min({5, 2048 / p.block, (std::max(n, 1) + d.sms - 1) / d.sms}));
     const size_t share = (parts <= 2 ? d.smem_per_sm : kSmemBesideL1) / (size_t)parts - d.reserve;
     p.smem_arr_cap = 0;
     if (place == EAT_PLACE_AUTO && vmin < vmax && base(0) + kQueueEntryBytes * qmin > share && fits(1)) {
-        const int64_t room = (int64_t)share - (int64_t)base(1) - (int64_t)(kQueueEntryBytes * 512);
-        const int32_t cap = (int32_t)std::min<int64_t>(room / 4 & ~(int64_t)3, (int64_t)vmax);
-        if (cap >= vmin) {
+        // What the queue leaves holds the arrivals and bitmaps of a network that fits, or the
+        // bitmaps alone: 4.25 bytes a stop (and two bitmaps' padding).
+        const int64_t room = (int64_t)share - (int64_t)(kQueueEntryBytes * 512);
+        const int64_t cap = (room - 128) * 4 / 17 & ~(int64_t)3;
+        if (room >= (int64_t)mask_bytes && cap >= vmin) {
             p.mem = 3;
-            p.smem_arr_cap = cap;
+            p.smem_arr_cap = (int32_t)std::min<int64_t>(cap, vmax);
         }
     }
-    // One network whose arrivals fit an SM only once: with more than four queries per SM three
-    // blocks with their rows in global memory do more (30,000 stops, 1,024 queries 471 us
-    // against 603; 50,000: 570 against 701).
-    const bool spread = n_nets == 1 && !two_shared && n > 4 * d.sms && p.block <= 512 && fits(1) && rounds;
     if (p.mem == 3) {
-    } else if (place == EAT_PLACE_SHARED || (place == EAT_PLACE_AUTO && fits(0) && !spread)) p.mem = 0;
+    } else if (place == EAT_PLACE_SHARED || (place == EAT_PLACE_AUTO && fits(0) && !(spread && fits(1)))) p.mem = 0;
     else if (place == EAT_PLACE_GLOBAL_ARR || (place == EAT_PLACE_AUTO && fits(1))) p.mem = 1;
     else p.mem = 2;
 
@@ -467,11 +479,15 @@ static int make_plan_core(int dev, int32_t vmax, int32_t n, int n_nets, const ea
     // (where they have fewer, a stop is seldom improved again and a horizon only adds rounds:
     // 3,000-stop grid, 300 queries 105 -> 119 us with four hours): two hours with arrivals in
     // global memory (200,000 stops, 96 queries 2,960 -> 1,600; one hour and four hours within
-    // 7 %), four hours in shared memory for full batches (20,000-stop city, 256 queries
-    // 390 -> 287) and for a few queries (37: 268 -> 224; a single one gains nothing).
+    // 7 %), four hours in shared memory (20,000-stop city, 37 queries 268 -> 224, 256 queries
+    // 390 -> 287) for all but a single query, which gains nothing, and batches of about one
+    // query per SM, which keep the shape that is documented for them unless stops have 2.6
+    // edges or more (30,000 stops with 2.7, 160 queries 888 -> 468).
     int32_t automatic = 0;
-    if (own_workspace && n_nets == 1 && tuned && tuned->branching && !(o && o->max_rounds > 0))
-        automatic = p.mem != 0 ? 7200 : full || (n > 1 && 2 * (int64_t)n <= d.sms) ? 14400 : 0;
+    if (own_workspace && branching && !(o && o->max_rounds > 0)) {
+        const bool one_each = n >= d.sms && n <= d.sms + d.sms / 8;
+        automatic = p.mem != 0 ? 7200 : n > 1 && (!one_each || tuned->branching > 1) ? 14400 : 0;
+    }
     p.horizon = oh > 0 ? oh : oh < 0 ? 0 : tb ? th : automatic;
     // Threads at work in a default-shaped block (the others leave): no more than the rounds
     // of a small network fill (1,024 stops, 256 queries: 128 of 512 threads 62 us, all 69;
@@ -479,11 +495,17 @@ static int make_plan_core(int dev, int32_t vmax, int32_t n, int n_nets, const ea
     p.active = p.block;
     if (!(o && o->block) && !tb && p.mem == 0)
         p.active = std::min(p.block, vmax < 2048 ? 128 : vmax < 6144 ? 256 : vmax <= 32768 ? 512 : 1024);
+    p.build = p.block <= 512 ? kThree512 : n <= d.sms ? kOne1024 : kTwo1024;
     const size_t qbytes = kQueueEntryBytes;
-    // As many blocks per SM as the threads and the registers allow (shared memory is the only
-    // other limit, and the one sized here), and the largest queue, up to kQueueMost stops,
-    // that keeps them and leaves L1 its share.
-    const size_t bm = p.mem == 3 ? base(1) + (size_t)p.smem_arr_cap * 4 : base(p.mem);
+    // As many blocks per SM as the threads and the registers allow and, with rows in global
+    // memory, as leave L1 its share with a queue of 512 stops each (200,000 stops, 1,024
+    // queries: three 512-thread blocks 2,400 us, four, which leave L1 28 KB, 3,500; with rows
+    // in shared memory one block more is worth more than L1: 14,500-stop city, 583 queries,
+    // three blocks 286, two 347); then the largest queue, up to kQueueMost stops, that keeps
+    // them and L1's share.
+    const size_t cap_words = ((size_t)p.smem_arr_cap + 31) / 32;
+    const size_t bm = p.mem == 3 ? std::max(align_up((size_t)p.smem_arr_cap, 4) * 4 + 8 * align_up(cap_words, 4), mask_bytes)
+                                 : base(p.mem);
     // The bitmap of waiting stops beside shared arrivals, where that leaves room for a queue.
     const size_t wait_bytes = (size_t)p.mask_words * 4;
     const bool wait_shared = p.mem == 0 && p.horizon > 0 && bm + wait_bytes + qbytes * qmin <= limit;
@@ -492,25 +514,24 @@ static int make_plan_core(int dev, int32_t vmax, int32_t n, int n_nets, const ea
     int reg_blocks = 0;
     {
         DeviceGuard guard(dev);
-        const void *k = cta_kernel(p.nets, p.mem, p.block, false, p.horizon > 0);
+        const void *k = cta_kernel(p.nets, p.mem, p.build, false, p.horizon > 0);
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&reg_blocks, k, p.block, 0) != cudaSuccess) {
             cudaGetLastError();
             reg_blocks = 0;
         }
     }
     const int max_blocks = std::max(1, std::min(2048 / p.block, reg_blocks > 0 ? reg_blocks : 2048));
-    p.qcap = (int32_t)qmin;
-    for (int b = max_blocks; b >= 1; --b) {
-        const size_t budget = std::min(limit, d.smem_per_sm / (size_t)b - d.reserve);
-        if (d.smem_per_sm / (size_t)b < d.reserve || b0 + qbytes * qmin > budget) continue;
-        const size_t beside = kSmemBesideL1 / (size_t)b - 1024;   // 1 KB of each block is the driver's
-        const size_t room = b0 + qbytes * qmin <= beside ? std::min(budget, beside) : budget;
-        size_t cap = std::min({(room - b0) / qbytes, (size_t)std::max(vmax, 1), kQueueMost});
-        if (cap >= 64) cap &= ~(size_t)31;
-        p.qcap = (int32_t)std::max(cap, qmin);
-        break;
-    }
-    p.smem_mask_off = p.mem == 0 ? (int32_t)(arr_bytes / 4) : p.mem == 3 ? p.smem_arr_cap : 0;
+    const size_t qplenty = qbytes * (p.mem == 0 ? qmin : std::min<size_t>((size_t)std::max(vmax, 1), 512)) + 1024;
+    const size_t most = p.mem == 0 ? d.smem_per_sm - 1024 : kSmemBesideL1;   // 1 KB of each block is the driver's
+    int blocks = max_blocks;
+    while (blocks > 1 && (size_t)blocks * (b0 + qplenty) > most) --blocks;
+    const size_t beside = kSmemBesideL1 / (size_t)blocks - 1024;
+    const size_t room = b0 + qbytes * qmin <= beside ? beside : std::min(limit, d.smem_per_sm / (size_t)blocks - d.reserve);
+    size_t cap = room > b0 ? (room - b0) / qbytes : 0;
+    cap = std::min({cap, (size_t)std::max(vmax, 1), kQueueMost});
+    if (cap >= 64) cap &= ~(size_t)31;
+    p.qcap = (int32_t)std::max(cap, qmin);
+    p.smem_mask_off = p.mem == 0 ? (int32_t)(arr_bytes / 4) : 0;   // mem 3: after the query's own row
     p.smem_q_off = (int32_t)(b0 / 4);
     p.smem = b0 + qbytes * (size_t)p.qcap;
 
@@ -519,7 +540,7 @@ static int make_plan_core(int dev, int32_t vmax, int32_t n, int n_nets, const ea
     {
         DeviceGuard guard(dev);
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-            &per_sm, cta_kernel(p.nets, p.mem, p.block, false, p.horizon > 0), p.block, p.smem);
+            &per_sm, cta_kernel(p.nets, p.mem, p.build, false, p.horizon > 0), p.block, p.smem);
     }
     if (e != cudaSuccess) return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
     if (per_sm < 1) return fail(EAT_ERR_INVALID, "kernel does not fit on an SM with this block size");
@@ -547,15 +568,16 @@ static int make_plan(int dev, int32_t vmax, int32_t n, int n_nets, const eat_que
     // Automatic, on one network: sorted when some queries must wait for a free block or share
     // an SM of a network of 8,192 stops or more (they then start longest first) and in the
     // paired mode (an early query shares its block with a late one); a batch that starts
-    // all at once gains nothing for the sort's launch.  Batches over several networks keep
-    // index order (measured only so).
+    // all at once gains nothing for the sort's launch.  Batches over several networks only
+    // with one of 8,192 stops or more among them (64 grids of up to 50,000 stops, 4,096 queries
+    // 1,041 -> 709 us, 256 queries 366 -> 317).
     DeviceInfo d;
     rc = device_info(dev, d);
     if (rc) return rc;
     const bool waits = p.cluster == 0 && !p.pair && (n > p.grid || (vmax >= kWideMinStops && n > d.sms));
     if (own_workspace && n > 1 &&
         (order == EAT_ORDER_BY_TIME ||
-         (order == EAT_ORDER_AUTO && n_nets == 1 && (waits || p.pair)))) {
+         (order == EAT_ORDER_AUTO && (n_nets == 1 || vmax >= kWideMinStops) && (waits || p.pair)))) {
         p.order = true;
         p.off_order = align_up(p.ws_bytes, 256);
         p.ws_bytes = p.off_order + align_up((size_t)n * 4, 256);
@@ -693,7 +715,7 @@ static int run_batch(const eat_net *const *nets, int n_nets, const int32_t *net_
     e = p.cluster ? launch_cluster(devs[0], qa, p.cluster, p.grid, p.block, p.smem, st)
         : p.pair  ? launch_pair(devs[0], qa, p.grid, p.block, p.smem, st)
         : p.async ? launch_async(devs, n_nets, qa, p.mem, p.grid, p.block, p.smem, st)
-                  : launch_cta(edges, n_nets, qa, p.mem, p.grid, p.block, p.smem, st);
+                  : launch_cta(edges, n_nets, qa, p.mem, p.build, p.grid, p.block, p.smem, st);
     if (e != cudaSuccess) return cuda_fail(e, "query kernel launch");
     return EAT_OK;
 }
@@ -865,7 +887,7 @@ static int upload(eat_net *net) {
     x.big = h.n_stops > kMaxPackedStops;
     int64_t tails = 0;
     for (int32_t u = 0; u < h.n_stops; ++u) tails += h.erow[u + 1] > h.erow[u];
-    net->branching = tails > 0 && x.n_edges >= 2 * tails;
+    net->branching = tails == 0 ? 0 : 5 * (int64_t)x.n_edges >= 13 * tails ? 2 : x.n_edges >= 2 * tails ? 1 : 0;
     // No host view shows the edge table: its host copy goes.
     for (std::vector<int32_t> *w : {&h.erow, &h.er, &h.ee, &h.ex, &h.etypes}) std::vector<int32_t>().swap(*w);
     return EAT_OK;
@@ -1435,7 +1457,10 @@ extern "C" int eat_autotune(eat_net *net, const int32_t *sources, const int32_t 
             blocks.push_back(b);
     const bool hours = first.horizon > 0;
     auto with_horizons = [&](int b) {
-        for (int h : {3600, 7200, 14400, 43200}) cands.push_back({EAT_MODE_CTA, b, 8, EAT_ORDER_AUTO, h, {}});
+        const int own = first.horizon == 7200 || first.horizon == 14400 ? first.horizon : 3600;
+        cands.push_back({EAT_MODE_CTA, b, 8, EAT_ORDER_AUTO, own, {}});
+        for (int h : {3600, 7200, 14400, 43200})
+            if (h != own) cands.push_back({EAT_MODE_CTA, b, 8, EAT_ORDER_AUTO, h, {}});
     };
     if (hours)
         for (int b : blocks) with_horizons(b);
@@ -1512,20 +1537,34 @@ extern "C" int eat_autotune_multi(const eat_net *const *nets, int32_t n_nets, co
         cudaFree(d_offs);
         return cuda_fail(e, "cudaMemcpy of the row offsets");
     }
-    // Candidates in a fixed order, the library's default for a batch over several
-    // networks first (512 threads, vwarp 8, index order): block sizes 512, 1,024 and
-    // 256, each with vwarp 8, 4, 16 and the round-free mode, each in index order and then
-    // in order of t_s; then horizons of 2 and 12 hours (512 threads, vwarp 8, in order of
-    // t_s).
+    // Candidates in a fixed order, the automatic start order and block size first (256 where
+    // that is 384): each start order with three block sizes, each with vwarp 8, 4, 16 and the
+    // round-free mode; then horizons of 2 and 12 hours (512 threads, vwarp 8, in order of t_s).
+    int32_t vmax = 0, vmin = INT32_MAX;
+    for (int i = 0; i < n_nets; ++i) {
+        vmax = std::max(vmax, nets[i]->host.n_stops);
+        vmin = std::min(vmin, nets[i]->host.n_stops);
+    }
+    Plan first;
+    eat_query_opts plain{};
+    int rc = make_plan(dev, vmax, n, n_nets, &plain, first, vmin, n_nets == 1 ? nets[0] : nullptr, true, false);
+    if (rc) {
+        cudaFree(d_offs);
+        return rc;
+    }
+    std::vector<int> blocks;
+    for (int b : {first.block < 512 ? 256 : first.block < 1024 ? 512 : 1024, 512, 1024, 256})
+        if (std::find(blocks.begin(), blocks.end(), b) == blocks.end()) blocks.push_back(b);
     std::vector<TuneCand> cands;
-    for (int ord : {EAT_ORDER_AS_GIVEN, EAT_ORDER_BY_TIME})
-        for (int b : {512, 1024, 256}) {
+    const int ord0 = first.order ? EAT_ORDER_BY_TIME : EAT_ORDER_AS_GIVEN;
+    for (int ord : {ord0, EAT_ORDER_BY_TIME + EAT_ORDER_AS_GIVEN - ord0})
+        for (int b : blocks) {
             for (int v : {8, 4, 16}) cands.push_back({EAT_MODE_CTA, b, v, ord, 0, {}});
             cands.push_back({EAT_MODE_ASYNC, b, 8, ord, 0, {}});
         }
     for (int h : {7200, 43200}) cands.push_back({EAT_MODE_CTA, 512, 8, EAT_ORDER_BY_TIME, h, {}});
     size_t ws_need = 0;
-    int rc = usable_candidates(nets, n_nets, n, cands, ws_need);
+    rc = usable_candidates(nets, n_nets, n, cands, ws_need);
     TuneCand win{EAT_MODE_CTA, 512, 8, EAT_ORDER_AS_GIVEN, 0, {}};
     if (!rc)
         rc = time_candidates(dev, cands, ws_need, (size_t)total * 4, st,
@@ -1621,7 +1660,7 @@ extern "C" int eat_query_batch_noalloc(const eat_net *net, const int32_t *source
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync(no-allocation scratch)");
     e = p.pair    ? launch_pair(net->dev, qa, grid, p.block, p.smem, st)
         : p.async ? launch_async(&net->dev, 1, qa, p.mem, grid, p.block, p.smem, st)
-                  : launch_cta(&net->edev, 1, qa, p.mem, grid, p.block, p.smem, st);
+                  : launch_cta(&net->edev, 1, qa, p.mem, p.build, grid, p.block, p.smem, st);
     if (e != cudaSuccess) return cuda_fail(e, "query kernel launch");
     return EAT_OK;
 }

@@ -163,7 +163,7 @@ struct eat_net {
     int64_t blob_bytes = 0;
     eat::NetDev dev{};
     eat::EdgeDev edev{};
-    bool branching = false;          // two or more edges per stop that has any
+    int branching = 0;               // 1: two or more edges per stop that has any, 2: 2.6 or more
     // Internal workspace and staging buffers (eat_query, NULL-workspace batches).
     mutable std::mutex ws_lock;
     mutable void *ws = nullptr;

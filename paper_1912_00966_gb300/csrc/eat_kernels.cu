@@ -171,13 +171,16 @@ __device__ __forceinline__ void fill_inf(int32_t *p, int32_t n, int tid, int nth
 // queries 117 -> 58, city 37 queries 690 -> 233, 256 queries 527 -> 305, 60,000 stops 300
 // queries 3,753 -> 954, large 96 queries 4,296 -> 1,041, 1,024 queries 6,325 -> 2,453, 64
 // ragged networks 4,096 queries 1,959 -> 868.
-// Blocks of up to 512 threads are built for three a SM (at most 40 registers): large network,
-// 1,024 queries 3,414 us against 3,787 for two.
+// BUILD: registers by how many blocks an SM is to hold (large network: 1,024 queries in
+// 512-thread blocks 2,400 us at 40 registers, three per SM, against 2,525 at 32; 96 queries in
+// 1,024-thread blocks 1,039 at 56 against 1,113 at 32; 60,000 stops, 300 queries, two
+// 1,024-thread blocks per SM 851 against 969 for one).
 // COUNT: the build that fills qa.counters; without it the per-thread work counters are
 // dead code and compiled away (the timed launches pass no counters).  HZ: the build that
 // honours qa.horizon.
-template <int NETS, int ARR, bool SMEM_MASK, int MAXT = 1024, bool RING = false, bool COUNT = false, bool HZ = true>
-__global__ void __launch_bounds__(MAXT, MAXT == 512 ? 3 : 1)
+template <int NETS, int ARR, bool SMEM_MASK, int BUILD, bool RING = false, bool COUNT = false, bool HZ = true>
+__global__ void __launch_bounds__(BUILD == kThree512 ? 512 : 1024,
+                                  BUILD == kThree512 ? 3 : BUILD == kTwo1024 ? 2 : 1)
 eat_cta_kernel(const __grid_constant__ EdgeTable<NETS> nets, const QueryArgs qa) {
     extern __shared__ __align__(16) int32_t smem[];
     __shared__ int32_t s_q;
@@ -237,8 +240,9 @@ eat_cta_kernel(const __grid_constant__ EdgeTable<NETS> nets, const QueryArgs qa)
                              : qa.arr_rows ? qa.arr_rows + (int64_t)blockIdx.x * qa.arr_rows_stride
                                            : out;
         const int32_t nwords = (V + 31) >> 5;
-        uint32_t *const mask0 = mask_base;
-        uint32_t *const mask1 = mask_base + qa.mask_words;
+        // Per-query placement: the bitmaps follow the query's own row (or take its place).
+        uint32_t *const mask0 = mask_base + (ARR == kArrPerQuery && arr_shared ? (V + 3) & ~3 : 0);
+        uint32_t *const mask1 = mask0 + (ARR == kArrPerQuery ? (nwords + 3) & ~3 : qa.mask_words);
 
         // Algorithm 2: every stop passive at infinity.
         fill_inf(arr, V, tid, nthr);
@@ -1242,27 +1246,32 @@ eat_cluster_kernel(const __grid_constant__ NetTable<NETS> nets, const QueryArgs 
     cluster.sync();                                   // block 0 is done reading the others
 }
 
-template <int NETS, int MAXT, bool COUNT, bool HZ>
+template <int NETS, int BUILD, bool COUNT, bool HZ>
 static const void *cta_kernel_ptr(int mem) {
     switch (mem) {
-    case 0: return (const void *)eat_cta_kernel<NETS, kArrShared, true, MAXT, false, COUNT, HZ>;
-    case 1: return (const void *)eat_cta_kernel<NETS, kArrGlobal, true, MAXT, false, COUNT, HZ>;
-    case 3: return (const void *)eat_cta_kernel<NETS, kArrPerQuery, true, MAXT, false, COUNT, HZ>;
-    default: return (const void *)eat_cta_kernel<NETS, kArrGlobal, false, MAXT, false, COUNT, HZ>;
+    case 0: return (const void *)eat_cta_kernel<NETS, kArrShared, true, BUILD, false, COUNT, HZ>;
+    case 1: return (const void *)eat_cta_kernel<NETS, kArrGlobal, true, BUILD, false, COUNT, HZ>;
+    case 3: return (const void *)eat_cta_kernel<NETS, kArrPerQuery, true, BUILD, false, COUNT, HZ>;
+    default: return (const void *)eat_cta_kernel<NETS, kArrGlobal, false, BUILD, false, COUNT, HZ>;
     }
 }
 
 template <int NETS>
-static const void *cta_kernel_for(int mem, int block, bool count, bool hz) {
-    if (count) return cta_kernel_ptr<NETS, 1024, true, true>(mem);   // honours a horizon, if there is one
-    if (block > 512)
-        return hz ? cta_kernel_ptr<NETS, 1024, false, true>(mem) : cta_kernel_ptr<NETS, 1024, false, false>(mem);
-    return hz ? cta_kernel_ptr<NETS, 512, false, true>(mem) : cta_kernel_ptr<NETS, 512, false, false>(mem);
+static const void *cta_kernel_for(int mem, int build, bool count, bool hz) {
+    if (count) return cta_kernel_ptr<NETS, kOne1024, true, true>(mem);   // honours a horizon, if there is one
+    switch (build) {
+    case kThree512:
+        return hz ? cta_kernel_ptr<NETS, kThree512, false, true>(mem) : cta_kernel_ptr<NETS, kThree512, false, false>(mem);
+    case kTwo1024:
+        return hz ? cta_kernel_ptr<NETS, kTwo1024, false, true>(mem) : cta_kernel_ptr<NETS, kTwo1024, false, false>(mem);
+    default:
+        return hz ? cta_kernel_ptr<NETS, kOne1024, false, true>(mem) : cta_kernel_ptr<NETS, kOne1024, false, false>(mem);
+    }
 }
 
-const void *cta_kernel(int nets, int mem, int block, bool count, bool hz) {
-    return nets == 1 ? cta_kernel_for<1>(mem, block, count, hz)
-                     : cta_kernel_for<EAT_MAX_NETS>(mem, block, count, hz);
+const void *cta_kernel(int nets, int mem, int build, bool count, bool hz) {
+    return nets == 1 ? cta_kernel_for<1>(mem, build, count, hz)
+                     : cta_kernel_for<EAT_MAX_NETS>(mem, build, count, hz);
 }
 
 template <int NETS>
@@ -1309,19 +1318,18 @@ static cudaError_t launch_cta_t(const void *kernel, const EdgeDev *nets, int n_n
     return cudaLaunchKernel(kernel, dim3((unsigned)grid), dim3((unsigned)block), args, smem, st);
 }
 
-cudaError_t launch_cta(const EdgeDev *nets, int n_nets, const QueryArgs &qa, int mem, int grid,
+cudaError_t launch_cta(const EdgeDev *nets, int n_nets, const QueryArgs &qa, int mem, int build, int grid,
                        int block, size_t smem, cudaStream_t st) {
-    const void *k = cta_kernel(n_nets == 1 ? 1 : EAT_MAX_NETS, mem, block, qa.counters != nullptr,
-                               qa.horizon > 0);
+    const void *k = cta_kernel(n_nets == 1 ? 1 : EAT_MAX_NETS, mem, build, qa.counters != nullptr, qa.horizon > 0);
     return n_nets == 1 ? launch_cta_t<1>(k, nets, n_nets, qa, grid, block, smem, st)
                        : launch_cta_t<EAT_MAX_NETS>(k, nets, n_nets, qa, grid, block, smem, st);
 }
 
 const void *ring_kernel(int mem) {
     switch (mem) {
-    case 0: return (const void *)eat_cta_kernel<EAT_MAX_NETS, kArrShared, true, 512, true, false, false>;
-    case 3: return (const void *)eat_cta_kernel<EAT_MAX_NETS, kArrPerQuery, true, 512, true, false, false>;
-    default: return (const void *)eat_cta_kernel<EAT_MAX_NETS, kArrGlobal, true, 512, true, false, false>;
+    case 0: return (const void *)eat_cta_kernel<EAT_MAX_NETS, kArrShared, true, kThree512, true, false, false>;
+    case 3: return (const void *)eat_cta_kernel<EAT_MAX_NETS, kArrPerQuery, true, kThree512, true, false, false>;
+    default: return (const void *)eat_cta_kernel<EAT_MAX_NETS, kArrGlobal, true, kThree512, true, false, false>;
     }
 }
 

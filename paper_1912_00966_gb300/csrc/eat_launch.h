@@ -30,6 +30,9 @@ struct RingArgs {
                                  // idle block leaves
 };
 
+// Builds of the round kernel: the block size and blocks per SM that its registers allow.
+enum { kThree512, kOne1024, kTwo1024 };
+
 struct QueryArgs {
     const int32_t *net_idx;    // [n] or nullptr (single network)
     const int32_t *src;        // [n]
@@ -71,10 +74,11 @@ struct QueryArgs {
 // mem: 0 = arrivals and bitmaps in shared memory, 1 = arrivals global / bitmaps
 // shared, 2 = both global, 3 = bitmaps shared and arrivals shared per query when
 // the query's network fits.  nets: 1 or EAT_MAX_NETS (kernel table size).
+// build: kThree512 for blocks of up to 512 threads, kOne1024 or kTwo1024 (per SM) for larger.
 // count: the instantiation that fills qa.counters (launch_cta picks it when counters are
 // given); hz: the one that honours qa.horizon (launch_cta picks it when qa.horizon > 0).
-const void *cta_kernel(int nets, int mem, int block, bool count = false, bool hz = false);
-cudaError_t launch_cta(const EdgeDev *nets, int n_nets, const QueryArgs &qa, int mem, int grid,
+const void *cta_kernel(int nets, int mem, int build, bool count = false, bool hz = false);
+cudaError_t launch_cta(const EdgeDev *nets, int n_nets, const QueryArgs &qa, int mem, int build, int grid,
                        int block, size_t smem, cudaStream_t st);
 // Ring mode of the per-query kernel (serving): persistent blocks take requests from
 // qa.rg until the host's stop flag is set and no request is left, or until they find
