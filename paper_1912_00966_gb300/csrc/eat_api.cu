@@ -832,7 +832,7 @@ static int upload(eat_net *net) {
     size_t off_erow = align_up(off_apx + h.apx.size() * 4 + 16, 256);
     size_t off_er = align_up(off_erow + h.erow.size() * 4, 256);
     size_t off_ee = align_up(off_er + h.er.size() * 4, 256);
-    size_t off_ex = align_up(off_ee + h.ee.size() * 4, 256);
+    size_t off_ex = align_up(off_ee + h.ee_words * 4, 256);
     size_t off_et = align_up(off_ex + h.ex.size() * 4, 256);
     size_t total = align_up(off_et + h.etypes.size() * 4 + 16, 256);
     DeviceGuard guard(net->device);
@@ -852,7 +852,7 @@ static int upload(eat_net *net) {
         {off_apx, h.apx.data(), h.apx.size() * 4},
         {off_erow, h.erow.data(), h.erow.size() * 4},
         {off_er, h.er.data(), h.er.size() * 4},
-        {off_ee, h.ee.data(), h.ee.size() * 4},
+        {off_ee, h.ee.get(), h.ee_words * 4},
         {off_ex, h.ex.data(), h.ex.size() * 4},
         {off_et, h.etypes.data(), h.etypes.size() * 4},
     };
@@ -889,7 +889,8 @@ static int upload(eat_net *net) {
     for (int32_t u = 0; u < h.n_stops; ++u) tails += h.erow[u + 1] > h.erow[u];
     net->branching = tails == 0 ? 0 : 5 * (int64_t)x.n_edges >= 13 * tails ? 2 : x.n_edges >= 2 * tails ? 1 : 0;
     // No host view shows the edge table: its host copy goes.
-    for (std::vector<int32_t> *w : {&h.erow, &h.er, &h.ee, &h.ex, &h.etypes}) std::vector<int32_t>().swap(*w);
+    for (std::vector<int32_t> *w : {&h.erow, &h.er, &h.ex, &h.etypes}) std::vector<int32_t>().swap(*w);
+    h.ee.reset();
     return EAT_OK;
 }
 
