@@ -165,7 +165,8 @@ static constexpr size_t kQueueEntryBytes = 16;  // 8-byte queue entry x 2 buffer
 // 512-thread blocks per SM, horizon one hour 3,556 us against 2,595; 96 queries, one
 // 1,024-thread block 1,452 against 1,103; 60,000 stops, 300 queries 1,177 against 1,007.
 static constexpr size_t kSmemBesideL1 = 196 << 10;
-static constexpr size_t kQueueMost = 1024;      // stops queued in shared memory per buffer
+static constexpr size_t kQueueMost = 1024;      // stops queued in shared memory per buffer (half
+                                                // of it beside shared rows, with fewer stops)
 
 // Default round cap: n_stops + 1 rounds always reach the fixpoint (every productive round
 // fixes one more stop); with a horizon, each move of the horizon can add one round in
@@ -511,8 +512,8 @@ static int make_plan_core(int dev, int32_t vmax, int32_t n, int n_nets, const ea
     const bool wait_shared = p.mem == 0 && p.horizon > 0 && bm + wait_bytes + qbytes * qmin <= limit;
     p.smem_wait_off = wait_shared ? (int32_t)(bm / 4) : 0;
     const size_t b0 = bm + (wait_shared ? wait_bytes : 0);
-    int reg_blocks = 0;
-    {
+    int reg_blocks = 1;                       // with at most one query per SM one is all it holds
+    if (n > d.sms) {
         DeviceGuard guard(dev);
         const void *k = cta_kernel(p.nets, p.mem, p.build, false, p.horizon > 0);
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&reg_blocks, k, p.block, 0) != cudaSuccess) {
@@ -528,16 +529,16 @@ static int make_plan_core(int dev, int32_t vmax, int32_t n, int n_nets, const ea
     const size_t beside = kSmemBesideL1 / (size_t)blocks - 1024;
     const size_t room = b0 + qbytes * qmin <= beside ? beside : std::min(limit, d.smem_per_sm / (size_t)blocks - d.reserve);
     size_t cap = room > b0 ? (room - b0) / qbytes : 0;
-    cap = std::min({cap, (size_t)std::max(vmax, 1), kQueueMost});
+    cap = std::min({cap, (size_t)std::max(vmax, 1), p.mem == 0 ? kQueueMost / 2 : kQueueMost});
     if (cap >= 64) cap &= ~(size_t)31;
     p.qcap = (int32_t)std::max(cap, qmin);
     p.smem_mask_off = p.mem == 0 ? (int32_t)(arr_bytes / 4) : 0;   // mem 3: after the query's own row
     p.smem_q_off = (int32_t)(b0 / 4);
     p.smem = b0 + qbytes * (size_t)p.qcap;
 
-    int per_sm = 0;
-    cudaError_t e;
-    {
+    int per_sm = 1;
+    cudaError_t e = cudaSuccess;
+    if (n != 1) {                             // a single query: a block always fits an SM
         DeviceGuard guard(dev);
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
             &per_sm, cta_kernel(p.nets, p.mem, p.build, false, p.horizon > 0), p.block, p.smem);
@@ -610,6 +611,7 @@ static QueryArgs make_args(const Plan &p, int grid, char *ws, const int32_t *net
     qa.net_idx = net_idx;
     qa.src = src;
     qa.ts = ts;
+    qa.one_src = qa.one_ts = 0;
     qa.arr_off = arr_off;
     qa.arr_out = arr_out;
     qa.spill = (int32_t *)(ws + kWsHeader);
@@ -888,6 +890,12 @@ static int upload(eat_net *net) {
     int64_t tails = 0;
     for (int32_t u = 0; u < h.n_stops; ++u) tails += h.erow[u + 1] > h.erow[u];
     net->branching = tails == 0 ? 0 : 5 * (int64_t)x.n_edges >= 13 * tails ? 2 : x.n_edges >= 2 * tails ? 1 : 0;
+    if (cudaHostAlloc(&net->pin, 128, cudaHostAllocMapped) != cudaSuccess ||
+        cudaHostGetDevicePointer(&net->pin_dev, net->pin, 0) != cudaSuccess) {
+        cudaGetLastError();
+        if (net->pin) cudaFreeHost(net->pin);
+        net->pin = net->pin_dev = nullptr;
+    }
     // No host view shows the edge table: its host copy goes.
     for (std::vector<int32_t> *w : {&h.erow, &h.er, &h.ex, &h.etypes}) std::vector<int32_t>().swap(*w);
     h.ee.reset();
@@ -967,6 +975,7 @@ void eat_free(eat_net *net) {
         if (net->blob) cudaFree(net->blob);
         if (net->ws) cudaFree(net->ws);
         if (net->stage) cudaFree(net->stage);
+        if (net->pin) cudaFreeHost(net->pin);
     }
     delete net;
 }
@@ -1057,7 +1066,12 @@ int eat_query(const eat_net *net, int32_t s, int32_t t_s, int32_t *arr_out,
     if (!net || !arr_out) return fail(EAT_ERR_INVALID, "NULL argument");
     if (net->device < 0) return fail(EAT_ERR_NO_DEVICE, "network was built host-only");
     if (s < 0 || s >= net->host.n_stops) return fail(EAT_ERR_INVALID, "source out of range");
-    if (foreign_ptr(arr_out, net->device)) return foreign_fail();
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, arr_out) != cudaSuccess) {
+        cudaGetLastError();
+        at.type = cudaMemoryTypeUnregistered;
+    }
+    if (at.type == cudaMemoryTypeDevice && at.device != net->device) return foreign_fail();
     std::lock_guard<std::mutex> g(net->ws_lock);
     Plan p;
     int rc = make_plan(net->device, net->host.n_stops, 1, 1, nullptr, p, -1, net);
@@ -1065,8 +1079,40 @@ int eat_query(const eat_net *net, int32_t s, int32_t t_s, int32_t *arr_out,
     DeviceGuard guard(net->device);
     // A page-locked host row is written in place; arrivals that do not fit in shared
     // memory then live in the device row below and are copied over at the end.
-    const bool dev_out = is_device_ptr(arr_out);
-    int32_t *const out_map = dev_out ? nullptr : (int32_t *)mapped_host_ptr(arr_out);
+    const bool dev_out = at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
+    int32_t *const out_map = at.type == cudaMemoryTypeHost ? (int32_t *)at.devicePointer : nullptr;
+    if (net->pin && !p.async && !p.pair && !p.cluster) {
+        // The round kernel takes the query as an argument and leaves status and counters in
+        // mapped host memory: one launch, no copy but that of a pageable row (20,000-stop city
+        // 199 -> 145 us; two copies to the device, two back and a second plan before).
+        const size_t row_bytes = dev_out || (out_map && p.mem == 0) ? 0 : align_up((size_t)net->host.n_stops * 4, 256);
+        rc = ensure_buffer(net->ws, net->ws_bytes, p.ws_bytes + row_bytes);
+        if (rc) return rc;
+        int32_t *const dev_row = (int32_t *)((char *)net->ws + p.ws_bytes);
+        eat_counters *const cnt = (eat_counters *)(net->pin_dev + 16);
+        QueryArgs qa = make_args(p, 1, (char *)net->ws, nullptr, nullptr, nullptr, 1, 1,
+                                 dev_out ? arr_out : out_map ? out_map : dev_row, nullptr,
+                                 default_round_cap(net->host.n_stops, p.horizon), net->pin_dev,
+                                 counters ? cnt : nullptr);
+        qa.one_src = s;
+        qa.one_ts = t_s;
+        const eat_net *nets[1] = {net};
+        qa.prefetch = prefetch_wanted(nets, 1);
+        if (out_map && p.mem != 0) {
+            qa.arr_rows = dev_row;
+            qa.arr_rows_stride = (int64_t)align_up((size_t)p.vmax, 64);
+        }
+        cudaError_t e = launch_cta(&net->edev, 1, qa, p.mem, p.build, 1, p.block, p.smem, 0);
+        if (e == cudaSuccess && !dev_out && !out_map)
+            e = cudaMemcpyAsync(arr_out, dev_row, (size_t)net->host.n_stops * 4, cudaMemcpyDeviceToHost, 0);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(0);
+        if (e != cudaSuccess) return cuda_fail(e, "eat_query");
+        if (counters) std::memcpy(counters, net->pin + 16, sizeof(eat_counters));
+        const int32_t st = net->pin[0];
+        return st == EAT_ERR_NO_CONVERGENCE ? fail(st, "round cap reached")
+               : st                         ? fail(st, "query failed")
+                                            : EAT_OK;
+    }
     const size_t rows = dev_out ? 0 : align_up((size_t)net->host.n_stops * 4, 256);
     rc = ensure_buffer(net->ws, net->ws_bytes, p.ws_bytes + rows + 256);
     if (rc) return rc;

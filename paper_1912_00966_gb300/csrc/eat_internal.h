@@ -172,6 +172,9 @@ struct eat_net {
     mutable size_t ws_bytes = 0;
     mutable void *stage = nullptr;
     mutable size_t stage_bytes = 0;
+    // Mapped host memory for a single query's status and counters, and its device address
+    // (nullptr if it could not be had).
+    int32_t *pin = nullptr, *pin_dev = nullptr;
     // Launch shape chosen by eat_autotune per batch-size class (log2 of n), packed as
     // block | vwarp << 16 | mode << 24 | horizon << 32 (0 = none) so that a query call
     // on another thread reads one whole shape.

@@ -259,8 +259,8 @@ eat_cta_kernel(const __grid_constant__ EdgeTable<NETS> nets, const QueryArgs qa)
             s_min[tid] = kInf;
             s_rel[tid] = 0;
         }
-        const int32_t s = RING ? s_ring[1] : __ldg(qa.src + q);
-        const int32_t t_s = RING ? s_ring[2] : __ldg(qa.ts + q);
+        const int32_t s = RING ? s_ring[1] : qa.src ? __ldg(qa.src + q) : qa.one_src;
+        const int32_t t_s = RING ? s_ring[2] : qa.src ? __ldg(qa.ts + q) : qa.one_ts;
         const bool valid = net_ok && (unsigned)s < (unsigned)V;
         __syncthreads();
         // The source is the frontier of "round -1": buffer 1.

@@ -35,8 +35,9 @@ enum { kThree512, kOne1024, kTwo1024 };
 
 struct QueryArgs {
     const int32_t *net_idx;    // [n] or nullptr (single network)
-    const int32_t *src;        // [n]
+    const int32_t *src;        // [n], or nullptr: the one query (one_src, one_ts) (round kernel)
     const int32_t *ts;         // [n]
+    int32_t one_src, one_ts;
     const int64_t *arr_off;    // [n] or nullptr (row q at q * n_stops)
     int32_t *arr_out;
     int32_t *spill;            // [slots][spill_stride]: spilled frontier stops (2 x vmax)

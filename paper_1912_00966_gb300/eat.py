@@ -327,8 +327,9 @@ def eat_query(net: Net, s: int, t_s: int, out=None, counters: bool = False):
     numpy when None).  Returns out, or (out, counters dict) if counters=True."""
     if out is None:
         out = np.empty(eat_get_stats(net)["n_stops"], dtype=np.int32)
-    c = eat_counters()
-    _check(_lib.eat_query(net.handle, int(s), int(t_s), _ptr(out), ctypes.byref(c)), "eat_query")
+    c = eat_counters() if counters else None
+    _check(_lib.eat_query(net.handle, int(s), int(t_s), _ptr(out),
+                          ctypes.byref(c) if counters else None), "eat_query")
     if counters:
         return out, {f: getattr(c, f) for f in COUNTER_FIELDS}
     return out
