@@ -724,14 +724,15 @@ int build_edges(HostNet &h) {
         // Half of that where the table does not stay in L2 anyway (200,000 stops, 96 queries
         // 1,030 -> 980 us, 1,024 queries 2,382 -> 2,336; but 256 queries of the 20,000-stop
         // city, whose 72 MB stay there, 277 -> 305).  Wider only to keep the table within
-        // 2 GB, or within the cluster table's size where that is larger.
+        // 2 GB, or within the cluster table's size (up to 16 GB) where that is larger: a
+        // network whose cluster table fills most of the device still fits beside it.
         const int64_t span = (int64_t)last - first + 1;
         const double headway = (double)span * (double)E / (double)n_pairs;
         auto slots = [&](int32_t s) { return ((int64_t)last - first) / ((int64_t)1 << s) + 1; };
         int32_t s = 3;
         while (s < 15 && (double)((int64_t)2 << s) <= headway) ++s;
         if (s > 3 && E * slots(s) * 16 > ((int64_t)96 << 20)) --s;
-        const int64_t most = std::max((int64_t)2 << 30, (int64_t)h.n_types * h.y * 32);
+        const int64_t most = std::max((int64_t)2 << 30, std::min((int64_t)16 << 30, (int64_t)h.n_types * h.y * 32));
         while (s < 15 && E * slots(s) * 16 > most) ++s;
         h.e_shift = s;
         h.e_y = (int32_t)slots(s);
