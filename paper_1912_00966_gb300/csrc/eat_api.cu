@@ -134,7 +134,8 @@ struct Plan {
     int grid = 0;
     size_t smem = 0;              // dynamic shared memory bytes
     int32_t vmax = 0;
-    int32_t qcap = 0;             // shared-memory (stop, type) items per buffer
+    int32_t qcap = 0;             // shared-memory queue entries per buffer (stops; paired and
+                                  // cluster mode: (stop, type) items)
     int32_t mask_words = 0;       // words per bitmap
     int32_t smem_mask_off = 0;    // int offsets into dynamic shared memory
     int32_t smem_q_off = 0;
@@ -148,7 +149,7 @@ struct Plan {
     bool async = false;           // round-free kernel (EAT_MODE_ASYNC)
     int cluster = 0;              // blocks per query in cluster mode (EAT_MODE_CLUSTER), else 0
     bool pair = false;            // two queries per block (EAT_MODE_PAIR)
-    bool edge = false;            // warp min per head stop, degree-chosen mapping (EAT_MODE_EDGE)
+    bool edge = false;            // EAT_MODE_EDGE asked for or tuned: reported; the round kernel runs
     bool order = false;           // queries start by t_s (EAT_ORDER_BY_TIME): order array at off_order
     size_t off_order = 0;
     int32_t horizon = 0;          // seconds (eat_query_opts.horizon resolved), 0 = none
@@ -587,9 +588,10 @@ static int make_plan(int dev, int32_t vmax, int32_t n, int n_nets, const eat_que
 }
 
 // Whether the round kernel prefetches: the edge tables of a launch's networks together do not
-// stay in L2.  (Large network, 1.1 GB, 96 queries 1,526 -> 1,426 us; 60,000 stops, 218 MB, 300
-// queries 1,210 -> 1,164; 64 ragged networks, 700 MB, 1,700 -> 1,538; but the city's 62 MB
-// stay in L2, and its 256 queries took 302 us with the prefetches against 287.)
+// stay in L2.  (Slots of a whole headway: large network, 1.1 GB, 96 queries 1,526 -> 1,426
+// us; 60,000 stops, 218 MB, 300 queries 1,210 -> 1,164; 64 ragged networks, 700 MB, 1,700 ->
+// 1,538; but the city's 62 MB stay in L2, and its 256 queries took 302 us with the
+// prefetches against 287.)
 static constexpr int64_t kPrefetchBytes = (int64_t)96 << 20;
 
 static int32_t prefetch_wanted(const eat_net *const *nets, int n_nets) {

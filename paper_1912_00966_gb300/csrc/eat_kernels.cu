@@ -4,17 +4,18 @@
 //   init     e[] = INF, e[s] = t_s, frontier = {s}                 (Algorithm 2)
 //   round    for every stop u of the frontier and every connection type
 //            (u, v, lambda) leaving u: find the first departure t_c >= e[u]
-//            (the APs of e[u]'s cluster, else the next non-empty cluster;
-//            Algorithm 6), and if t_c + lambda < e[v] lower e[v] with atomicMin
-//            and put v on the next frontier                        (Algorithm 3)
+//            (Algorithm 6; the round kernel reads it from the edge's slot, the
+//            paired, round-free and cluster kernels from the type's cluster), and
+//            if t_c + lambda < e[v] lower e[v] with atomicMin and put v on the
+//            next frontier                                         (Algorithm 3)
 //   stop     when a round puts nobody on the next frontier.
 // The frontier replaces the paper's active[]/nextactive[] flags (Section III-B):
 // a stop joins the next frontier only after its e[] was lowered, through a
 // test-and-set on a per-round bitmap, so each stop appears at most once per
 // round; atomicMin resolves concurrent lowerings (Section III-C).
 //
-// CTA mode: one thread block owns one query at a time (persistent blocks take
-// queries from an atomic counter), so rounds are separated by one block barrier
+// CTA mode: one thread block owns one query at a time (the block's own index
+// first, then queries from an atomic counter), so rounds are separated by one block barrier
 // and there is no grid-wide synchronisation and no spin-wait.  The round-free
 // mode (eat_async_kernel) and the cluster mode (eat_cluster_kernel) are
 // described at their kernels below.
@@ -169,9 +170,9 @@ __device__ __forceinline__ void fill_inf(int32_t *p, int32_t n, int tid, int nth
 // of a test for the last one, spilled stops in a loop of their own), counters that are never
 // reset, two barriers only where the horizon moves.  us per step, against one thread per
 // (stop, connection type) item with 32-byte cluster entries and no room for L1: grid 256
-// queries 117 -> 58, city 37 queries 690 -> 233, 256 queries 527 -> 305, 60,000 stops 300
-// queries 3,753 -> 954, large 96 queries 4,296 -> 1,041, 1,024 queries 6,325 -> 2,453, 64
-// ragged networks 4,096 queries 1,959 -> 868.
+// queries 117 -> 58, city 37 queries 690 -> 229, 256 queries 530 -> 292, 60,000 stops 300
+// queries 3,760 -> 880, large 96 queries 4,340 -> 935, 1,024 queries 6,430 -> 2,338, 64
+// ragged networks 4,096 queries 1,970 -> 826.
 // BUILD: registers by how many blocks an SM is to hold (large network: 1,024 queries in
 // 512-thread blocks 2,400 us at 40 registers, three per SM, against 2,525 at 32; 96 queries in
 // 1,024-thread blocks 1,039 at 56 against 1,113 at 32; 60,000 stops, 300 queries, two

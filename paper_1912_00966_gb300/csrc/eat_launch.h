@@ -42,7 +42,7 @@ struct QueryArgs {
     int32_t *arr_out;
     int32_t *spill;            // [slots][spill_stride]: spilled frontier stops (2 x vmax)
     uint32_t *gmask;           // [slots][mask_stride]: both bitmaps when not in shared memory
-    int32_t *work;             // query counter (zeroed before launch)
+    int32_t *work;             // query counter (zeroed before a launch that reads it)
     int32_t *status;           // [n] or nullptr
     eat_counters *counters;    // [n] or nullptr
     int64_t spill_stride;      // ints per slot (>= 2 * vmax)
@@ -56,7 +56,7 @@ struct QueryArgs {
                                // and cluster mode: (stop, type) items)
     int32_t mask_words;        // words per bitmap (padded)
     int32_t smem_mask_off;     // int offset of the bitmaps in dynamic shared memory
-    int32_t smem_q_off;        // int offset of the item buffers in dynamic shared memory
+    int32_t smem_q_off;        // int offset of the queues in dynamic shared memory
     int32_t smem_wait_off;     // int offset of the waiting stops' bitmap, 0 = after the spilled stops
     int32_t smem_arr_cap;      // per-query placement: arrivals shared when n_stops <= this
     int32_t *arr_rows;         // [grid][arr_rows_stride]: a block's arrivals when they are not
