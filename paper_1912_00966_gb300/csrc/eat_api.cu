@@ -160,6 +160,7 @@ struct Plan {
 static constexpr size_t kWsHeader = 256;   // work counter + internal status / counters
 static constexpr int32_t kDefaultIdleCap = 1 << 24;   // round-free mode's wait limit (full scans)
 static constexpr size_t kQueueEntryBytes = 16;  // 8-byte queue entry x 2 buffers
+static constexpr size_t kQueueArrivalBytes = 8; // 4-byte arrival x 2 buffers (leaves_back_out)
 // Shared memory that an SM's blocks take together where that can be had: the 196 KB step of
 // the SM's division leaves 60 KB of the 256 to L1, in which every load in flight holds a
 // line.  A queue that took all there was left L1 28 KB: large network, 1,024 queries, three
@@ -498,7 +499,9 @@ static int make_plan_core(int dev, int32_t vmax, int32_t n, int n_nets, const ea
     if (!(o && o->block) && !tb && p.mem == 0)
         p.active = std::min(p.block, vmax < 2048 ? 128 : vmax < 6144 ? 256 : vmax <= 32768 ? 512 : 1024);
     p.build = p.block <= 512 ? kThree512 : n <= d.sms ? kOne1024 : kTwo1024;
-    const size_t qbytes = kQueueEntryBytes;
+    const bool back = leaves_back_out(p.mem, p.build);
+    const size_t qbytes = kQueueEntryBytes + (back ? kQueueArrivalBytes : 0), qpad = back ? 8 : 0;
+    const size_t qleast = back ? std::min<size_t>(qmin, 168) : qmin;   // in the room of qmin records alone
     // As many blocks per SM as the threads and the registers allow and, with rows in global
     // memory, as leave L1 its share with a queue of 512 stops each (200,000 stops, 1,024
     // queries: three 512-thread blocks 2,400 us, four, which leave L1 28 KB, 3,500; with rows
@@ -528,14 +531,14 @@ static int make_plan_core(int dev, int32_t vmax, int32_t n, int n_nets, const ea
     int blocks = max_blocks;
     while (blocks > 1 && (size_t)blocks * (b0 + qplenty) > most) --blocks;
     const size_t beside = kSmemBesideL1 / (size_t)blocks - 1024;
-    const size_t room = b0 + qbytes * qmin <= beside ? beside : std::min(limit, d.smem_per_sm / (size_t)blocks - d.reserve);
-    size_t cap = room > b0 ? (room - b0) / qbytes : 0;
+    const size_t room = b0 + qbytes * qleast + qpad <= beside ? beside : std::min(limit, d.smem_per_sm / (size_t)blocks - d.reserve);
+    size_t cap = room > b0 + qpad ? (room - b0 - qpad) / qbytes : 0;
     cap = std::min({cap, (size_t)std::max(vmax, 1), p.mem == 0 ? kQueueMost / 2 : kQueueMost});
     if (cap >= 64) cap &= ~(size_t)31;
-    p.qcap = (int32_t)std::max(cap, qmin);
+    p.qcap = (int32_t)std::max(cap, qleast);
     p.smem_mask_off = p.mem == 0 ? (int32_t)(arr_bytes / 4) : 0;   // mem 3: after the query's own row
     p.smem_q_off = (int32_t)(b0 / 4);
-    p.smem = b0 + qbytes * (size_t)p.qcap;
+    p.smem = b0 + qbytes * (size_t)p.qcap + qpad;   // an odd number of arrivals is rounded up
 
     int per_sm = 1;
     cudaError_t e = cudaSuccess;
@@ -640,6 +643,7 @@ static QueryArgs make_args(const Plan &p, int grid, char *ws, const int32_t *net
     qa.idle_cap = kDefaultIdleCap;
     qa.rg = RingArgs{};
     qa.horizon = p.horizon;
+    qa.back = leaves_back_out(p.mem, p.build);
     qa.active = p.active ? p.active : p.block;
     qa.prefetch = 0;
     return qa;

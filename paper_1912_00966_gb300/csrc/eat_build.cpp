@@ -737,10 +737,12 @@ int build_edges(HostNet &h) {
         h.e_shift = s;
         h.e_y = (int32_t)slots(s);
     }
+    std::vector<int32_t> heads;
     try {
         h.erow.assign((size_t)V + 1, 0);
         h.er.assign((size_t)E * 2, 0);
         h.etypes.assign((size_t)E, 0);
+        heads.reserve((size_t)E);
         // and one slot without departures, for tails reached after the last slot
         h.ee_words = (size_t)E * ((size_t)h.e_y + 1) * 4;
         h.ee.reset(new int32_t[h.ee_words]);
@@ -755,15 +757,20 @@ int build_edges(HostNet &h) {
                 r += p.per_u[i];
             }
         h.erow[V] = r;
+        for (const Part &p : parts) heads.insert(heads.end(), p.head.begin(), p.head.end());
     }
     // Entries, with list offsets local to the part; the lists' places follow from their sizes.
     const bool big = V > kMaxPackedStops;
     auto fill = [&](Part &p) {
         const int64_t e0 = e_off[&p - parts.data()];
+        int32_t u = p.u_begin;
         for (size_t e = 0; e < p.head.size(); ++e) {
-            const int32_t v = p.head[e], d = std::min(h.erow[v + 1] - h.erow[v], kCountOverflow);
+            const int32_t v = p.head[e], d = std::min(h.erow[v + 1] - h.erow[v], kEdgeOverflow);
+            while (e0 + (int64_t)e >= h.erow[u + 1]) ++u;
+            const int32_t *const hv = heads.data() + h.erow[v];
+            const int32_t b = (int32_t)(std::find(hv, hv + d, u) - hv);
             int32_t *r = &h.er[2 * (size_t)(e0 + (int64_t)e)];
-            r[0] = big ? v : (int32_t)((uint32_t)v | (uint32_t)d << 24);
+            r[0] = big ? v : (int32_t)((uint32_t)v | (uint32_t)(b < d ? b : kEdgeOverflow) << 24 | (uint32_t)d << 28);
             r[1] = h.erow[v];
             h.etypes[(size_t)(e0 + (int64_t)e)] = p.types[e];
             const Pair *q = p.pairs.data() + p.ptr[e], *const end = p.pairs.data() + p.ptr[e + 1];

@@ -52,8 +52,9 @@ constexpr int32_t kInlineAps = 4;
 // one dominates (departs no earlier, arrives no later): the earliest arrival over the edge
 // for a tail reached at e is then the arrival of the first listed departure >= e, one
 // relaxation for the edge instead of one per connection type (Section II-E).
-//   er[i]        8-byte record of edge i: {v | d << 24, erow[v]}: head stop, edges leaving
-//                it (255 = read erow), its first edge; networks of more than 2^24 stops:
+//   er[i]        8-byte record of edge i = (u, v): {v | b << 24 | d << 28, erow[v]}: head stop,
+//                edges leaving it (15 = read erow), which of them goes back to u (15 = none
+//                of the first 15), its first edge; networks of more than 2^24 stops:
 //                {v, erow[v]}, d always read from erow
 //   ee[k*E + i]  16-byte entry of edge i for slot k, slot-major (a round's lookups are at
 //                nearby times and fall in few slabs): the listed departures inside the slot
@@ -69,6 +70,7 @@ constexpr int32_t kInlineAps = 4;
 // departure left: a large query of a 1,024-query step looks up 65,000 edges instead of
 // 194,000 types, and the table takes 2.0 GB instead of 5.1 GB.
 constexpr int32_t kNoDeparture = 0xffff;
+constexpr int32_t kEdgeOverflow = 15;
 constexpr int32_t kMaxPackedStops = 1 << 24;
 
 struct EdgeDev {

@@ -24,7 +24,8 @@
 // eat_internal.h): all connection types of an edge (u, v) are merged, per time slot, into one
 // 16-byte entry, so that an edge is one lookup and one relaxation (Section II-E).  The
 // frontier is a queue of stops in shared memory: the thread that lowers e[v] stores
-// {v, degree, first edge} (8 bytes, taken from the edge's record), and the next round
+// {v, degree, first edge} (8 bytes, taken from the edge's record; with rows in global memory
+// and several blocks per SM also the arrival it was queued with), and the next round
 // gives each queued stop a sub-warp (Section II-F's virtual warps) whose lanes take its
 // edges.  Per lane: the queue entry and e[u] (the same for the sub-warp), the edge's 8-byte
 // record, then the 16-byte entry of e[u]'s slot beside e[v].  Queue entries past the shared
@@ -171,7 +172,7 @@ __device__ __forceinline__ void fill_inf(int32_t *p, int32_t n, int tid, int nth
 // reset, two barriers only where the horizon moves.  us per step, against one thread per
 // (stop, connection type) item with 32-byte cluster entries and no room for L1: grid 256
 // queries 117 -> 58, city 37 queries 690 -> 229, 256 queries 530 -> 292, 60,000 stops 300
-// queries 3,760 -> 880, large 96 queries 4,340 -> 935, 1,024 queries 6,430 -> 2,338, 64
+// queries 3,760 -> 808, large 96 queries 4,340 -> 932, 1,024 queries 6,430 -> 2,280, 64
 // ragged networks 4,096 queries 1,970 -> 826.
 // BUILD: registers by how many blocks an SM is to hold (large network: 1,024 queries in
 // 512-thread blocks 2,400 us at 40 registers, three per SM, against 2,525 at 32; 96 queries in
@@ -199,6 +200,15 @@ eat_cta_kernel(const __grid_constant__ EdgeTable<NETS> nets, const QueryArgs qa)
 
     // Stop queues and spilled stops; round r writes buffer r & 1.
     int2 *const queue = reinterpret_cast<int2 *>(smem + qa.smem_q_off);
+    // Whether a stop's edge back to the stop that queued it is left out (see expand): a queue
+    // entry then also has the arrival it was queued with, the arrivals after the records.
+    constexpr bool kBack = ARR == kArrGlobal && SMEM_MASK && !RING && (COUNT || BUILD != kOne1024);
+    const bool back_out = kBack && (!COUNT || qa.back);
+    const int32_t qlen = back_out ? qcap + ((qcap + 1) >> 1) : qcap;
+    auto from = [&](int2 *q) { return reinterpret_cast<int32_t *>(q + qcap); };
+    auto queued = [](int32_t v, int32_t d) {          // no edge known to lead back
+        return (int32_t)((uint32_t)v | (uint32_t)kEdgeOverflow << 24 | (uint32_t)d << 28);
+    };
     int32_t *const spill_base = qa.spill + (int64_t)blockIdx.x * qa.spill_stride;
     uint32_t *const mask_base = SMEM_MASK ? (uint32_t *)(smem + qa.smem_mask_off)
                                           : qa.gmask + (int64_t)blockIdx.x * qa.mask_stride;
@@ -268,8 +278,9 @@ eat_cta_kernel(const __grid_constant__ EdgeTable<NETS> nets, const QueryArgs qa)
         if (tid == 0 && valid) {
             arr[s] = t_s;
             const int32_t row = __ldg(N.erow + s);
-            const int32_t d = min(__ldg(N.erow + s + 1) - row, kCountOverflow);
-            queue[qcap] = make_int2(big ? s : (int32_t)((uint32_t)s | (uint32_t)d << 24), row);
+            const int32_t d = min(__ldg(N.erow + s + 1) - row, kEdgeOverflow);
+            queue[qlen] = make_int2(big ? s : queued(s, d), row);
+            if (back_out) from(queue + qlen)[0] = t_s;
         }
         __syncthreads();
 
@@ -281,7 +292,7 @@ eat_cta_kernel(const __grid_constant__ EdgeTable<NETS> nets, const QueryArgs qa)
         int wl = 0;                                       // counters that new waiting stops use
         int32_t seen_wr = 0, seen_rd = 0;                 // s_n of either parity before the round
         int32_t c_vert = 0, c_types = 0, c_evals = 0, c_lookups = 0, c_aps = 0, c_relax = 0;
-        int2 *q_rd = queue + qcap, *q_wr = queue;         // stops queued last round, this round
+        int2 *q_rd = queue + qlen, *q_wr = queue;         // stops queued last round, this round
         int32_t *sp_rd = spill_base + qa.vmax, *sp_wr = spill_base;
         uint32_t *cmask = mask1, *pmask = mask0;
         int32_t *n_rd = s_n + 1, *n_wr = s_n;
@@ -306,7 +317,7 @@ eat_cta_kernel(const __grid_constant__ EdgeTable<NETS> nets, const QueryArgs qa)
                 if (cand >= ev) return;
                 ++c_relax;
                 atomicMin(arr + v, cand);
-                const bool leaf = big ? __ldg(N.erow + v + 1) == h.y : (uint32_t)h.x < 1u << 24;
+                const bool leaf = big ? __ldg(N.erow + v + 1) == h.y : (uint32_t)h.x < 1u << 28;
                 const uint32_t bit = 1u << (v & 31);
                 if (HZ && cand >= H) {
                     if (leaf) return;
@@ -322,18 +333,29 @@ eat_cta_kernel(const __grid_constant__ EdgeTable<NETS> nets, const QueryArgs qa)
                     int32_t start;
                     const uint32_t k = min(edge_slot(N.base, N.shift, cand, rel, start), (uint32_t)N.y);
                     const int4 *const p = N.ee + (uint64_t)k * (uint32_t)N.n_edges + h.y;
-                    const uint32_t d = (uint32_t)h.x >> 24;
+                    const uint32_t d = (uint32_t)h.x >> 28;
                     asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
                     if (d > 1) asm volatile("prefetch.global.L2 [%0];" ::"l"(p + (d - 1)));
                 }
-                if (__builtin_expect(pos < qcap, 1)) q_wr[pos] = h;
-                else sp_wr[pos - qcap] = v;
+                if (__builtin_expect(pos < qcap, 1)) {
+                    q_wr[pos] = h;
+                    if (back_out) from(q_wr)[pos] = cand;
+                } else {
+                    sp_wr[pos - qcap] = v;
+                }
             };
-            // Stop u's edges t, t + P, ... of its d by the lanes of a sub-warp.
-            auto expand = [&](int32_t u, int32_t t, int32_t d, int P, int lane) {
+            // Stop u's edges t, t + P, ... of its d by the lanes of a sub-warp.  Its edge b leads
+            // back to the stop whose candidate `arrived` queued u: while e[u] is that candidate
+            // it cannot lower that stop's arrival, which is below it, and is left out where
+            // lookups of rows and entries in L2 and memory are what several blocks per SM
+            // share (60,000 stops, 300 queries 877 -> 809 us, 200,000 stops, 1,024 queries
+            // 2,340 -> 2,300).  Where a round is a chain of loads alone, the arrival's store and
+            // test only lengthen it (one block per SM, 96 large queries 927 -> 971; rows in
+            // shared memory 826 -> 855 for 64 ragged networks).
+            auto expand = [&](int32_t u, int32_t t, int32_t d, int P, int lane, int32_t arrived, int32_t b) {
                 const int32_t e_u = load_arr(arr, u, arr_shared);
                 cmask[u >> 5] = 0u;                         // every stop of the word is in this queue
-                if (d == kCountOverflow) d = __ldg(N.erow + u + 1) - t;
+                if (d == kEdgeOverflow) d = __ldg(N.erow + u + 1) - t;
                 uint32_t rel;
                 int32_t start;
                 // slot y holds no departures
@@ -341,9 +363,11 @@ eat_cta_kernel(const __grid_constant__ EdgeTable<NETS> nets, const QueryArgs qa)
                 const int4 *const slab = N.ee + (uint64_t)k * (uint32_t)N.n_edges;
                 if (COUNT) c_vert += lane == 0;
                 const int32_t end = t + d;
+                const int32_t back = back_out && e_u == arrived && b != kEdgeOverflow ? t + b : -1;
 #pragma unroll 1
                 for (t += lane; t < end; t += P) {
                     const int2 h = __ldg(N.er + t);
+                    if (back_out && t == back) continue;
                     const int4 c = load_slot<ARR == kArrShared>(slab + t);
                     const int32_t v = big ? h.x : h.x & 0xffffff;
                     const int32_t ev = load_arr(arr, v, arr_shared);
@@ -368,14 +392,14 @@ eat_cta_kernel(const __grid_constant__ EdgeTable<NETS> nets, const QueryArgs qa)
 #pragma unroll 1
             for (int32_t i = tid >> pl; i < nq; i += nsub) {
                 const int2 e = q_rd[i];
-                expand(big ? e.x : e.x & 0xffffff, e.y, big ? kCountOverflow : (int32_t)((uint32_t)e.x >> 24),
-                       1 << pl, lane);
+                expand(big ? e.x : e.x & 0xffffff, e.y, big ? kEdgeOverflow : (int32_t)((uint32_t)e.x >> 28),
+                       1 << pl, lane, back_out ? from(q_rd)[i] : 0, big ? kEdgeOverflow : (int32_t)((uint32_t)e.x >> 24 & 15u));
             }
             if (n > qcap) {                                 // spilled stops
 #pragma unroll 1
                 for (int32_t i = tid >> 3; i < n - qcap; i += nthr >> 3) {
                     const int32_t u = __ldcg(sp_rd + i);
-                    expand(u, __ldg(N.erow + u), kCountOverflow, 8, tid & 7);
+                    expand(u, __ldg(N.erow + u), kEdgeOverflow, 8, tid & 7, 0, kEdgeOverflow);
                 }
             }
             __syncthreads();
@@ -411,9 +435,8 @@ eat_cta_kernel(const __grid_constant__ EdgeTable<NETS> nets, const QueryArgs qa)
                             const int32_t pos = atomicAdd(&s_rel[wl], 1);
                             if (pos < qcap) {
                                 const int32_t row = __ldg(N.erow + v[j]);
-                                const int32_t d = min(__ldg(N.erow + v[j] + 1) - row, kCountOverflow);
-                                q_wr[pos] = make_int2(
-                                    big ? v[j] : (int32_t)((uint32_t)v[j] | (uint32_t)d << 24), row);
+                                const int32_t d = min(__ldg(N.erow + v[j] + 1) - row, kEdgeOverflow);
+                                q_wr[pos] = make_int2(big ? v[j] : queued(v[j], d), row);
                             } else {
                                 sp_wr[pos - qcap] = v[j];
                             }

@@ -33,6 +33,10 @@ struct RingArgs {
 // Builds of the round kernel: the block size and blocks per SM that its registers allow.
 enum { kThree512, kOne1024, kTwo1024 };
 
+// Whether the round kernel leaves out a stop's edge back to the stop that queued it, and so
+// keeps an arrival with each queued stop: rows in global memory, several blocks per SM.
+inline bool leaves_back_out(int mem, int build) { return mem == 1 && build != kOne1024; }
+
 struct QueryArgs {
     const int32_t *net_idx;    // [n] or nullptr (single network)
     const int32_t *src;        // [n], or nullptr: the one query (one_src, one_ts) (round kernel)
@@ -66,6 +70,7 @@ struct QueryArgs {
     int32_t idle_cap;          // round-free mode: empty 32-word bitmap scans in a row per warp
     RingArgs rg;               // ring mode only
     int32_t prefetch;          // round kernel: a queued stop's entries are prefetched into L2
+    int32_t back;              // round kernel: queue entries of 12 bytes (leaves_back_out)
     int32_t active;            // round kernel: threads of a block that work (a multiple of 32)
     int32_t horizon;           // seconds, 0 = none: stops lowered to an arrival at or after
                                // the horizon wait (per-query kernel); with one,

@@ -70,8 +70,13 @@ int main(int argc, char **argv) {
         for (int32_t i = h.erow[s]; i < h.erow[s + 1]; ++i) {
             const uint32_t x = (uint32_t)h.er[2 * (size_t)i];
             const int32_t head = (int32_t)(x & 0xffffffu);
-            const int32_t deg = std::min(h.erow[head + 1] - h.erow[head], kCountOverflow);
-            if ((int32_t)(x >> 24) != deg || h.er[2 * (size_t)i + 1] != h.erow[head]) return 1;
+            const int32_t deg = std::min(h.erow[head + 1] - h.erow[head], kEdgeOverflow);
+            if ((int32_t)(x >> 28) != deg || h.er[2 * (size_t)i + 1] != h.erow[head]) return 1;
+            // the head's edge back to s, where it is one of its first 15
+            int32_t back = kEdgeOverflow;
+            for (int32_t j = h.erow[head]; j < h.erow[head] + deg; ++j)
+                if ((h.er[2 * (size_t)j] & 0xffffff) == s) back = j - h.erow[head];
+            if ((int32_t)(x >> 24 & 15) != back) return 1;
             const auto &conns = edges.at({s, head});
             std::vector<int64_t> times = {INT32_MIN, t0 - 1, t0 + t_max + 1, INT32_MAX - 1, INT32_MAX};
             for (const auto &q : conns)

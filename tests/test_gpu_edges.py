@@ -98,3 +98,28 @@ def test_automatic_shapes(family, stops):
             eat.eat_query_batch(net, src[:n], ts[:n], out[:n], **more)
             assert torch.equal(out[:n], want[:n]), (n, list(more))
     net.close()
+
+
+@pytest.mark.parametrize("stops,degree", [(5, 3), (167, 14), (169, 15), (1001, 16), (20001, 4)])
+def test_edges_back(stops, degree):
+    """Edges in both directions between most pairs (of which rows in global memory leave the one
+    back to the stop that queued a stop out), stops of 14 to 16 edges about, odd queue sizes."""
+    from paper_1912_00966_gb300 import eat
+    rng = np.random.default_rng(stops)
+    a = np.tile(np.arange(stops), degree // 2 + 1)
+    b = rng.integers(0, stops, a.shape[0])
+    u, v = np.tile(np.concatenate([a, b]), 6), np.tile(np.concatenate([b, a]), 6)
+    tt = _timetable(stops, u, v, rng.integers(0, 20000, u.shape[0]), rng.integers(1, 900, u.shape[0]))
+    net = eat.eat_build(tt.n_stops, tt.u, tt.v, tt.dep, tt.dur, device=0)
+    n = torch.cuda.get_device_properties(0).multi_processor_count + 9
+    src, ts = rng.integers(0, stops, n).astype(np.int32), rng.integers(0, 9000, n).astype(np.int32)
+    want, _ = oracle.csa_many(oracle.SortedConnections(tt), src, ts, 8)
+    out = torch.empty((n, stops), dtype=torch.int32, device="cuda")
+    counters = torch.zeros((n, 7), dtype=torch.int64, device="cuda")
+    src, ts = torch.as_tensor(src).cuda(), torch.as_tensor(ts).cuda()
+    for opts in ({"block": 512}, {"block": 1024}, {"block": 64, "vwarp": 2}, {"block": 512, "horizon": 700},
+                 {"block": 1024, "horizon": 700, "counters": counters}):
+        out.fill_(-7)
+        eat.eat_query_batch(net, src, ts, out, placement=eat.EAT_PLACE_GLOBAL_ARR, **opts)
+        assert np.array_equal(out.cpu().numpy(), want), list(opts)
+    net.close()
