@@ -2,7 +2,7 @@
 
 Workload (default "large"): a 200,000-stop random geometric transit network (k = 5
 nearest neighbours, 4,000 routes of 40-80 stops run both ways, headways 3-30 min,
-10 % jittered trips, three duration bands), about 46 M connections, 1.8 GB on the
+10 % jittered trips, three duration bands), about 46 M connections, 7.1 GB on the
 device; one step = one batch of 1,024 queries (random source with departures, t_s
 uniform in 05:00-22:00), all relaxation rounds of all queries in one launch (the
 launch shape by the library's autotuner unless given; the batch's queries cannot
@@ -61,8 +61,8 @@ BYTES = {"vertices": 12, "lookups": 28, "relaxed": 12}
 # cluster width, so that another kernel or launch shape reports null until it is
 # profiled again.
 NCU_TRAFFIC_PER_QUERY = {
-    "large": ("2de258fb4eb0b1dc", "eat_cta_kernel", 512, 3600, 600, 14555841037 / 1024),
-    "city": ("2de258fb4eb0b1dc", "eat_cta_kernel", 1024, -1, 600, 135806746 / 256),
+    "large": ("b5fafcd224b20f19", "eat_cta_kernel", 512, 7200, 600, 8606264768 / 1024),
+    "city": ("b5fafcd224b20f19", "eat_cta_kernel", 512, 14400, 600, 49174323 / 256),
 }
 KERNEL_OF_MODE = {1: "eat_cta_kernel", 2: "eat_cluster_kernel", 3: "eat_async_kernel",
                   4: "eat_pair_kernel", 5: "eat_cta_kernel"}
