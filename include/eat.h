@@ -156,7 +156,9 @@ typedef struct {
     int64_t evals;     /* of the lookups, those that found a departure at or after e[u] */
     int64_t lookups;   /* table entries read for the examined types: one per edge in the
                           round-based modes (EAT_MODE_CTA, EAT_MODE_EDGE), one per type
-                          (Section II-D) in the others; types >= lookups >= evals */
+                          (Section II-D) in the others; types >= lookups >= evals.
+                          An edge back to the stop an arrival came from may be left
+                          out (it cannot lower that stop), with its types */
     int64_t aps;       /* departures (round-based modes) or AP records (Algorithm 6)
                           examined by the lookups */
     int64_t relaxed;   /* relaxations that lowered e[v] (Algorithm 3): candidates below
