@@ -340,9 +340,21 @@ static int log2_class(int32_t n) {
     return c;
 }
 
-static int make_plan_core(int dev, int32_t vmax, int32_t n, int n_nets, const eat_query_opts *o,
-                          Plan &p, int32_t vmin, const eat_net *tuned, bool own_workspace, bool use_tuned) {
-    if (vmin < 0) vmin = vmax;
+// What a plan is for: a batch, the autotuner's first candidates (a batch whose stored shape is
+// left aside), a call on the fixed scratch, the serving ring.
+enum PlanFor { kForBatch, kForTuner, kForNoAlloc, kForRing };
+
+static int make_plan_core(const eat_net *const *nets, int n_nets, int32_t n, const eat_query_opts *o,
+                          Plan &p, PlanFor why) {
+    const int dev = nets[0]->device;
+    const eat_net *const tuned = n_nets == 1 && why != kForRing ? nets[0] : nullptr;
+    const bool own_workspace = why == kForBatch || why == kForTuner, use_tuned = why != kForTuner;
+    int32_t vmax = 0, vmin = INT32_MAX, level = 0;
+    for (int i = 0; i < n_nets; ++i) {
+        vmax = std::max(vmax, nets[i]->host.n_stops);
+        vmin = std::min(vmin, nets[i]->host.n_stops);
+        level = std::max(level, nets[i]->host.e_level);
+    }
     DeviceInfo d;
     int rc = device_info(dev, d);
     if (rc) return rc;
@@ -361,7 +373,11 @@ static int make_plan_core(int dev, int32_t vmax, int32_t n, int n_nets, const ea
     // queries wait).  Fuller batches on one network: as many threads as its rounds fill, several
     // blocks per SM (us for 300 / 1,024 queries: 3,000-stop grid 96 / 114 with 128 threads
     // against 105 / 160 with 512; 10,000-stop city 212 / 363 with 256 against 210 / 408;
-    // 20,000-stop city 293 / 637 with 512 against 309 / 736 with 1,024).  With arrivals in
+    // 20,000-stop city 293 / 637 with 512 against 309 / 736 with 1,024), which is what a level
+    // of the network has edges for (HostNet::e_level; by stops alone a street network; us for
+    // 256 / 1,024 queries: 2,000 stops joined at random 127 / 177 with 128 threads, 56 / 146
+    // with 512; 20,000 444 / 847 with 512, 309 / 628 with 1,024; 10,000-stop full grid 238 /
+    // 297 with 256, 208 / 354 with 512).  With arrivals in
     // global memory two 1,024-thread blocks per SM, until there are enough queries to keep
     // three of 512 threads busy (us for 512 / 1,024 queries: 60,000 stops 1,031 / 1,929
     // against 1,224 / 1,468; 200,000 stops 1,478 / 2,594 against 1,976 / 2,472).  Batches over
@@ -384,8 +400,9 @@ static int make_plan_core(int dev, int32_t vmax, int32_t n, int n_nets, const ea
     else if (!rounds) block = 512;
     else if (n_nets > 1) block = vmax < 16384 || n > 16 * d.sms ? 384 : n > 4 * d.sms ? 512 : 1024;
     else if (!full) block = wide ? 1024 : 512;
-    else if (vmax < 4096) block = 128;
-    else if (vmax < 12288) block = 256;
+    else if (vmax < 4096) block = level > 128 ? 512 : 128;
+    else if (vmax < 12288) block = level > (n <= 3 * d.sms ? 256 : 512) ? 512 : 256;
+    else if (two_shared && level > 512) block = 1024;
     else if (!two_shared && n <= (one_shared ? 3 : vmax < 80000 ? 4 : 5) * d.sms && (branching || !one_shared))
         block = 1024;
     p.block = (o && o->block) ? o->block : (tb ? tb : block);
@@ -494,10 +511,14 @@ static int make_plan_core(int dev, int32_t vmax, int32_t n, int n_nets, const ea
     p.horizon = oh > 0 ? oh : oh < 0 ? 0 : tb ? th : automatic;
     // Threads at work in a default-shaped block (the others leave): no more than the rounds
     // of a small network fill (1,024 stops, 256 queries: 128 of 512 threads 62 us, all 69;
-    // 16,000 stops, 100 queries: 512 157, 1,024 187).
+    // 16,000 stops, 100 queries: 512 157, 1,024 187), unless a level of the network has more
+    // edges than that (HostNet::e_level): all (300 stops joined each to each, one query: 128 of
+    // 1,024 threads 426 us, all 130; 2,000 joined at random 70 and 34).
     p.active = p.block;
-    if (!(o && o->block) && !tb && p.mem == 0)
-        p.active = std::min(p.block, vmax < 2048 ? 128 : vmax < 6144 ? 256 : vmax <= 32768 ? 512 : 1024);
+    if (!(o && o->block) && !tb && p.mem == 0) {
+        const int few = vmax < 2048 ? 128 : vmax < 6144 ? 256 : vmax <= kFewStops ? 512 : 1024;
+        if (level <= few) p.active = std::min(p.block, few);
+    }
     p.build = p.block <= 512 ? kThree512 : n <= d.sms ? kOne1024 : kTwo1024;
     const bool back = leaves_back_out(p.mem, p.build);
     const size_t qbytes = kQueueEntryBytes + (back ? kQueueArrivalBytes : 0), qpad = back ? 8 : 0;
@@ -562,13 +583,12 @@ static int make_plan_core(int dev, int32_t vmax, int32_t n, int n_nets, const ea
 
 // Launch plan for n queries; with a workspace of its own, a batch of more than one query
 // also gets its start order (EAT_ORDER_BY_TIME) at the end of the workspace.
-static int make_plan(int dev, int32_t vmax, int32_t n, int n_nets, const eat_query_opts *o,
-                     Plan &p, int32_t vmin = -1, const eat_net *tuned = nullptr,
-                     bool own_workspace = true, bool use_tuned = true) {
+static int make_plan(const eat_net *const *nets, int n_nets, int32_t n, const eat_query_opts *o,
+                     Plan &p, PlanFor why = kForBatch) {
     const int order = o ? o->order : EAT_ORDER_AUTO;
     if (order < EAT_ORDER_AUTO || order > EAT_ORDER_AS_GIVEN)
         return fail(EAT_ERR_INVALID, "order must be one of EAT_ORDER_*");
-    int rc = make_plan_core(dev, vmax, n, n_nets, o, p, vmin < 0 ? vmax : vmin, tuned, own_workspace, use_tuned);
+    int rc = make_plan_core(nets, n_nets, n, o, p, why);
     if (rc) return rc;
     // Automatic, on one network: sorted when some queries must wait for a free block or share
     // an SM of a network of 8,192 stops or more (they then start longest first) and in the
@@ -577,12 +597,12 @@ static int make_plan(int dev, int32_t vmax, int32_t n, int n_nets, const eat_que
     // with one of 8,192 stops or more among them (64 grids of up to 50,000 stops, 4,096 queries
     // 1,041 -> 709 us, 256 queries 366 -> 317).
     DeviceInfo d;
-    rc = device_info(dev, d);
+    rc = device_info(nets[0]->device, d);
     if (rc) return rc;
-    const bool waits = p.cluster == 0 && !p.pair && (n > p.grid || (vmax >= kWideMinStops && n > d.sms));
-    if (own_workspace && n > 1 &&
+    const bool waits = p.cluster == 0 && !p.pair && (n > p.grid || (p.vmax >= kWideMinStops && n > d.sms));
+    if ((why == kForBatch || why == kForTuner) && n > 1 &&
         (order == EAT_ORDER_BY_TIME ||
-         (order == EAT_ORDER_AUTO && (n_nets == 1 || vmax >= kWideMinStops) && (waits || p.pair)))) {
+         (order == EAT_ORDER_AUTO && (n_nets == 1 || p.vmax >= kWideMinStops) && (waits || p.pair)))) {
         p.order = true;
         p.off_order = align_up(p.ws_bytes, 256);
         p.ws_bytes = p.off_order + align_up((size_t)n * 4, 256);
@@ -683,19 +703,14 @@ static int run_batch(const eat_net *const *nets, int n_nets, const int32_t *net_
                      eat_counters *counters_override, int32_t *arr_rows = nullptr,
                      size_t arr_rows_size = 0) {
     const int dev = nets[0]->device;
-    int32_t vmax = 0, vmin = INT32_MAX;
-    for (int i = 0; i < n_nets; ++i) {
-        vmax = std::max(vmax, nets[i]->host.n_stops);
-        vmin = std::min(vmin, nets[i]->host.n_stops);
-    }
     Plan p;
-    int rc = make_plan(dev, vmax, n, n_nets, o, p, vmin, n_nets == 1 ? nets[0] : nullptr);
+    int rc = make_plan(nets, n_nets, n, o, p);
     if (rc) return rc;
     if (ws_bytes < p.ws_bytes)
         return fail(EAT_ERR_WORKSPACE, "workspace of " + std::to_string(ws_bytes) +
                                            " bytes, need " + std::to_string(p.ws_bytes));
     if (n == 0) return EAT_OK;
-    const int32_t cap = (o && o->max_rounds > 0) ? o->max_rounds : default_round_cap(vmax, p.horizon);
+    const int32_t cap = (o && o->max_rounds > 0) ? o->max_rounds : default_round_cap(p.vmax, p.horizon);
     QueryArgs qa = make_args(p, p.grid, (char *)ws, net_idx, src, ts, n, n_nets, arr_out, arr_off,
                              cap, status_override ? status_override : (o ? o->status : nullptr),
                              counters_override ? counters_override : (o ? o->counters : nullptr));
@@ -732,11 +747,6 @@ static int run_batch(const eat_net *const *nets, int n_nets, const int32_t *net_
 // default shape of a full batch over these networks (all blocks the SMs hold),
 // frontier bitmaps in shared memory.
 int ring_setup(const eat_net *const *nets, int n_nets, RingLaunch &rl) {
-    int32_t vmax = 0, vmin = INT32_MAX;
-    for (int i = 0; i < n_nets; ++i) {
-        vmax = std::max(vmax, nets[i]->host.n_stops);
-        vmin = std::min(vmin, nets[i]->host.n_stops);
-    }
     DeviceInfo d;
     int rc = device_info(nets[0]->device, d);
     if (rc) return rc;
@@ -744,7 +754,7 @@ int ring_setup(const eat_net *const *nets, int n_nets, RingLaunch &rl) {
     o.mode = EAT_MODE_CTA;
     o.block = 512;
     Plan p;
-    rc = make_plan(nets[0]->device, vmax, 4 * d.sms, n_nets, &o, p, vmin, nullptr, false);
+    rc = make_plan(nets, n_nets, 4 * d.sms, &o, p, kForRing);
     if (rc) return rc;
     if (p.mem == 2)
         return fail(EAT_ERR_INVALID, "ring admission keeps the frontier bitmaps in shared memory; "
@@ -1027,15 +1037,10 @@ size_t eat_workspace_bytes(const eat_net *const *nets, int32_t n_nets, int32_t n
                            const eat_query_opts *opts) {
     clear_error();
     if (!nets || n_nets < 1 || n_nets > EAT_MAX_NETS || n < 0) return 0;
-    int32_t vmax = 0, vmin = INT32_MAX;
-    for (int i = 0; i < n_nets; ++i) {
+    for (int i = 0; i < n_nets; ++i)
         if (!nets[i] || nets[i]->device < 0 || nets[i]->device != nets[0]->device) return 0;
-        vmax = std::max(vmax, nets[i]->host.n_stops);
-        vmin = std::min(vmin, nets[i]->host.n_stops);
-    }
     Plan p;
-    if (make_plan(nets[0]->device, vmax, n, n_nets, opts, p, vmin, n_nets == 1 ? nets[0] : nullptr))
-        return 0;
+    if (make_plan(nets, n_nets, n, opts, p)) return 0;
     return p.ws_bytes;
 }
 
@@ -1044,16 +1049,13 @@ int eat_launch_shape(const eat_net *const *nets, int32_t n_nets, int32_t n,
     clear_error();
     if (!nets || !shape || n_nets < 1 || n_nets > EAT_MAX_NETS || n < 0)
         return fail(EAT_ERR_INVALID, "invalid arguments");
-    int32_t vmax = 0, vmin = INT32_MAX;
     for (int i = 0; i < n_nets; ++i) {
         if (!nets[i]) return fail(EAT_ERR_INVALID, "NULL network");
         if (nets[i]->device < 0) return fail(EAT_ERR_NO_DEVICE, "network was built host-only");
         if (nets[i]->device != nets[0]->device) return fail(EAT_ERR_INVALID, "networks on different devices");
-        vmax = std::max(vmax, nets[i]->host.n_stops);
-        vmin = std::min(vmin, nets[i]->host.n_stops);
     }
     Plan p;
-    int rc = make_plan(nets[0]->device, vmax, n, n_nets, opts, p, vmin, n_nets == 1 ? nets[0] : nullptr);
+    int rc = make_plan(nets, n_nets, n, opts, p);
     if (rc) return rc;
     *shape = opts ? *opts : eat_query_opts{};
     shape->block = p.block;
@@ -1080,7 +1082,7 @@ int eat_query(const eat_net *net, int32_t s, int32_t t_s, int32_t *arr_out,
     if (at.type == cudaMemoryTypeDevice && at.device != net->device) return foreign_fail();
     std::lock_guard<std::mutex> g(net->ws_lock);
     Plan p;
-    int rc = make_plan(net->device, net->host.n_stops, 1, 1, nullptr, p, -1, net);
+    int rc = make_plan(&net, 1, 1, nullptr, p);
     if (rc) return rc;
     DeviceGuard guard(net->device);
     // A page-locked host row is written in place; arrivals that do not fit in shared
@@ -1203,13 +1205,8 @@ int eat_query_batch_multi(const eat_net *const *nets, int32_t n_nets, const int3
     int32_t *out_map = dev_out ? nullptr : (int32_t *)mapped_host_ptr(arr_out);
     size_t rows_bytes = 0;
     if (out_map) {
-        int32_t vmax = 0, vmin = INT32_MAX;
-        for (int i = 0; i < n_nets; ++i) {
-            vmax = std::max(vmax, nets[i]->host.n_stops);
-            vmin = std::min(vmin, nets[i]->host.n_stops);
-        }
         Plan p;
-        if (make_plan(nets[0]->device, vmax, n, n_nets, opts, p, vmin, n_nets == 1 ? nets[0] : nullptr)) {
+        if (make_plan(nets, n_nets, n, opts, p)) {
             clear_error();
             out_map = nullptr;
         } else {
@@ -1295,7 +1292,7 @@ int eat_query_batch(const eat_net *net, const int32_t *sources, const int32_t *t
     size_t rows_bytes = 0;                       // per-block arrival rows (host rows only)
     if (out_map) {
         Plan p;
-        if (make_plan(net->device, net->host.n_stops, n, 1, opts, p, -1, net) != EAT_OK) {
+        if (make_plan(nets, 1, n, opts, p) != EAT_OK) {
             clear_error();
             out_map = nullptr;
         } else {
@@ -1502,7 +1499,7 @@ extern "C" int eat_autotune(eat_net *net, const int32_t *sources, const int32_t 
     eat_query_opts plain{};
     plain.mode = EAT_MODE_CTA;
     Plan first;
-    const int frc = make_plan(net->device, net->host.n_stops, n, 1, &plain, first, -1, net, true, false);
+    const int frc = make_plan(nets, 1, n, &plain, first, kForTuner);
     if (frc) return frc;
     std::vector<int> blocks;
     for (int b : {first.block, 1024, 512, 256})
@@ -1593,14 +1590,9 @@ extern "C" int eat_autotune_multi(const eat_net *const *nets, int32_t n_nets, co
     // Candidates in a fixed order, the automatic start order and block size first (256 where
     // that is 384): each start order with three block sizes, each with vwarp 8, 4, 16 and the
     // round-free mode; then horizons of 2 and 12 hours (512 threads, vwarp 8, in order of t_s).
-    int32_t vmax = 0, vmin = INT32_MAX;
-    for (int i = 0; i < n_nets; ++i) {
-        vmax = std::max(vmax, nets[i]->host.n_stops);
-        vmin = std::min(vmin, nets[i]->host.n_stops);
-    }
     Plan first;
     eat_query_opts plain{};
-    int rc = make_plan(dev, vmax, n, n_nets, &plain, first, vmin, n_nets == 1 ? nets[0] : nullptr, true, false);
+    int rc = make_plan(nets, n_nets, n, &plain, first, kForTuner);
     if (rc) {
         cudaFree(d_offs);
         return rc;
@@ -1685,7 +1677,7 @@ extern "C" int eat_query_batch_noalloc(const eat_net *net, const int32_t *source
     for (const void *b : {(const void *)sources, (const void *)times, (const void *)arr_out})
         if (foreign_ptr(b, net->device)) return foreign_fail();
     Plan p;
-    int rc = make_plan(net->device, net->host.n_stops, n, 1, opts, p, -1, net, false);
+    int rc = make_plan(&net, 1, n, opts, p, kForNoAlloc);
     if (rc) return rc;
     // Fewer persistent blocks so that their queue spill fits the fixed scratch (with a horizon
     // the documented 16 bytes a stop are asked for, though the bitmap takes less).

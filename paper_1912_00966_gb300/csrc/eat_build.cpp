@@ -608,6 +608,30 @@ int build_fused(HostNet &h) {
     return EAT_OK;
 }
 
+// See HostNet::e_level; head stops of the edges in `heads`.
+static int32_t mean_level(const HostNet &h, const std::vector<int32_t> &heads) {
+    std::vector<int32_t> tails, queue((size_t)h.n_stops), seen((size_t)h.n_stops, -1);
+    for (int32_t u = 0; u < h.n_stops; ++u)
+        if (h.erow[u + 1] > h.erow[u]) tails.push_back(u);
+    int64_t most = 0;
+    for (int32_t k = 0; k < 4 && !tails.empty(); ++k) {
+        int64_t edges = 0, levels = 0;
+        size_t n = 0;
+        const int32_t s = tails[tails.size() * (size_t)k / 4];
+        seen[s] = k;
+        queue[n++] = s;
+        for (size_t i = 0, end; i < n; ++levels)
+            for (end = n; i < end; ++i)
+                for (int32_t e = h.erow[queue[i]]; e < h.erow[queue[i] + 1]; ++e, ++edges)
+                    if (const int32_t v = heads[e]; seen[v] != k) {
+                        seen[v] = k;
+                        if (h.erow[v + 1] > h.erow[v]) queue[n++] = v;
+                    }
+        most = std::max(most, edges / std::max<int64_t>(levels, 1));
+    }
+    return (int32_t)std::min<int64_t>(most, INT32_MAX);
+}
+
 // Edge table (see EdgeDev in eat_internal.h): per edge the merged departures of all its
 // connection types without dominated ones, cut into time slots of 2^shift seconds.
 int build_edges(HostNet &h) {
@@ -759,6 +783,7 @@ int build_edges(HostNet &h) {
         h.erow[V] = r;
         for (const Part &p : parts) heads.insert(heads.end(), p.head.begin(), p.head.end());
     }
+    h.e_level = V <= kFewStops ? mean_level(h, heads) : 0;
     // Entries, with list offsets local to the part; the lists' places follow from their sizes.
     const bool big = V > kMaxPackedStops;
     auto fill = [&](Part &p) {

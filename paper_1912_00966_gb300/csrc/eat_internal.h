@@ -132,6 +132,9 @@ struct EdgeTable {
     EdgeDev net[NETS];
 };
 
+// Networks of up to this many stops may leave threads of a block without work.
+constexpr int32_t kFewStops = 32768;
+
 // Host copy of the built arrays (kept for eat_net_host_view).
 struct HostNet {
     int32_t n_stops = 0, n_types = 0, n_edges = 0, width = 3600, t0 = 0;
@@ -156,6 +159,10 @@ struct HostNet {
     size_t ee_words = 0;
     std::vector<int32_t> ex;         // 2 per pair
     std::vector<int32_t> etypes;     // E
+    // Edges leaving the stops at one distance (in connections) from a source, on average over
+    // the distances: the most of four sources, 0 for networks of more than kFewStops stops.
+    // What a round has work for, about.
+    int32_t e_level = 0;
 };
 
 }  // namespace eat
