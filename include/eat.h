@@ -209,8 +209,10 @@ typedef struct {
                                 improved stop in the next round).
                                 0 = automatic (the value eat_autotune chose for this
                                 batch size, else, for a call without a round cap on one
-                                network whose stops have two or more edges on average,
-                                two hours when the arrivals are in global memory and four
+                                network whose stops have two or more edges on average
+                                and whose connections are short beside it (a mean of
+                                1,000 s or less with the wait, more where rounds are
+                                heavy), two hours when the arrivals are in global memory and four
                                 hours in shared memory for batches of two queries or more
                                 (from one to 1.125 queries per SM only where stops have 2.6
                                 edges or more); none otherwise and in

@@ -507,6 +507,16 @@ static int make_plan_core(const eat_net *const *nets, int n_nets, int32_t n, con
     if (own_workspace && branching && !(o && o->max_rounds > 0)) {
         const bool one_each = n >= d.sms && n <= d.sms + d.sms / 8;
         automatic = p.mem != 0 ? 7200 : n > 1 && (!one_each || tuned->branching > 1) ? 14400 : 0;
+        // Where a connection takes long, a horizon holds few of them and moves in nearly every
+        // round (us without / with it, 300 queries: 60,000-stop full grid, 1-hour connections
+        // every three hours 182 / 417, 15-minute ones every 15 minutes 462 / 565; 2,000 stops
+        // joined at random, 22-hour ones 33 / 115; streets: 10 minutes).  Up to 1,000 s a
+        // connection, then; or where rounds have more work than threads, so that fewer
+        // expansions outweigh more rounds (20,000 stops joined at random, 15-minute ones every
+        // three hours 360 / 266), unless it does not hold one (22-hour ones 50 / 110).
+        const HostNet &h = tuned->host;
+        const bool heavy = h.e_level > 512 && (int64_t)h.n_edges >= 16384;
+        if (h.e_travel > automatic || (h.e_travel + h.e_wait > 1000 && !heavy)) automatic = 0;
     }
     p.horizon = oh > 0 ? oh : oh < 0 ? 0 : tb ? th : automatic;
     // Threads at work in a default-shaped block (the others leave): no more than the rounds

@@ -644,6 +644,7 @@ int build_edges(HostNet &h) {
         std::vector<Pair> pairs;
         std::vector<int32_t> ex;
         int64_t quads = 0;
+        int64_t travel = 0, wait = 0, waits = 0;      // durations; gaps between departures, their number
         bool oom = false;
     };
     const unsigned hw = std::max(1u, std::min(32u, std::thread::hardware_concurrency()));
@@ -716,6 +717,9 @@ int build_edges(HostNet &h) {
                         all[keep] = all[m];
                     }
                 p.pairs.insert(p.pairs.end(), all.begin() + (ptrdiff_t)keep, all.end());
+                for (size_t m = keep; m < all.size(); ++m) p.travel += all[m].arr - all[m].dep;
+                p.wait += (int64_t)all.back().dep - all[keep].dep;
+                p.waits += (int64_t)(all.size() - keep) - 1;
                 p.ptr.push_back((int64_t)p.pairs.size());
                 p.head.push_back(head(ts[i]));
                 p.types.push_back((int32_t)(j - i));
@@ -726,18 +730,23 @@ int build_edges(HostNet &h) {
     });
     if (!ok) return fail(EAT_ERR_OOM, "host allocation of the edge table failed");
 
-    int64_t E = 0, n_pairs = 0;
+    int64_t E = 0, n_pairs = 0, travel = 0, wait = 0, waits = 0;
     int32_t first = EAT_INF, last = INT32_MIN;
     std::vector<int64_t> e_off((size_t)n_parts);
     for (int k = 0; k < n_parts; ++k) {
         e_off[k] = E;
         E += (int64_t)parts[k].head.size();
         n_pairs += (int64_t)parts[k].pairs.size();
+        travel += parts[k].travel;
+        wait += parts[k].wait;
+        waits += parts[k].waits;
         for (size_t e = 0; e < parts[k].head.size(); ++e) {
             first = std::min(first, parts[k].pairs[(size_t)parts[k].ptr[e]].dep);
             last = std::max(last, parts[k].pairs[(size_t)parts[k].ptr[e + 1] - 1].dep);
         }
     }
+    h.e_travel = n_pairs ? (int32_t)(travel / n_pairs) : 0;
+    h.e_wait = waits ? (int32_t)(wait / waits) / 2 : 0;
     h.e_base = E ? first : 0;
     h.e_shift = 0;
     h.e_y = 0;
@@ -783,7 +792,7 @@ int build_edges(HostNet &h) {
         h.erow[V] = r;
         for (const Part &p : parts) heads.insert(heads.end(), p.head.begin(), p.head.end());
     }
-    h.e_level = V <= kFewStops ? mean_level(h, heads) : 0;
+    h.e_level = mean_level(h, heads);
     // Entries, with list offsets local to the part; the lists' places follow from their sizes.
     const bool big = V > kMaxPackedStops;
     auto fill = [&](Part &p) {

@@ -160,9 +160,11 @@ struct HostNet {
     std::vector<int32_t> ex;         // 2 per pair
     std::vector<int32_t> etypes;     // E
     // Edges leaving the stops at one distance (in connections) from a source, on average over
-    // the distances: the most of four sources, 0 for networks of more than kFewStops stops.
-    // What a round has work for, about.
+    // the distances: the most of four sources.  What a round has work for, about.
     int32_t e_level = 0;
+    // Mean duration of the kept departures, and half the mean gap between an edge's: together
+    // the time that a connection takes a traveller, about.
+    int32_t e_travel = 0, e_wait = 0;
 };
 
 }  // namespace eat

@@ -85,3 +85,31 @@ def test_threads_fit_the_rounds(make, n):
     best = min(c.us(block=b) for b in (256, 512, 1024))
     assert c.us() < 1.5 * best
     c.net.close()
+
+
+@pytest.mark.parametrize("net,horizon", [
+    ("city", 14400), ("random, 10 minutes", 14400),
+    ("random, 22 hours", -1), ("grid, 1 hour every three", -1)])
+def test_horizon_where_it_holds_many_connections(net, horizon):
+    """An automatic horizon is for connections that are short beside it: with long or rare ones it
+    moves in nearly every round."""
+    if net == "city":
+        tt = synth.city()
+    elif net.startswith("random"):
+        long = net.endswith("hours")
+        t = _random(2000, 4)
+        e = np.unique(t.u.astype(np.int64) * 2000 + t.v)
+        dur = np.random.default_rng(3).integers(*((70000, 90000) if long else (60, 600)), e.shape[0])
+        tt = _service(2000, e // 2000, e % 2000, dur, 3 * HOUR if long else 600, 4, 0, 300000 if long else 23 * HOUR)
+    else:
+        x, y = np.divmod(np.arange(10000), 100)
+        at = np.arange(10000)
+        e = [(at[m], (at + s)[m]) for m, s in ((y < 99, 1), (y > 0, -1), (x < 99, 100), (x > 0, -100))]
+        u, v = (np.concatenate(a) for a in zip(*e))
+        tt = _service(10000, u, v, np.random.default_rng(3).integers(2400, 4800, u.shape[0]), 3 * HOUR, 4, 0, 200000)
+    c = _Case(tt, 37)
+    assert c.eat.eat_launch_shape(c.net, 37)["horizon"] == horizon
+    c.check()
+    if horizon < 0:
+        assert c.us() < 1.25 * c.us(horizon=-1)
+    c.net.close()
