@@ -113,9 +113,12 @@ static int device_info(int dev, DeviceInfo &out) {
                                       cta_kernel(nets, mem, kOne1024, false, true), cta_kernel(nets, mem, kTwo1024),
                                       cta_kernel(nets, mem, kTwo1024, false, true), cta_kernel(nets, mem, kThree512),
                                       cta_kernel(nets, mem, kThree512, false, true),
+                                      cta_kernel(nets, mem, kOne1024, false, true, true),
+                                      cta_kernel(nets, mem, kTwo1024, false, true, true),
+                                      cta_kernel(nets, mem, kThree512, false, true, true),
                                       async_kernel(nets, mem),
                                       cluster_kernel(), pair_kernel(false), pair_kernel(true),
-                                      ring_kernel(mem)}) {
+                                      ring_kernel(mem, false), ring_kernel(mem, true)}) {
                     e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)(d.smem_optin - d.reserve));
                     if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute");
@@ -350,10 +353,12 @@ static int make_plan_core(const eat_net *const *nets, int n_nets, int32_t n, con
     const eat_net *const tuned = n_nets == 1 && why != kForRing ? nets[0] : nullptr;
     const bool own_workspace = why == kForBatch || why == kForTuner, use_tuned = why != kForTuner;
     int32_t vmax = 0, vmin = INT32_MAX, level = 0;
+    bool hubs = false;
     for (int i = 0; i < n_nets; ++i) {
         vmax = std::max(vmax, nets[i]->host.n_stops);
         vmin = std::min(vmin, nets[i]->host.n_stops);
         level = std::max(level, nets[i]->host.e_level);
+        hubs = hubs || wants_hubs(&nets[i]->edev, 1);
     }
     DeviceInfo d;
     int rc = device_info(dev, d);
@@ -550,7 +555,7 @@ static int make_plan_core(const eat_net *const *nets, int n_nets, int32_t n, con
     int reg_blocks = 1;                       // with at most one query per SM one is all it holds
     if (n > d.sms) {
         DeviceGuard guard(dev);
-        const void *k = cta_kernel(p.nets, p.mem, p.build, false, p.horizon > 0);
+        const void *k = cta_kernel(p.nets, p.mem, p.build, false, p.horizon > 0, hubs);
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&reg_blocks, k, p.block, 0) != cudaSuccess) {
             cudaGetLastError();
             reg_blocks = 0;
@@ -576,7 +581,7 @@ static int make_plan_core(const eat_net *const *nets, int n_nets, int32_t n, con
     if (n != 1) {                             // a single query: a block always fits an SM
         DeviceGuard guard(dev);
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-            &per_sm, cta_kernel(p.nets, p.mem, p.build, false, p.horizon > 0), p.block, p.smem);
+            &per_sm, cta_kernel(p.nets, p.mem, p.build, false, p.horizon > 0, hubs), p.block, p.smem);
     }
     if (e != cudaSuccess) return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
     if (per_sm < 1) return fail(EAT_ERR_INVALID, "kernel does not fit on an SM with this block size");
@@ -770,9 +775,11 @@ int ring_setup(const eat_net *const *nets, int n_nets, RingLaunch &rl) {
         return fail(EAT_ERR_INVALID, "ring admission keeps the frontier bitmaps in shared memory; "
                                      "these networks are too large (use EAT_ADMIT_BATCH)");
     int per_sm = 0;
+    bool hubs = false;
+    for (int i = 0; i < n_nets; ++i) hubs = hubs || wants_hubs(&nets[i]->edev, 1);
     {
         DeviceGuard guard(nets[0]->device);
-        cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ring_kernel(p.mem),
+        cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ring_kernel(p.mem, hubs),
                                                                       p.block, p.smem);
         if (e != cudaSuccess) return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
     }
@@ -913,6 +920,7 @@ static int upload(eat_net *net) {
     x.shift = h.e_shift;
     x.y = h.e_y;
     x.big = h.n_stops > kMaxPackedStops;
+    x.lanes = h.e_lanes;
     int64_t tails = 0;
     for (int32_t u = 0; u < h.n_stops; ++u) tails += h.erow[u + 1] > h.erow[u];
     net->branching = tails == 0 ? 0 : 5 * (int64_t)x.n_edges >= 13 * tails ? 2 : x.n_edges >= 2 * tails ? 1 : 0;

@@ -72,8 +72,10 @@ constexpr int32_t kInlineAps = 4;
 constexpr int32_t kNoDeparture = 0xffff;
 constexpr int32_t kEdgeOverflow = 15;
 constexpr int32_t kMaxPackedStops = 1 << 24;
+constexpr int32_t kHubs = 4;          // in EdgeDev::lanes
 
 struct EdgeDev {
+    static constexpr int32_t kUsualLanes = 2;
     const int32_t *erow;      // [V + 1]
     const int2 *er;           // [E]
     const int4 *ee;           // [y * E], slot-major
@@ -85,6 +87,8 @@ struct EdgeDev {
     int32_t shift;            // slots of 2^shift seconds
     int32_t y;                // slots
     int32_t big;              // more than 2^24 stops: er holds no degree
+    int32_t lanes;            // log2 of the lanes per stop in a crowded round; | kHubs: some stop
+                              // has kEdgeOverflow edges or more
 };
 
 struct NetDev {
@@ -159,6 +163,7 @@ struct HostNet {
     size_t ee_words = 0;
     std::vector<int32_t> ex;         // 2 per pair
     std::vector<int32_t> etypes;     // E
+    int32_t e_lanes = EdgeDev::kUsualLanes;
     // Edges leaving the stops at one distance (in connections) from a source, on average over
     // the distances: the most of four sources.  What a round has work for, about.
     int32_t e_level = 0;

@@ -180,8 +180,11 @@ __device__ __forceinline__ void fill_inf(int32_t *p, int32_t n, int tid, int nth
 // 1,024-thread blocks per SM 851 against 969 for one).
 // COUNT: the build that fills qa.counters; without it the per-thread work counters are
 // dead code and compiled away (the timed launches pass no counters).  HZ: the build that
-// honours qa.horizon.
-template <int NETS, int ARR, bool SMEM_MASK, int BUILD, bool RING = false, bool COUNT = false, bool HZ = true>
+// honours qa.horizon.  HUB: the build for networks with hubs or with lanes per stop of their own
+// (EdgeDev::lanes); the others' rounds are 5 to 25 % longer with it (20,000-stop city 256
+// queries 292 -> 307 us, 60,000 stops 300 queries 812 -> 1,015: registers).
+template <int NETS, int ARR, bool SMEM_MASK, int BUILD, bool RING = false, bool COUNT = false, bool HZ = true,
+          bool HUB = COUNT>
 __global__ void __launch_bounds__(BUILD == kThree512 ? 512 : 1024,
                                   BUILD == kThree512 ? 3 : BUILD == kTwo1024 ? 2 : 1)
 eat_cta_kernel(const __grid_constant__ EdgeTable<NETS> nets, const QueryArgs qa) {
@@ -191,6 +194,7 @@ eat_cta_kernel(const __grid_constant__ EdgeTable<NETS> nets, const QueryArgs qa)
     __shared__ int32_t s_n[2];        // stops queued so far in even and in odd rounds
     __shared__ int32_t s_min[2];      // least arrival given to a waiting stop (alternating)
     __shared__ int32_t s_rel[2];      // stops released (alternating)
+    __shared__ int32_t s_hub;         // pieces of hubs listed this round
     __shared__ unsigned long long s_cnt[6];
 
     const int tid = threadIdx.x;
@@ -264,6 +268,7 @@ eat_cta_kernel(const __grid_constant__ EdgeTable<NETS> nets, const QueryArgs qa)
         }
         const bool hz_on = HZ && qa.horizon > 0;
         if (tid < 2) s_n[tid] = 0;
+        if (HUB && tid == 0) s_hub = 0;
         if (hz_on && clear_wait)
             for (int32_t i = tid; i < qa.mask_words; i += nthr) wait[i] = 0u;
         if (HZ && tid < 2) {
@@ -361,7 +366,6 @@ eat_cta_kernel(const __grid_constant__ EdgeTable<NETS> nets, const QueryArgs qa)
                 // slot y holds no departures
                 const uint32_t k = min(edge_slot(N.base, N.shift, e_u, rel, start), (uint32_t)N.y);
                 const int4 *const slab = N.ee + (uint64_t)k * (uint32_t)N.n_edges;
-                if (COUNT) c_vert += lane == 0;
                 const int32_t end = t + d;
                 const int32_t back = back_out && e_u == arrived && b != kEdgeOverflow ? t + b : -1;
 #pragma unroll 1
@@ -383,23 +387,76 @@ eat_cta_kernel(const __grid_constant__ EdgeTable<NETS> nets, const QueryArgs qa)
                 }
             };
 
+            // A hub, a stop of more edges than its sub-warp of 2^pl lanes takes in four passes, is
+            // listed in pieces of whole warps, as many as the block has at most, behind the
+            // spilled stops (whose buffer holds every stop twice over the rounds); the warps
+            // share the pieces once the queue is done.  One sub-warp alone kept the round
+            // waiting: 10 hubs of 2,000 spokes, one query 574 -> 60 us, 37 queries 716 -> 67;
+            // 100 of 200 302 -> 91 and 375 -> 113.
+            const int32_t pieces = (qa.vmax - max(n - qcap, 0)) >> 1;     // room for them
+            auto piece = [&](int32_t d) {                 // log2 of a piece's length
+                int l = 5;
+                while (l < 25 && d > nthr << (l - 5)) ++l;
+                return l;
+            };
+            auto hub = [&](int32_t u, int32_t t, int pl, int lane) {
+                const int32_t d = __ldg(N.erow + u + 1) - t;
+                if (d <= 4 << pl) return false;
+                const int l = piece(d);
+                const int32_t k = (d - 1 >> l) + 1;
+                const uint32_t lanes = 0xffffffffu >> (32 - (1 << pl)) << (tid & 31 & -(1 << pl));
+                int32_t pos = lane == 0 ? atomicAdd(&s_hub, k) : 0;
+                pos = __shfl_sync(lanes, pos, 0, 1 << pl);
+                const bool room = pos + k <= pieces;
+                for (int32_t j = lane; j < k && pos + j < pieces; j += 1 << pl) {
+                    int32_t *const p = sp_rd + qa.vmax - 2 * (pos + j + 1);
+                    p[0] = room ? u : -1;                     // no room for all of them: for none
+                    p[1] = t + (j << l);
+                }
+                return room;
+            };
+
             // A sub-warp of 2^pl lanes per stop: `vwarp` lanes while that keeps every stop of
-            // the round in one pass, else four.
-            const int pl = (n << qa.vw_log2) <= nthr ? qa.vw_log2 : min(qa.vw_log2, 2);
+            // the round in one pass, else four, or what most stops of the network have edges for.
+            const int few = HUB ? N.lanes & 3 : 2;
+            const int pl = (n << qa.vw_log2) <= nthr ? qa.vw_log2 : min(qa.vw_log2, few);
             const int lane = tid & ((1 << pl) - 1);
             const int nsub = nthr >> pl;
             const int32_t nq = min(n, qcap);
 #pragma unroll 1
             for (int32_t i = tid >> pl; i < nq; i += nsub) {
                 const int2 e = q_rd[i];
-                expand(big ? e.x : e.x & 0xffffff, e.y, big ? kEdgeOverflow : (int32_t)((uint32_t)e.x >> 28),
-                       1 << pl, lane, back_out ? from(q_rd)[i] : 0, big ? kEdgeOverflow : (int32_t)((uint32_t)e.x >> 24 & 15u));
+                const int32_t u = big ? e.x : e.x & 0xffffff;
+                const int32_t d = big ? kEdgeOverflow : (int32_t)((uint32_t)e.x >> 28);
+                if (COUNT) c_vert += lane == 0;
+                if (HUB && d == kEdgeOverflow && (N.lanes & kHubs) && hub(u, e.y, pl, lane)) continue;
+                expand(u, e.y, d, 1 << pl, lane, back_out ? from(q_rd)[i] : 0,
+                       big ? kEdgeOverflow : (int32_t)((uint32_t)e.x >> 24 & 15u));
             }
             if (n > qcap) {                                 // spilled stops
+                const int sl = few == 2 ? 3 : few, sub = tid & ((1 << sl) - 1);
 #pragma unroll 1
-                for (int32_t i = tid >> 3; i < n - qcap; i += nthr >> 3) {
-                    const int32_t u = __ldcg(sp_rd + i);
-                    expand(u, __ldg(N.erow + u), kEdgeOverflow, 8, tid & 7, 0, kEdgeOverflow);
+                for (int32_t i = tid >> sl; i < n - qcap; i += nthr >> sl) {
+                    const int32_t u = __ldcg(sp_rd + i), t = __ldg(N.erow + u);
+                    if (COUNT) c_vert += sub == 0;
+                    if (HUB && (N.lanes & kHubs) && hub(u, t, sl, sub)) continue;
+                    expand(u, t, kEdgeOverflow, 1 << sl, sub, 0, kEdgeOverflow);
+                }
+            }
+            if (HUB && (N.lanes & kHubs)) {
+                __syncthreads();
+                const int32_t wanted = s_hub, listed = min(wanted, pieces);
+                if (wanted > 0) {
+                    __syncthreads();                      // everyone has read it
+                    if (tid == 0) s_hub = 0;
+#pragma unroll 1
+                    for (int32_t i = tid >> 5; i < listed; i += nthr >> 5) {
+                        const int32_t *const p = sp_rd + qa.vmax - 2 * (i + 1);
+                        const int32_t u = __ldcg(p), t = __ldcg(p + 1);
+                        if (u < 0) continue;
+                        const int32_t end = __ldg(N.erow + u + 1);
+                        expand(u, t, min(1 << piece(end - __ldg(N.erow + u)), end - t), 32, tid & 31, 0, kEdgeOverflow);
+                    }
                 }
             }
             __syncthreads();
@@ -1271,19 +1328,24 @@ eat_cluster_kernel(const __grid_constant__ NetTable<NETS> nets, const QueryArgs 
     cluster.sync();                                   // block 0 is done reading the others
 }
 
-template <int NETS, int BUILD, bool COUNT, bool HZ>
+template <int NETS, int BUILD, bool COUNT, bool HZ, bool HUB = COUNT>
 static const void *cta_kernel_ptr(int mem) {
     switch (mem) {
-    case 0: return (const void *)eat_cta_kernel<NETS, kArrShared, true, BUILD, false, COUNT, HZ>;
-    case 1: return (const void *)eat_cta_kernel<NETS, kArrGlobal, true, BUILD, false, COUNT, HZ>;
-    case 3: return (const void *)eat_cta_kernel<NETS, kArrPerQuery, true, BUILD, false, COUNT, HZ>;
-    default: return (const void *)eat_cta_kernel<NETS, kArrGlobal, false, BUILD, false, COUNT, HZ>;
+    case 0: return (const void *)eat_cta_kernel<NETS, kArrShared, true, BUILD, false, COUNT, HZ, HUB>;
+    case 1: return (const void *)eat_cta_kernel<NETS, kArrGlobal, true, BUILD, false, COUNT, HZ, HUB>;
+    case 3: return (const void *)eat_cta_kernel<NETS, kArrPerQuery, true, BUILD, false, COUNT, HZ, HUB>;
+    default: return (const void *)eat_cta_kernel<NETS, kArrGlobal, false, BUILD, false, COUNT, HZ, HUB>;
     }
 }
 
 template <int NETS>
-static const void *cta_kernel_for(int mem, int build, bool count, bool hz) {
-    if (count) return cta_kernel_ptr<NETS, kOne1024, true, true>(mem);   // honours a horizon, if there is one
+static const void *cta_kernel_for(int mem, int build, bool count, bool hz, bool hubs) {
+    // These honour a horizon, if there is one.
+    if (count) return cta_kernel_ptr<NETS, kOne1024, true, true>(mem);
+    if (hubs)
+        return build == kThree512  ? cta_kernel_ptr<NETS, kThree512, false, true, true>(mem)
+               : build == kTwo1024 ? cta_kernel_ptr<NETS, kTwo1024, false, true, true>(mem)
+                                   : cta_kernel_ptr<NETS, kOne1024, false, true, true>(mem);
     switch (build) {
     case kThree512:
         return hz ? cta_kernel_ptr<NETS, kThree512, false, true>(mem) : cta_kernel_ptr<NETS, kThree512, false, false>(mem);
@@ -1294,9 +1356,15 @@ static const void *cta_kernel_for(int mem, int build, bool count, bool hz) {
     }
 }
 
-const void *cta_kernel(int nets, int mem, int build, bool count, bool hz) {
-    return nets == 1 ? cta_kernel_for<1>(mem, build, count, hz)
-                     : cta_kernel_for<EAT_MAX_NETS>(mem, build, count, hz);
+const void *cta_kernel(int nets, int mem, int build, bool count, bool hz, bool hubs) {
+    return nets == 1 ? cta_kernel_for<1>(mem, build, count, hz, hubs)
+                     : cta_kernel_for<EAT_MAX_NETS>(mem, build, count, hz, hubs);
+}
+
+bool wants_hubs(const EdgeDev *nets, int n_nets) {
+    bool any = false;
+    for (int i = 0; i < n_nets; ++i) any = any || nets[i].lanes != EdgeDev::kUsualLanes;
+    return any;
 }
 
 template <int NETS>
@@ -1345,22 +1413,28 @@ static cudaError_t launch_cta_t(const void *kernel, const EdgeDev *nets, int n_n
 
 cudaError_t launch_cta(const EdgeDev *nets, int n_nets, const QueryArgs &qa, int mem, int build, int grid,
                        int block, size_t smem, cudaStream_t st) {
-    const void *k = cta_kernel(n_nets == 1 ? 1 : EAT_MAX_NETS, mem, build, qa.counters != nullptr, qa.horizon > 0);
+    const void *k = cta_kernel(n_nets == 1 ? 1 : EAT_MAX_NETS, mem, build, qa.counters != nullptr, qa.horizon > 0,
+                               wants_hubs(nets, n_nets));
     return n_nets == 1 ? launch_cta_t<1>(k, nets, n_nets, qa, grid, block, smem, st)
                        : launch_cta_t<EAT_MAX_NETS>(k, nets, n_nets, qa, grid, block, smem, st);
 }
 
-const void *ring_kernel(int mem) {
+template <bool HUB>
+static const void *ring_kernel_ptr(int mem) {
     switch (mem) {
-    case 0: return (const void *)eat_cta_kernel<EAT_MAX_NETS, kArrShared, true, kThree512, true, false, false>;
-    case 3: return (const void *)eat_cta_kernel<EAT_MAX_NETS, kArrPerQuery, true, kThree512, true, false, false>;
-    default: return (const void *)eat_cta_kernel<EAT_MAX_NETS, kArrGlobal, true, kThree512, true, false, false>;
+    case 0: return (const void *)eat_cta_kernel<EAT_MAX_NETS, kArrShared, true, kThree512, true, false, false, HUB>;
+    case 3: return (const void *)eat_cta_kernel<EAT_MAX_NETS, kArrPerQuery, true, kThree512, true, false, false, HUB>;
+    default: return (const void *)eat_cta_kernel<EAT_MAX_NETS, kArrGlobal, true, kThree512, true, false, false, HUB>;
     }
+}
+
+const void *ring_kernel(int mem, bool hubs) {
+    return hubs ? ring_kernel_ptr<true>(mem) : ring_kernel_ptr<false>(mem);
 }
 
 cudaError_t launch_ring(const EdgeDev *nets, int n_nets, const QueryArgs &qa, int mem, int grid,
                         int block, size_t smem, cudaStream_t st) {
-    return launch_cta_t<EAT_MAX_NETS>(ring_kernel(mem), nets, n_nets, qa, grid, block, smem, st);
+    return launch_cta_t<EAT_MAX_NETS>(ring_kernel(mem, wants_hubs(nets, n_nets)), nets, n_nets, qa, grid, block, smem, st);
 }
 
 const void *pair_kernel(bool count) {

@@ -39,6 +39,20 @@ def _random(n, degree):
     return _service(n, key // n, key % n, rng.integers(60, 600, key.shape[0]), 300, n)
 
 
+def _hubs(degrees, leaves, seed=1):
+    """A ring of stops with `degrees` spokes each; a spoke leads back unless it is a leaf."""
+    degrees = np.asarray(degrees)
+    h = degrees.shape[0]
+    hub = np.repeat(np.arange(h), degrees)
+    spoke = h + np.arange(hub.shape[0])
+    ring = np.arange(h)
+    rng = np.random.default_rng(seed)
+    u = np.concatenate([ring, hub] + ([] if leaves else [spoke, spoke]))
+    v = np.concatenate([(ring + 1) % h, spoke] + ([] if leaves else [hub, rng.permutation(spoke)]))
+    dur = rng.integers(60, 1200, u.shape[0])
+    return _service(h + spoke.shape[0], u, v, dur, rng.integers(300, 2400, u.shape[0]), seed)
+
+
 class _Case:
     def __init__(self, tt, n, seed=5):
         from paper_1912_00966_gb300 import eat
@@ -113,3 +127,80 @@ def test_horizon_where_it_holds_many_connections(net, horizon):
     if horizon < 0:
         assert c.us() < 1.25 * c.us(horizon=-1)
     c.net.close()
+
+
+HUBS = {
+    "about a sub-warp's passes": lambda: _hubs([12, 13, 14, 15, 16, 30, 31, 32, 62, 63, 64, 126, 127, 128], False),
+    "pieces of more than a warp": lambda: _hubs([2046, 2047, 2048, 5000, 9000, 15], False),
+    "more pieces than room": lambda: _complete(41),
+    "spilled hubs": lambda: _hubs([40] * 1200, False),
+    "rows in global memory": lambda: _hubs([700] * 100, False),
+    "spokes of one edge": lambda: _hubs([20] * 900, True),
+}
+
+
+@pytest.mark.parametrize("which", HUBS)
+def test_hub_rows(which):
+    """Stops of more edges than a sub-warp takes are shared by the block's warps: rows, status and
+    the counted build, at block sizes and lanes of every kind."""
+    tt = HUBS[which]()
+    c = _Case(tt, 60)
+    eat = c.eat
+    want, _ = oracle.csa_many(oracle.SortedConnections(tt), c.q.source, c.q.t_s, 8)
+    counters = torch.zeros((60, 7), dtype=torch.int64, device="cuda")
+    for opts in ({}, {"block": 64}, {"block": 96, "vwarp": 32}, {"block": 512, "vwarp": 1}, {"block": 1024, "vwarp": 2},
+                 {"block": 256, "horizon": 900}, {"block": 1024, "horizon": 900, "counters": counters},
+                 {"placement": eat.EAT_PLACE_GLOBAL_ARR, "block": 512}, {"placement": eat.EAT_PLACE_GLOBAL, "block": 1024},
+                 {"placement": eat.EAT_PLACE_GLOBAL_ARR, "block": 320, "horizon": 900}):
+        status = torch.full((60,), -9, dtype=torch.int32, device="cuda")
+        c.out.fill_(-7)
+        c.run(status=status, **opts)
+        assert np.array_equal(c.out.cpu().numpy(), want), list(opts.items())
+        assert not status.any()
+    reached = torch.as_tensor((want < 2**31 - 1).sum(axis=1)).cuda()
+    assert (counters[:, 6] >= reached - 1).all() and (counters[:, 2] >= counters[:, 4]).all()
+    assert np.array_equal(eat.eat_query(c.net, int(c.q.source[7]), int(c.q.t_s[7])), want[7])
+    c.net.close()
+
+
+def test_hubs_beside_other_networks():
+    """One launch and one server over networks with hubs and without."""
+    from paper_1912_00966_gb300 import eat
+    tts = [_hubs([100, 40, 16, 300], False), synth.small_grid(), _hubs([20] * 200, True), _complete(30)]
+    nets = [eat.eat_build(t.n_stops, t.u, t.v, t.dep, t.dur, device=0) for t in tts]
+    q = synth.random_queries(tts, 400, 9)
+    sizes = np.array([tts[i].n_stops for i in q.net], np.int64)
+    offs = np.concatenate([[0], np.cumsum(sizes)[:-1]])
+    want = np.concatenate([oracle.csa(oracle.SortedConnections(tts[i]), int(s), int(t))
+                           for i, s, t in zip(q.net, q.source, q.t_s)])
+    out = torch.full((int(sizes.sum()),), -7, dtype=torch.int32, device="cuda")
+    dev = [torch.as_tensor(a).cuda() for a in (q.net, q.source, q.t_s)]
+    for opts in ({}, {"block": 1024}, {"horizon": 1200}):
+        out.fill_(-7)
+        eat.eat_query_batch_multi(nets, *dev, out, torch.as_tensor(offs).cuda(), **opts)
+        assert np.array_equal(out.cpu().numpy(), want), opts
+    server = eat.Server(nets)
+    rows = np.split(np.full(int(sizes.sum()), -7, np.int32), offs[1:])
+    for k in range(400):
+        server.submit(int(q.net[k]), int(q.source[k]), int(q.t_s[k]), rows[k], k)
+    left = 400
+    while left:
+        for _, status, _, _ in server.poll(timeout_us=1000):
+            assert status == 0
+            left -= 1
+    assert np.array_equal(np.concatenate(rows), want)
+    server.close()
+    for n in nets:
+        n.close()
+
+
+def test_hub_does_not_hold_up_its_round():
+    """A ring of 40 stops, alone and with 1,000 leaves at each: with one sub-warp to a stop the leaves
+    made a round some 60 times as long; the block's threads take them in one pass."""
+    ring, hubs = _Case(_hubs([0] * 40, True), 1), _Case(_hubs([1000] * 40, True), 1)
+    for c in (ring, hubs):
+        c.q.source[0], c.q.t_s[0] = c.src[0], c.ts[0] = 0, 6 * HOUR
+        c.check()
+    assert hubs.us() < 10 * ring.us()
+    ring.net.close()
+    hubs.net.close()
