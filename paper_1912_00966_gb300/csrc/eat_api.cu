@@ -353,12 +353,12 @@ static int make_plan_core(const eat_net *const *nets, int n_nets, int32_t n, con
     const eat_net *const tuned = n_nets == 1 && why != kForRing ? nets[0] : nullptr;
     const bool own_workspace = why == kForBatch || why == kForTuner, use_tuned = why != kForTuner;
     int32_t vmax = 0, vmin = INT32_MAX, level = 0;
-    bool hubs = false;
+    bool odd = false;
     for (int i = 0; i < n_nets; ++i) {
         vmax = std::max(vmax, nets[i]->host.n_stops);
         vmin = std::min(vmin, nets[i]->host.n_stops);
         level = std::max(level, nets[i]->host.e_level);
-        hubs = hubs || wants_hubs(&nets[i]->edev, 1);
+        odd = odd || any_odd(&nets[i]->edev, 1);
     }
     DeviceInfo d;
     int rc = device_info(dev, d);
@@ -555,7 +555,7 @@ static int make_plan_core(const eat_net *const *nets, int n_nets, int32_t n, con
     int reg_blocks = 1;                       // with at most one query per SM one is all it holds
     if (n > d.sms) {
         DeviceGuard guard(dev);
-        const void *k = cta_kernel(p.nets, p.mem, p.build, false, p.horizon > 0, hubs);
+        const void *k = cta_kernel(p.nets, p.mem, p.build, false, p.horizon > 0, odd);
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&reg_blocks, k, p.block, 0) != cudaSuccess) {
             cudaGetLastError();
             reg_blocks = 0;
@@ -581,7 +581,7 @@ static int make_plan_core(const eat_net *const *nets, int n_nets, int32_t n, con
     if (n != 1) {                             // a single query: a block always fits an SM
         DeviceGuard guard(dev);
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-            &per_sm, cta_kernel(p.nets, p.mem, p.build, false, p.horizon > 0, hubs), p.block, p.smem);
+            &per_sm, cta_kernel(p.nets, p.mem, p.build, false, p.horizon > 0, odd), p.block, p.smem);
     }
     if (e != cudaSuccess) return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
     if (per_sm < 1) return fail(EAT_ERR_INVALID, "kernel does not fit on an SM with this block size");
@@ -775,11 +775,11 @@ int ring_setup(const eat_net *const *nets, int n_nets, RingLaunch &rl) {
         return fail(EAT_ERR_INVALID, "ring admission keeps the frontier bitmaps in shared memory; "
                                      "these networks are too large (use EAT_ADMIT_BATCH)");
     int per_sm = 0;
-    bool hubs = false;
-    for (int i = 0; i < n_nets; ++i) hubs = hubs || wants_hubs(&nets[i]->edev, 1);
+    bool odd = false;
+    for (int i = 0; i < n_nets; ++i) odd = odd || any_odd(&nets[i]->edev, 1);
     {
         DeviceGuard guard(nets[0]->device);
-        cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ring_kernel(p.mem, hubs),
+        cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ring_kernel(p.mem, odd),
                                                                       p.block, p.smem);
         if (e != cudaSuccess) return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
     }

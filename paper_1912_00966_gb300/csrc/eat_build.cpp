@@ -675,6 +675,8 @@ int build_edges(HostNet &h) {
         std::vector<Pair> pairs;
         std::vector<int32_t> ex;
         int64_t quads = 0;
+        std::vector<int64_t> tables;                  // first quad of each long list's table and its parts'
+        int64_t longest = 0, walk = 0;                // quads of a list; quads before a departure's own, summed
         int64_t travel = 0, wait = 0, waits = 0;      // durations; gaps between departures, their number
         bool oom = false;
     };
@@ -827,6 +829,46 @@ int build_edges(HostNet &h) {
     h.e_lanes = crowded_lanes(h);
     // Entries, with list offsets local to the part; the lists' places follow from their sizes.
     const bool big = V > kMaxPackedStops;
+    // The first of the departures q .. z - 1 as an entry's 16-bit numbers for a slot that starts
+    // at lo; returns the first one that is not among them.
+    auto inline3 = [](const Pair *q, const Pair *z, int64_t lo, int32_t *w) {
+        const Pair *m = q;
+        for (int j = 0; j < 3; ++j) {
+            uint32_t dep = (uint32_t)kNoDeparture, dur = 0;
+            if (m == q + j && m < z && m->dep - lo < kNoDeparture && m->arr - m->dep <= 0xffff) {
+                dep = (uint32_t)(m->dep - lo);
+                dur = (uint32_t)(m->arr - m->dep);
+                ++m;
+            }
+            w[j] = (int32_t)(dep | dur << 16);
+        }
+        return m;
+    };
+    // The table at quad `at` of a list (departures listed .. z - 1 from quad `list` on): an entry
+    // for each part of the slot of 2^shift seconds from lo, q its first departure.
+    auto table = [&](auto &self, Part &p, int64_t at, int64_t list, const Pair *listed, const Pair *q,
+                     const Pair *z, int64_t lo, int32_t shift) -> void {
+        p.tables.push_back(at);
+        shift -= kSubLog2;
+        for (int32_t k = 0; k < kSubSlots; ++k) {
+            const int64_t from = lo + ((int64_t)k << shift), to = from + ((int64_t)1 << shift);
+            while (q < z && q->dep < from) ++q;
+            const Pair *last = q;
+            while (last < z && last->dep < to) ++last;
+            if (last < z) ++last;
+            int32_t w[4];
+            const Pair *const m = inline3(q, last, from, w);
+            w[3] = 0;
+            if (m < last) w[3] = (int32_t)(list + (m - listed) / 4 + 1);
+            if (last - m > kLongList && shift >= kSubLog2) {
+                const int64_t sub = (int64_t)p.ex.size() / 8;
+                p.ex.resize(p.ex.size() + 4 * kSubSlots);
+                w[3] = (int32_t)-(sub + 1);
+                self(self, p, sub, list, listed, q, last, from, shift);
+            }
+            std::copy(w, w + 4, p.ex.begin() + at * 8 + 4 * k);
+        }
+    };
     auto fill = [&](Part &p) {
         const int64_t e0 = e_off[&p - parts.data()];
         int32_t u = p.u_begin;
@@ -847,40 +889,48 @@ int build_edges(HostNet &h) {
                 const Pair *z = q;
                 while (z < end && z->dep < hi) ++z;
                 if (z < end) ++z;                     // the first departure after the slot
-                uint32_t dep[3], dur[3] = {0, 0, 0};
-                const Pair *m = q;
-                for (int j = 0; j < 3; ++j) {
-                    dep[j] = (uint32_t)kNoDeparture;
-                    if (m == q + j && m < z && m->dep - lo < kNoDeparture && m->arr - m->dep <= 0xffff) {
-                        dep[j] = (uint32_t)(m->dep - lo);
-                        dur[j] = (uint32_t)(m->arr - m->dep);
-                        ++m;
-                    }
-                }
                 int32_t *w = &h.ee[((size_t)k * (size_t)E + (size_t)(e0 + (int64_t)e)) * 4];
-                for (int j = 0; j < 3; ++j) w[j] = (int32_t)(dep[j] | dur[j] << 16);
+                const Pair *const m = inline3(q, z, lo, w);
                 w[3] = 0;
                 if (m == z) continue;
-                w[3] = (int32_t)(p.quads + 1);
+                // A long list starts at a quad 7 (mod 8), its table just before; others elsewhere.
+                const bool is_long = z - m > kLongList && h.e_shift >= kSubLog2;
+                if (is_long) {
+                    while (p.ex.size() / 8 % 8 != 7) p.ex.resize(p.ex.size() + 8, EAT_INF);
+                    p.ex.resize(p.ex.size() + 4 * kSubSlots);
+                } else if (p.ex.size() / 8 % 8 == 7) {
+                    p.ex.resize(p.ex.size() + 8, EAT_INF);
+                }
+                const int64_t list = (int64_t)p.ex.size() / 8;
+                w[3] = (int32_t)(list + 1);
                 const bool open = z == end && z[-1].dep < hi;   // nothing after the slot
-                for (; m < z; ++m) p.ex.insert(p.ex.end(), {m->dep, m->arr});
+                p.longest = std::max<int64_t>(p.longest, (z - m + 3) / 4);
+                p.walk += (z - m) * (z - m) / 8;
+                for (const Pair *i = m; i < z; ++i) p.ex.insert(p.ex.end(), {i->dep, i->arr});
                 if (open) p.ex.insert(p.ex.end(), {EAT_INF, EAT_INF});
                 while (p.ex.size() % 8) p.ex.push_back(EAT_INF);
-                p.quads = (int64_t)p.ex.size() / 8;
+                if (is_long) table(table, p, list - kSubSlots / 2, list, m, q, z, lo, h.e_shift);
             }
             int32_t *w = &h.ee[((size_t)h.e_y * (size_t)E + (size_t)(e0 + (int64_t)e)) * 4];
             w[0] = w[1] = w[2] = -1;
             w[3] = 0;
         }
+        while (p.ex.size() / 8 % 8) p.ex.resize(p.ex.size() + 8, EAT_INF);
+        p.quads = (int64_t)p.ex.size() / 8;
         std::vector<Pair>().swap(p.pairs);
     };
     if (!run(fill)) return fail(EAT_ERR_OOM, "host allocation of the edge table failed");
     std::vector<int64_t> q_off((size_t)n_parts);
-    int64_t quads = 0;
+    int64_t quads = 0, longest = 0, walk = 0;
     for (int k = 0; k < n_parts; ++k) {
         q_off[k] = quads;
         quads += parts[k].quads;
+        longest = std::max(longest, parts[k].longest);
+        walk += parts[k].walk;
     }
+    // The tables pay for a build that makes every round longer where a departure is walked to
+    // over a quad or more on average, or some list is walked over many.
+    if (walk > n_pairs || longest > 32) h.e_lanes |= kLongLists;
     if (quads >= INT32_MAX) return fail(EAT_ERR_INVALID, "edge lists too large for 32-bit indices");
     try {
         h.ex.resize((size_t)quads * 8);
@@ -891,6 +941,11 @@ int build_edges(HostNet &h) {
         const size_t k = (size_t)(&p - parts.data());
         std::copy(p.ex.begin(), p.ex.end(), h.ex.begin() + q_off[k] * 8);
         if (!q_off[k]) return;
+        for (int64_t t : p.tables)
+            for (int32_t j = 0; j < kSubSlots; ++j) {
+                int32_t &x = h.ex[(size_t)(q_off[k] + t) * 8 + 4 * (size_t)j + 3];
+                if (x) x += x < 0 ? -(int32_t)q_off[k] : (int32_t)q_off[k];
+            }
         for (int32_t s = 0; s < h.e_y; ++s)
             for (size_t e = 0; e < p.head.size(); ++e) {
                 int32_t &x = h.ee[((size_t)s * (size_t)E + (size_t)e_off[k] + e) * 4 + 3];

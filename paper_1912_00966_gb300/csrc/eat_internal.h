@@ -56,14 +56,19 @@ constexpr int32_t kInlineAps = 4;
 //                edges leaving it (15 = read erow), which of them goes back to u (15 = none
 //                of the first 15), its first edge; networks of more than 2^24 stops:
 //                {v, erow[v]}, d always read from erow
-//   ee[k*E + i]  16-byte entry of edge i for slot k, slot-major (a round's lookups are at
+//   ee[k*E + i]  16-byte entry of edge i for slot k of y + 1, slot-major (the last one, for tails
+//                reached after slot y - 1, holds no departures; a round's lookups are at
 //                nearby times and fall in few slabs): the listed departures inside the slot
 //                and the first one after it, the first three as 16-bit numbers
 //                {d0 | l0 << 16, d1 | l1 << 16, d2 | l2 << 16, x}: departure d (relative to
 //                the slot's start, 0xffff = none), duration l; the others (or values that
 //                do not fit 16 bits) from ex[4 * (x - 1)] on, x = 0 if there are none
-//   ex[]         {departure, arrival} pairs, each list a multiple of four pairs (32 bytes)
-//                ended by the first departure after the slot or by {INF, INF}
+//   ex[]         {departure, arrival} pairs, each list a multiple of four pairs (32 bytes, a
+//                quad) ended by the first departure after the slot or by {INF, INF}.  A list of
+//                more than kLongList pairs, and no other, has x a multiple of 8, and its table in
+//                the 8 quads before it: 16 entries like ee's, one for each sixteenth of the slot,
+//                whose x > 0 is the quad of the list to go on from and x < 0 the table at quad
+//                -x - 1, of sixteenths again
 //   erow[V+1]    edges leaving stop u are erow[u] .. erow[u+1]-1
 // Against one 16-byte record and one 32-byte entry per (type, cluster) this reads 24 bytes
 // per edge, where an edge has two (city) or three (large) types of which half have no
@@ -72,13 +77,13 @@ constexpr int32_t kInlineAps = 4;
 constexpr int32_t kNoDeparture = 0xffff;
 constexpr int32_t kEdgeOverflow = 15;
 constexpr int32_t kMaxPackedStops = 1 << 24;
-constexpr int32_t kHubs = 4;          // in EdgeDev::lanes
+constexpr int32_t kHubs = 4, kLongLists = 8;      // in EdgeDev::lanes
 
 struct EdgeDev {
     static constexpr int32_t kUsualLanes = 2;
     const int32_t *erow;      // [V + 1]
     const int2 *er;           // [E]
-    const int4 *ee;           // [y * E], slot-major
+    const int4 *ee;           // [(y + 1) * E], slot-major
     const int2 *ex;
     const int32_t *etypes;    // [E] connection types of each edge (work counters only)
     int32_t n_stops;
@@ -88,7 +93,8 @@ struct EdgeDev {
     int32_t y;                // slots
     int32_t big;              // more than 2^24 stops: er holds no degree
     int32_t lanes;            // log2 of the lanes per stop in a crowded round; | kHubs: some stop
-                              // has kEdgeOverflow edges or more
+                              // has kEdgeOverflow edges or more; | kLongLists: long lists are
+                              // looked up through their tables
 };
 
 struct NetDev {
@@ -123,6 +129,17 @@ EAT_HD inline int32_t edge_inline(const int4 c, uint32_t rel, int32_t start) {
     const uint32_t p = rel <= (x & 0xffffu) ? x : rel <= (y & 0xffffu) ? y : z;
     const uint32_t d = p & 0xffffu;
     return rel <= d && d != (uint32_t)kNoDeparture ? (int32_t)((uint32_t)start + d + (p >> 16)) : EAT_INF;
+}
+
+// Part of a slot of 2^(shift + kSubLog2) seconds that `rel` falls into; rel and start become
+// those of the part.
+constexpr int32_t kSubLog2 = 4, kSubSlots = 1 << kSubLog2, kLongList = 8;
+
+EAT_HD inline int32_t edge_part(int32_t shift, uint32_t &rel, int32_t &start) {
+    const uint32_t k = rel >> shift;
+    rel -= k << shift;
+    start = (int32_t)((uint32_t)start + (k << shift));
+    return (int32_t)k;
 }
 
 // Up to NETS networks passed by value as a kernel parameter.

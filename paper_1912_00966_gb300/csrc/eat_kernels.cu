@@ -180,11 +180,12 @@ __device__ __forceinline__ void fill_inf(int32_t *p, int32_t n, int tid, int nth
 // 1,024-thread blocks per SM 851 against 969 for one).
 // COUNT: the build that fills qa.counters; without it the per-thread work counters are
 // dead code and compiled away (the timed launches pass no counters).  HZ: the build that
-// honours qa.horizon.  HUB: the build for networks with hubs or with lanes per stop of their own
-// (EdgeDev::lanes); the others' rounds are 5 to 25 % longer with it (20,000-stop city 256
-// queries 292 -> 307 us, 60,000 stops 300 queries 812 -> 1,015: registers).
+// honours qa.horizon.  ODD: the build for networks with hubs, long lists or lanes per stop of
+// their own (EdgeDev::lanes); the others' rounds are longer with it, for the registers (20,000-stop
+// city 256 queries 292 -> 307 us for either part, 60,000 stops 300 queries 812 -> 1,015 for hubs,
+// 200,000 stops 96 queries 961 -> 1,141 for lists).
 template <int NETS, int ARR, bool SMEM_MASK, int BUILD, bool RING = false, bool COUNT = false, bool HZ = true,
-          bool HUB = COUNT>
+          bool ODD = COUNT>
 __global__ void __launch_bounds__(BUILD == kThree512 ? 512 : 1024,
                                   BUILD == kThree512 ? 3 : BUILD == kTwo1024 ? 2 : 1)
 eat_cta_kernel(const __grid_constant__ EdgeTable<NETS> nets, const QueryArgs qa) {
@@ -268,7 +269,7 @@ eat_cta_kernel(const __grid_constant__ EdgeTable<NETS> nets, const QueryArgs qa)
         }
         const bool hz_on = HZ && qa.horizon > 0;
         if (tid < 2) s_n[tid] = 0;
-        if (HUB && tid == 0) s_hub = 0;
+        if (ODD && tid == 0) s_hub = 0;
         if (hz_on && clear_wait)
             for (int32_t i = tid; i < qa.mask_words; i += nthr) wait[i] = 0u;
         if (HZ && tid < 2) {
@@ -376,7 +377,7 @@ eat_cta_kernel(const __grid_constant__ EdgeTable<NETS> nets, const QueryArgs qa)
                     const int32_t v = big ? h.x : h.x & 0xffffff;
                     const int32_t ev = load_arr(arr, v, arr_shared);
                     int32_t cand = edge_inline(c, rel, start), seen = 3;
-                    if (__builtin_expect(cand == kInf && c.w != 0, 0)) cand = edge_list(N, c.w, e_u, seen);
+                    if (__builtin_expect(cand == kInf && c.w != 0, 0)) cand = edge_list<ODD>(N, c.w, e_u, rel, start, seen);
                     if (COUNT) {
                         c_types += __ldg(N.etypes + t);
                         ++c_lookups;
@@ -418,7 +419,7 @@ eat_cta_kernel(const __grid_constant__ EdgeTable<NETS> nets, const QueryArgs qa)
 
             // A sub-warp of 2^pl lanes per stop: `vwarp` lanes while that keeps every stop of
             // the round in one pass, else four, or what most stops of the network have edges for.
-            const int few = HUB ? N.lanes & 3 : 2;
+            const int few = ODD ? N.lanes & 3 : 2;
             const int pl = (n << qa.vw_log2) <= nthr ? qa.vw_log2 : min(qa.vw_log2, few);
             const int lane = tid & ((1 << pl) - 1);
             const int nsub = nthr >> pl;
@@ -429,7 +430,7 @@ eat_cta_kernel(const __grid_constant__ EdgeTable<NETS> nets, const QueryArgs qa)
                 const int32_t u = big ? e.x : e.x & 0xffffff;
                 const int32_t d = big ? kEdgeOverflow : (int32_t)((uint32_t)e.x >> 28);
                 if (COUNT) c_vert += lane == 0;
-                if (HUB && d == kEdgeOverflow && (N.lanes & kHubs) && hub(u, e.y, pl, lane)) continue;
+                if (ODD && d == kEdgeOverflow && (N.lanes & kHubs) && hub(u, e.y, pl, lane)) continue;
                 expand(u, e.y, d, 1 << pl, lane, back_out ? from(q_rd)[i] : 0,
                        big ? kEdgeOverflow : (int32_t)((uint32_t)e.x >> 24 & 15u));
             }
@@ -439,11 +440,11 @@ eat_cta_kernel(const __grid_constant__ EdgeTable<NETS> nets, const QueryArgs qa)
                 for (int32_t i = tid >> sl; i < n - qcap; i += nthr >> sl) {
                     const int32_t u = __ldcg(sp_rd + i), t = __ldg(N.erow + u);
                     if (COUNT) c_vert += sub == 0;
-                    if (HUB && (N.lanes & kHubs) && hub(u, t, sl, sub)) continue;
+                    if (ODD && (N.lanes & kHubs) && hub(u, t, sl, sub)) continue;
                     expand(u, t, kEdgeOverflow, 1 << sl, sub, 0, kEdgeOverflow);
                 }
             }
-            if (HUB && (N.lanes & kHubs)) {
+            if (ODD && (N.lanes & kHubs)) {
                 __syncthreads();
                 const int32_t wanted = s_hub, listed = min(wanted, pieces);
                 if (wanted > 0) {
@@ -1328,21 +1329,21 @@ eat_cluster_kernel(const __grid_constant__ NetTable<NETS> nets, const QueryArgs 
     cluster.sync();                                   // block 0 is done reading the others
 }
 
-template <int NETS, int BUILD, bool COUNT, bool HZ, bool HUB = COUNT>
+template <int NETS, int BUILD, bool COUNT, bool HZ, bool ODD = COUNT>
 static const void *cta_kernel_ptr(int mem) {
     switch (mem) {
-    case 0: return (const void *)eat_cta_kernel<NETS, kArrShared, true, BUILD, false, COUNT, HZ, HUB>;
-    case 1: return (const void *)eat_cta_kernel<NETS, kArrGlobal, true, BUILD, false, COUNT, HZ, HUB>;
-    case 3: return (const void *)eat_cta_kernel<NETS, kArrPerQuery, true, BUILD, false, COUNT, HZ, HUB>;
-    default: return (const void *)eat_cta_kernel<NETS, kArrGlobal, false, BUILD, false, COUNT, HZ, HUB>;
+    case 0: return (const void *)eat_cta_kernel<NETS, kArrShared, true, BUILD, false, COUNT, HZ, ODD>;
+    case 1: return (const void *)eat_cta_kernel<NETS, kArrGlobal, true, BUILD, false, COUNT, HZ, ODD>;
+    case 3: return (const void *)eat_cta_kernel<NETS, kArrPerQuery, true, BUILD, false, COUNT, HZ, ODD>;
+    default: return (const void *)eat_cta_kernel<NETS, kArrGlobal, false, BUILD, false, COUNT, HZ, ODD>;
     }
 }
 
 template <int NETS>
-static const void *cta_kernel_for(int mem, int build, bool count, bool hz, bool hubs) {
+static const void *cta_kernel_for(int mem, int build, bool count, bool hz, bool odd) {
     // These honour a horizon, if there is one.
     if (count) return cta_kernel_ptr<NETS, kOne1024, true, true>(mem);
-    if (hubs)
+    if (odd)
         return build == kThree512  ? cta_kernel_ptr<NETS, kThree512, false, true, true>(mem)
                : build == kTwo1024 ? cta_kernel_ptr<NETS, kTwo1024, false, true, true>(mem)
                                    : cta_kernel_ptr<NETS, kOne1024, false, true, true>(mem);
@@ -1356,12 +1357,12 @@ static const void *cta_kernel_for(int mem, int build, bool count, bool hz, bool 
     }
 }
 
-const void *cta_kernel(int nets, int mem, int build, bool count, bool hz, bool hubs) {
-    return nets == 1 ? cta_kernel_for<1>(mem, build, count, hz, hubs)
-                     : cta_kernel_for<EAT_MAX_NETS>(mem, build, count, hz, hubs);
+const void *cta_kernel(int nets, int mem, int build, bool count, bool hz, bool odd) {
+    return nets == 1 ? cta_kernel_for<1>(mem, build, count, hz, odd)
+                     : cta_kernel_for<EAT_MAX_NETS>(mem, build, count, hz, odd);
 }
 
-bool wants_hubs(const EdgeDev *nets, int n_nets) {
+bool any_odd(const EdgeDev *nets, int n_nets) {
     bool any = false;
     for (int i = 0; i < n_nets; ++i) any = any || nets[i].lanes != EdgeDev::kUsualLanes;
     return any;
@@ -1414,27 +1415,27 @@ static cudaError_t launch_cta_t(const void *kernel, const EdgeDev *nets, int n_n
 cudaError_t launch_cta(const EdgeDev *nets, int n_nets, const QueryArgs &qa, int mem, int build, int grid,
                        int block, size_t smem, cudaStream_t st) {
     const void *k = cta_kernel(n_nets == 1 ? 1 : EAT_MAX_NETS, mem, build, qa.counters != nullptr, qa.horizon > 0,
-                               wants_hubs(nets, n_nets));
+                               any_odd(nets, n_nets));
     return n_nets == 1 ? launch_cta_t<1>(k, nets, n_nets, qa, grid, block, smem, st)
                        : launch_cta_t<EAT_MAX_NETS>(k, nets, n_nets, qa, grid, block, smem, st);
 }
 
-template <bool HUB>
+template <bool ODD>
 static const void *ring_kernel_ptr(int mem) {
     switch (mem) {
-    case 0: return (const void *)eat_cta_kernel<EAT_MAX_NETS, kArrShared, true, kThree512, true, false, false, HUB>;
-    case 3: return (const void *)eat_cta_kernel<EAT_MAX_NETS, kArrPerQuery, true, kThree512, true, false, false, HUB>;
-    default: return (const void *)eat_cta_kernel<EAT_MAX_NETS, kArrGlobal, true, kThree512, true, false, false, HUB>;
+    case 0: return (const void *)eat_cta_kernel<EAT_MAX_NETS, kArrShared, true, kThree512, true, false, false, ODD>;
+    case 3: return (const void *)eat_cta_kernel<EAT_MAX_NETS, kArrPerQuery, true, kThree512, true, false, false, ODD>;
+    default: return (const void *)eat_cta_kernel<EAT_MAX_NETS, kArrGlobal, true, kThree512, true, false, false, ODD>;
     }
 }
 
-const void *ring_kernel(int mem, bool hubs) {
-    return hubs ? ring_kernel_ptr<true>(mem) : ring_kernel_ptr<false>(mem);
+const void *ring_kernel(int mem, bool odd) {
+    return odd ? ring_kernel_ptr<true>(mem) : ring_kernel_ptr<false>(mem);
 }
 
 cudaError_t launch_ring(const EdgeDev *nets, int n_nets, const QueryArgs &qa, int mem, int grid,
                         int block, size_t smem, cudaStream_t st) {
-    return launch_cta_t<EAT_MAX_NETS>(ring_kernel(mem, wants_hubs(nets, n_nets)), nets, n_nets, qa, grid, block, smem, st);
+    return launch_cta_t<EAT_MAX_NETS>(ring_kernel(mem, any_odd(nets, n_nets)), nets, n_nets, qa, grid, block, smem, st);
 }
 
 const void *pair_kernel(bool count) {

@@ -83,16 +83,16 @@ struct QueryArgs {
 // build: kThree512 for blocks of up to 512 threads, kOne1024 or kTwo1024 (per SM) for larger.
 // count: the instantiation that fills qa.counters (launch_cta picks it when counters are
 // given); hz: the one that honours qa.horizon (launch_cta picks it when qa.horizon > 0).
-// hubs: the one for networks of which wants_hubs() says so (launch_cta asks it).
-const void *cta_kernel(int nets, int mem, int build, bool count = false, bool hz = false, bool hubs = false);
-bool wants_hubs(const EdgeDev *nets, int n_nets);
+// odd: the one for networks of which any_odd() says so (launch_cta asks it).
+const void *cta_kernel(int nets, int mem, int build, bool count = false, bool hz = false, bool odd = false);
+bool any_odd(const EdgeDev *nets, int n_nets);
 cudaError_t launch_cta(const EdgeDev *nets, int n_nets, const QueryArgs &qa, int mem, int build, int grid,
                        int block, size_t smem, cudaStream_t st);
 // Ring mode of the per-query kernel (serving): persistent blocks take requests from
 // qa.rg until the host's stop flag is set and no request is left, or until they find
 // none for rg.idle_iters polls; mem 0, 1 or 3; rows go to arr_out + row * row_stride,
 // arrivals not in shared memory live in the block's arr_rows row meanwhile.
-const void *ring_kernel(int mem, bool hubs);
+const void *ring_kernel(int mem, bool odd);
 cudaError_t launch_ring(const EdgeDev *nets, int n_nets, const QueryArgs &qa, int mem, int grid,
                         int block, size_t smem, cudaStream_t st);
 // Asynchronous (round-free) kernel; mem 0, 1 or 3 as above (bitmap always shared).

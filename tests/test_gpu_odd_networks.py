@@ -204,3 +204,56 @@ def test_hub_does_not_hold_up_its_round():
     assert hubs.us() < 10 * ring.us()
     ring.net.close()
     hubs.net.close()
+
+
+def _with_extra(tt, day):
+    """One more departure, `day` days on: the slots of the whole network get longer."""
+    c = [np.append(a, b).astype(np.int32) for a, b in
+         ((tt.u, tt.u[0]), (tt.v, tt.v[0]), (tt.dep, 86400 * day), (tt.dur, tt.dur[0]))]
+    z = np.zeros(c[0].shape[0], np.int32)
+    return synth.Timetable("extra", tt.n_stops, *c, z, z)
+
+
+def _metro(headway):
+    """A line of 60 stops served every `headway` seconds both ways, in a net of rare connections."""
+    rng = np.random.default_rng(headway)
+    u = np.repeat(np.arange(6000), 3)
+    key = np.unique(np.concatenate([u * 6000 + (u + rng.integers(1, 6000, u.shape[0])) % 6000,
+                                    np.arange(59) * 6001 + 1, np.arange(1, 60) * 6001 - 1]))
+    busy = np.abs(key // 6000 - key % 6000) == 1
+    busy &= (key // 6000 < 60) & (key % 6000 < 60)
+    return _service(6000, key // 6000, key % 6000, rng.integers(60, 900, key.shape[0]),
+                    np.where(busy, headway, 4 * HOUR), headway)
+
+
+@pytest.mark.parametrize("make", [lambda: _metro(60), lambda: _metro(7),
+                                  lambda: _with_extra(synth.small_grid(), 20),
+                                  lambda: _with_extra(synth.small_grid(), 3000)])
+def test_long_list_rows(make):
+    """Long lists of departures through their tables, one to three levels deep."""
+    tt = make()
+    c = _Case(tt, 200)
+    eat = c.eat
+    want, _ = oracle.csa_many(oracle.SortedConnections(tt), c.q.source, c.q.t_s, 8)
+    counters = torch.zeros((200, 7), dtype=torch.int64, device="cuda")
+    for opts in ({}, {"block": 512, "horizon": 1800}, {"block": 1024, "counters": counters},
+                 {"placement": eat.EAT_PLACE_GLOBAL_ARR, "block": 512},
+                 {"placement": eat.EAT_PLACE_GLOBAL_ARR, "block": 1024, "horizon": 7200},
+                 {"placement": eat.EAT_PLACE_GLOBAL}):
+        c.out.fill_(-7)
+        c.run(**opts)
+        assert np.array_equal(c.out.cpu().numpy(), want), list(opts.items())
+    c.net.close()
+
+
+@pytest.mark.parametrize("n", [1, 300])
+def test_one_far_departure_costs_little(n):
+    """A city and the same city with one departure 30 days on: walked from their start, the lists that
+    its longer slots bring took three times as long."""
+    plain, far = _Case(synth.city(), n), _Case(_with_extra(synth.city(), 30), n)
+    for c in (plain, far):
+        c.run()
+    assert torch.equal(plain.out, far.out)
+    assert far.us() < 2 * plain.us()
+    plain.net.close()
+    far.net.close()
