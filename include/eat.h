@@ -381,7 +381,8 @@ int eat_query(const eat_net *net, int32_t s, int32_t t_s, int32_t *arr_out,
 
 /*
  * eat_workspace_bytes -- device workspace needed by eat_query_batch(_multi) for
- * n queries over the given networks with these options (opts may be NULL).
+ * n queries over the given networks with these options (opts may be NULL).  Unless the
+ * launch shape of some batch size was tuned, it also holds any smaller batch.
  * Returns 0 on invalid arguments.
  */
 size_t eat_workspace_bytes(const eat_net *const *nets, int32_t n_nets, int32_t n,

@@ -586,9 +586,11 @@ static int make_plan_core(const eat_net *const *nets, int n_nets, int32_t n, con
     if (e != cudaSuccess) return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
     if (per_sm < 1) return fail(EAT_ERR_INVALID, "kernel does not fit on an SM with this block size");
     p.grid = (int)std::min<int64_t>((int64_t)std::max(n, 1), (int64_t)per_sm * d.sms);
-    // With a horizon a block also keeps the bitmap of waiting stops.
-    p.spill_stride = p.horizon > 0 ? (int64_t)align_up((size_t)vmax * 2 + (size_t)p.mask_words, 64)
-                                   : (int64_t)align_up((size_t)vmax * 2, 64);
+    // With a horizon a block also keeps the bitmap of waiting stops.  In a workspace of the
+    // call's own it has room in any case, since the automatic horizon comes and goes with n: a
+    // workspace for n queries then holds fewer as well.
+    p.spill_stride = p.horizon > 0 || own_workspace ? (int64_t)align_up((size_t)vmax * 2 + (size_t)p.mask_words, 64)
+                                                    : (int64_t)align_up((size_t)vmax * 2, 64);
     p.mask_stride = p.mem == 2 ? (int64_t)align_up(2 * (size_t)p.mask_words, 64) : 0;
     p.off_spill = kWsHeader;
     p.off_mask = p.off_spill + (size_t)p.grid * (size_t)p.spill_stride * 4;

@@ -257,3 +257,23 @@ def test_one_far_departure_costs_little(n):
     assert far.us() < 2 * plain.us()
     plain.net.close()
     far.net.close()
+
+
+@pytest.mark.parametrize("which", ["grid", "city", "city, rows alone on an SM", "complete", "several"])
+def test_workspace_holds_smaller_batches(which):
+    """A program sizes one workspace for its largest batch: no smaller one needs more, whatever
+    shape and horizon its size gets."""
+    from paper_1912_00966_gb300 import eat
+    geometric = lambda n: synth.transit.geometric_timetable(n, 4, n // 200, (30, 60), (5, 20), 0.2,
+                                                            synth.transit.PEAK_BANDS, 5)
+    tts = {"grid": [synth.small_grid()], "city": [geometric(10000)], "city, rows alone on an SM": [geometric(35000)],
+           "complete": [_complete(200)], "several": [synth.small_grid(), geometric(9000)]}[which]
+    nets = [eat.eat_build(t.n_stops, t.u, t.v, t.dep, t.dur, device=0) for t in tts]
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    for opts in ({}, {"block": 512}, {"max_rounds": 9}):
+        need = [eat.eat_workspace_bytes(nets if len(nets) > 1 else nets[0], n, **opts) for n in range(1, 9 * sms, 3)]
+        assert need[0] > 0 and need == sorted(need), opts
+        need = [eat.eat_workspace_bytes(nets if len(nets) > 1 else nets[0], n, **opts) for n in range(sms - 3, 2 * sms)]
+        assert need == sorted(need), opts
+    for n in nets:
+        n.close()
