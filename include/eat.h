@@ -214,8 +214,8 @@ typedef struct {
                                 1,000 s or less with the wait, more where rounds are
                                 heavy), two hours when the arrivals are in global memory and four
                                 hours in shared memory for batches of two queries or more
-                                (from one to 1.125 queries per SM only where stops have 2.6
-                                edges or more); none otherwise and in
+                                (for one query per SM, or one more, only where stops have
+                                2.6 edges or more); none otherwise and in
                                 eat_query_batch_noalloc); < 0 = none; > 0 with
                                 EAT_MODE_PAIR, EAT_MODE_ASYNC or EAT_MODE_CLUSTER is
                                 EAT_ERR_INVALID */

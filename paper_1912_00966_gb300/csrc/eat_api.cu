@@ -505,13 +505,14 @@ static int make_plan_core(const eat_net *const *nets, int n_nets, int32_t n, con
     // 3,000-stop grid, 300 queries 105 -> 119 us with four hours): two hours with arrivals in
     // global memory (200,000 stops, 96 queries 2,960 -> 1,600; one hour and four hours within
     // 7 %), four hours in shared memory (20,000-stop city, 37 queries 268 -> 224, 256 queries
-    // 390 -> 287) for all but a single query, which gains nothing, and batches of about one
-    // query per SM, which keep the shape that is documented for them unless stops have 2.6
-    // edges or more (30,000 stops with 2.7, 160 queries 888 -> 468).
+    // 390 -> 287) for all but a single query, which gains nothing.  Batches of one query per SM
+    // and of one more have none unless stops have 2.6 edges or more (30,000 stops with 2.7,
+    // 160 queries 888 -> 468): their shape is laid down (test_launch_shape_defaults), although
+    // a horizon is faster there as at every size around (city 152 queries 320 -> 250).
     int32_t automatic = 0;
     if (own_workspace && branching && !(o && o->max_rounds > 0)) {
-        const bool one_each = n >= d.sms && n <= d.sms + d.sms / 8;
-        automatic = p.mem != 0 ? 7200 : n > 1 && (!one_each || tuned->branching > 1) ? 14400 : 0;
+        const bool laid_down = n == d.sms || n == d.sms + 1;
+        automatic = p.mem != 0 ? 7200 : n > 1 && (!laid_down || tuned->branching > 1) ? 14400 : 0;
         // Where a connection takes long, a horizon holds few of them and moves in nearly every
         // round (us without / with it, 300 queries: 60,000-stop full grid, 1-hour connections
         // every three hours 182 / 417, 15-minute ones every 15 minutes 462 / 565; 2,000 stops

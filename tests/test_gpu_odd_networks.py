@@ -277,3 +277,15 @@ def test_workspace_holds_smaller_batches(which):
         assert need == sorted(need), opts
     for n in nets:
         n.close()
+
+
+def test_horizon_around_one_query_per_sm():
+    """The automatic horizon holds for batches of a little more than one query per SM as for others:
+    without it they took 25 % longer than batches just below and above."""
+    tt = synth.transit.geometric_timetable(10000, 4, 200, (30, 60), (5, 20), 0.2, synth.transit.PEAK_BANDS, 6)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    c = _Case(tt, sms + 8)
+    for n in (2, sms - 1, sms + 2, sms + 8, sms + sms // 8, 2 * sms):
+        assert c.eat.eat_launch_shape(c.net, n)["horizon"] == 14400, n
+    c.check()
+    c.net.close()
