@@ -178,9 +178,9 @@ typedef struct {
                                 from 8,192 stops on, else 512, and for fuller batches 128
                                 to 1024 by the network's size and the batch's; 384 to 1024
                                 over several networks);
-                                else 64..1024, multiple of 32.  In an automatic block on a
-                                small network the threads that its rounds cannot fill leave
-                                at once */
+                                else 64..1024, multiple of 32.  In a block of the automatic
+                                size, asked for or not, the threads that a small network's
+                                rounds cannot fill leave at once */
     int32_t vwarp;           /* lanes per active stop (1, 2, 4, 8, 16 or 32), at most four of
                                 them in rounds with more stops than the block has
                                 sub-warps; 0 = automatic (8) */

@@ -525,13 +525,14 @@ static int make_plan_core(const eat_net *const *nets, int n_nets, int32_t n, con
         if (h.e_travel > automatic || (h.e_travel + h.e_wait > 1000 && !heavy)) automatic = 0;
     }
     p.horizon = oh > 0 ? oh : oh < 0 ? 0 : tb ? th : automatic;
-    // Threads at work in a default-shaped block (the others leave): no more than the rounds
+    // Threads at work in a block of the automatic size, asked for or not, so that a shape read
+    // back from eat_launch_shape or a tuner runs as it did (the others leave): no more than the rounds
     // of a small network fill (1,024 stops, 256 queries: 128 of 512 threads 62 us, all 69;
     // 16,000 stops, 100 queries: 512 157, 1,024 187), unless a level of the network has more
     // edges than that (HostNet::e_level): all (300 stops joined each to each, one query: 128 of
     // 1,024 threads 426 us, all 130; 2,000 joined at random 70 and 34).
     p.active = p.block;
-    if (!(o && o->block) && !tb && p.mem == 0) {
+    if (p.block == block && p.mem == 0) {
         const int few = vmax < 2048 ? 128 : vmax < 6144 ? 256 : vmax <= kFewStops ? 512 : 1024;
         if (level <= few) p.active = std::min(p.block, few);
     }

@@ -289,3 +289,14 @@ def test_horizon_around_one_query_per_sm():
         assert c.eat.eat_launch_shape(c.net, n)["horizon"] == 14400, n
     c.check()
     c.net.close()
+
+
+def test_shape_read_back_runs_alike():
+    """A call with the shape that eat_launch_shape reports takes the time of the automatic call: the
+    threads that a small network's rounds cannot fill leave either way."""
+    tt = synth.grid_timetable(16000, 800, 77, force_stop0=False)
+    c = _Case(tt, 100)
+    shape = c.eat.eat_launch_shape(c.net, 100)
+    assert c.us(**shape) < 1.1 * c.us()
+    c.check(**shape)
+    c.net.close()
