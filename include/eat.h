@@ -466,8 +466,8 @@ int eat_next_departure(const eat_net *net, const int32_t *types, const int32_t *
  * eat_autotune -- choose the launch shape for this network by measurement (no
  * counterpart in the paper, which fixes one thread per type or per edge and
  * sweeps the virtual-warp size by hand, Section IV-B).  Candidates, in this
- * order: the automatic shape's block size first if it is one of 1024, 512 and 256
- * threads, then the others of these, each with the round-based mode and vwarp 8, 4
+ * order: the automatic shape's block size first, then the others of 1024, 512 and 256
+ * threads, each with the round-based mode and vwarp 8, 4
  * and 16 lanes per stop and with the asynchronous mode, without a horizon; when n
  * exceeds the SM count, the paired mode with vwarp 8, 4 and 16; and the round-based
  * mode with each block size, vwarp 8 and horizons of 1, 2, 4 and 12 hours, which come
@@ -499,7 +499,8 @@ int eat_autotune(eat_net *net, const int32_t *sources, const int32_t *times, int
  * the round-based mode and vwarp 8, 4, 16, then the
  * asynchronous mode; then the round-based mode with 512
  * threads, vwarp 8, start by t_s and horizons of 2 and 12 hours (the others run with
- * none); shapes without a plan for these networks are skipped.  They run on
+ * none); then the automatic shape's block size if it is another, with vwarp 8; shapes
+ * without a plan for these networks are skipped.  They run on
  * the sample batch (net_idx, sources, times: [n] int32 device memory; rows packed in
  * query order in a scratch buffer) and are timed as eat_autotune times them (nine rounds,
  * cold L2, median, earliest within 5 % wins).  Nothing is stored in the networks: the

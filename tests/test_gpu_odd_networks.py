@@ -300,3 +300,36 @@ def test_shape_read_back_runs_alike():
     assert c.us(**shape) < 1.1 * c.us()
     c.check(**shape)
     c.net.close()
+
+
+def test_tuned_is_not_slower_than_automatic():
+    """The tuners can choose the automatic shape: 64 networks of uneven size, and one small one."""
+    from paper_1912_00966_gb300 import eat
+    tts = synth.ragged_grids(64)
+    nets = [eat.eat_build(t.n_stops, t.u, t.v, t.dep, t.dur, device=0) for t in tts]
+    q = synth.random_queries(tts, 4096, 3)
+    sizes = np.array([tts[i].n_stops for i in q.net], np.int64)
+    offs = torch.as_tensor(np.concatenate([[0], np.cumsum(sizes)[:-1]])).cuda()
+    dev = [torch.as_tensor(a).cuda() for a in (q.net, q.source, q.t_s)]
+    out = torch.empty(int(sizes.sum()), dtype=torch.int32, device="cuda")
+
+    def us(**opts):
+        times = []
+        for _ in range(12):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            eat.eat_query_batch_multi(nets, *dev, out, offs, **opts)
+            b.record()
+            b.synchronize()
+            times.append(1e3 * a.elapsed_time(b))
+        return float(np.median(times[3:]))
+
+    automatic, shape = us(), eat.eat_autotune_multi(nets, *dev)
+    assert us(**shape) < 1.08 * automatic, shape
+    for n in nets:
+        n.close()
+    small = _Case(synth.grid_timetable(3000, 147, 78, force_stop0=False), 1024)
+    automatic = small.us()
+    shape = eat.eat_autotune(small.net, small.src, small.ts)
+    assert small.us() < 1.08 * automatic, shape
+    small.net.close()
