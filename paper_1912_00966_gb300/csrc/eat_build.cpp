@@ -665,7 +665,7 @@ static int32_t crowded_lanes(const HostNet &h) {
 
 // Edge table (see EdgeDev in eat_internal.h): per edge the merged departures of all its
 // connection types without dominated ones, cut into time slots of 2^shift seconds.
-int build_edges(HostNet &h) {
+static int fill_edges(HostNet &h) {
     const int32_t V = h.n_stops, W = h.width, t0 = h.t0;
     struct Pair { int32_t dep, arr; };
     struct Part {
@@ -706,7 +706,9 @@ int build_edges(HostNet &h) {
             }
         };
         std::vector<std::thread> th;
-        for (unsigned i = 1; i < hw; ++i) th.emplace_back(work);
+        try {
+            for (unsigned i = 1; i < hw; ++i) th.emplace_back(work);
+        } catch (const std::exception &) {}           // no more threads to be had: fewer
         work();
         for (auto &t : th) t.join();
         for (const Part &p : parts)
@@ -953,6 +955,18 @@ int build_edges(HostNet &h) {
             }
     });
     return EAT_OK;
+}
+
+int build_edges(HostNet &h) {
+    try {
+        return fill_edges(h);
+    } catch (const std::bad_alloc &) {
+    }
+    try {
+        return fail(EAT_ERR_OOM, "host allocation of the edge table failed");
+    } catch (const std::bad_alloc &) {                // not even of the message
+        return EAT_ERR_OOM;
+    }
 }
 
 }  // namespace eat

@@ -1,4 +1,4 @@
-"""CPU: lookups on edges that are far busier than the rest of their network."""
+"""CPU: the edge table on uneven timetables, and without threads or memory to build it."""
 import os
 import subprocess
 
@@ -9,14 +9,18 @@ from paper_1912_00966_gb300 import build as libbuild
 HERE = os.path.dirname(os.path.abspath(__file__))
 
 
-@pytest.fixture(scope="module")
-def program(tmp_path_factory):
-    exe = str(tmp_path_factory.mktemp("edge_lists") / "edge_lists")
+def _compiled(folder, name):
+    exe = str(folder / name)
     subprocess.run(["g++", "-O1", "-std=c++17", "-pthread", "-I", libbuild.INCLUDE, "-I", libbuild.CSRC,
                     "-I", os.path.join(libbuild.CUDA_HOME, "include"),
-                    os.path.join(HERE, "c", "edge_lists.cpp"),
-                    os.path.join(libbuild.CSRC, "eat_build.cpp"), "-o", exe], check=True)
+                    os.path.join(HERE, "c", name + ".cpp"),
+                    os.path.join(libbuild.CSRC, "eat_build.cpp"), "-o", exe, "-ldl"], check=True)
     return exe
+
+
+@pytest.fixture(scope="module")
+def program(tmp_path_factory):
+    return _compiled(tmp_path_factory.mktemp("edge_lists"), "edge_lists")
 
 
 @pytest.mark.parametrize("stops,rare,headway,days,extra", [
@@ -34,3 +38,9 @@ def test_busy_edges(program, stops, rare, headway, days, extra, seed):
     r = subprocess.run([program, *map(str, (seed, stops, rare, headway, days, extra))],
                        capture_output=True, text=True)
     assert r.returncode == 0, r.stdout + r.stderr
+
+
+def test_built_without_threads_or_memory(tmp_path):
+    """A thread that cannot be started is done without, an allocation that fails is EAT_ERR_OOM."""
+    r = subprocess.run([_compiled(tmp_path, "edge_limits")], capture_output=True, text=True)
+    assert r.returncode == 0, (r.returncode, r.stdout + r.stderr)
