@@ -519,10 +519,13 @@ static int make_plan_core(const eat_net *const *nets, int n_nets, int32_t n, con
         // joined at random, 22-hour ones 33 / 115; streets: 10 minutes).  Up to 1,000 s a
         // connection, then; or where rounds have more work than threads, so that fewer
         // expansions outweigh more rounds (20,000 stops joined at random, 15-minute ones every
-        // three hours 360 / 266), unless it does not hold one (22-hour ones 50 / 110).
+        // three hours 360 / 266), as long as it holds more than half a connection or so: 22-hour
+        // ones 50 / 110; with a few departures a day a query ends after some rounds (200,000
+        // stops, gaps of six hours 85 / 135, of three 1,239 / 1,067 on 60,000).
         const HostNet &h = tuned->host;
         const bool heavy = h.e_level > 512 && (int64_t)h.n_edges >= 16384;
-        if (h.e_travel > automatic || (h.e_travel + h.e_wait > 1000 && !heavy)) automatic = 0;
+        const int64_t each = (int64_t)h.e_travel + h.e_wait;
+        if (h.e_travel > automatic || each > (heavy ? 7 * (int64_t)automatic / 4 : 1000)) automatic = 0;
     }
     p.horizon = oh > 0 ? oh : oh < 0 ? 0 : tb ? th : automatic;
     // Threads at work in a block of the automatic size, asked for or not, so that a shape read

@@ -678,6 +678,7 @@ static int fill_edges(HostNet &h) {
         std::vector<int64_t> tables;                  // first quad of each long list's table and its parts'
         int64_t longest = 0, walk = 0;                // quads of a list; quads before a departure's own, summed
         int64_t travel = 0, wait = 0, waits = 0;      // durations; gaps between departures, their number
+        int64_t single = 0;                           // edges of one departure
         bool oom = false;
     };
     const unsigned hw = std::max(1u, std::min(32u, std::thread::hardware_concurrency()));
@@ -755,6 +756,7 @@ static int fill_edges(HostNet &h) {
                 for (size_t m = keep; m < all.size(); ++m) p.travel += all[m].arr - all[m].dep;
                 p.wait += (int64_t)all.back().dep - all[keep].dep;
                 p.waits += (int64_t)(all.size() - keep) - 1;
+                p.single += all.size() - keep == 1;
                 p.ptr.push_back((int64_t)p.pairs.size());
                 p.head.push_back(head(ts[i]));
                 p.types.push_back((int32_t)(j - i));
@@ -765,7 +767,7 @@ static int fill_edges(HostNet &h) {
     });
     if (!ok) return fail(EAT_ERR_OOM, "host allocation of the edge table failed");
 
-    int64_t E = 0, n_pairs = 0, travel = 0, wait = 0, waits = 0;
+    int64_t E = 0, n_pairs = 0, travel = 0, wait = 0, waits = 0, single = 0;
     int32_t first = EAT_INF, last = INT32_MIN;
     std::vector<int64_t> e_off((size_t)n_parts);
     for (int k = 0; k < n_parts; ++k) {
@@ -775,13 +777,15 @@ static int fill_edges(HostNet &h) {
         travel += parts[k].travel;
         wait += parts[k].wait;
         waits += parts[k].waits;
+        single += parts[k].single;
         for (size_t e = 0; e < parts[k].head.size(); ++e) {
             first = std::min(first, parts[k].pairs[(size_t)parts[k].ptr[e]].dep);
             last = std::max(last, parts[k].pairs[(size_t)parts[k].ptr[e + 1] - 1].dep);
         }
     }
     h.e_travel = n_pairs ? (int32_t)(travel / n_pairs) : 0;
-    h.e_wait = waits ? (int32_t)(wait / waits) / 2 : 0;
+    if (E) wait += single * ((int64_t)last - first + 1);      // a gap of the whole timetable
+    h.e_wait = E ? (int32_t)std::min<int64_t>(wait / (waits + single) / 2, EAT_INF) : 0;
     h.e_base = E ? first : 0;
     h.e_shift = 0;
     h.e_y = 0;

@@ -32,11 +32,11 @@ def _complete(n):
                     rng.integers(3, 6, u.shape[0]) * HOUR, n)
 
 
-def _random(n, degree):
+def _random(n, degree, headway=300):
     rng = np.random.default_rng(n)
     u = np.repeat(np.arange(n), degree)
     key = np.unique(u * n + (u + rng.integers(1, n, u.shape[0])) % n)
-    return _service(n, key // n, key % n, rng.integers(60, 600, key.shape[0]), 300, n)
+    return _service(n, key // n, key % n, rng.integers(60, 600, key.shape[0]), headway, n)
 
 
 def _hubs(degrees, leaves, seed=1):
@@ -103,12 +103,15 @@ def test_threads_fit_the_rounds(make, n):
 
 @pytest.mark.parametrize("net,horizon", [
     ("city", 14400), ("random, 10 minutes", 14400),
-    ("random, 22 hours", -1), ("grid, 1 hour every three", -1)])
+    ("random, 22 hours", -1), ("grid, 1 hour every three", -1), ("random, twice a day", -1),
+    ("random, once a day", -1)])
 def test_horizon_where_it_holds_many_connections(net, horizon):
     """An automatic horizon is for connections that are short beside it: with long or rare ones it
     moves in nearly every round."""
     if net == "city":
         tt = synth.city()
+    elif net.endswith("a day"):
+        tt = _random(60000, 3, (12 if "twice" in net else 24) * HOUR)
     elif net.startswith("random"):
         long = net.endswith("hours")
         t = _random(2000, 4)
