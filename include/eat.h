@@ -83,7 +83,10 @@ enum eat_subtrips {
 
 /* Build options.  Zero-initialise for the paper's defaults. */
 typedef struct {
-    int32_t cluster_width; /* seconds per cluster, 1..65535; 0 = 3600 (Section II-D) */
+    int32_t cluster_width; /* seconds per cluster, 1..65535; 0 = 3600 (Section II-D).  What
+                              the paired, round-free, cluster and topology-driven modes look
+                              up; the round-based modes read time slots whose length follows
+                              the timetable's headways */
     int32_t t0;            /* start of cluster 0; departures must be >= t0; default 0 */
     int32_t device;        /* CUDA device ordinal; -1 = host-only build (inspection only) */
     int32_t subtrips;      /* EAT_SUBTRIPS_*; needs conn->trip */
@@ -158,7 +161,9 @@ typedef struct {
                           round-based modes (EAT_MODE_CTA, EAT_MODE_EDGE), one per type
                           (Section II-D) in the others; types >= lookups >= evals.
                           An edge back to the stop an arrival came from may be left
-                          out (it cannot lower that stop), with its types */
+                          out (it cannot lower that stop), with its types: in launches
+                          with rows in global memory and several blocks per SM, so that
+                          counts of one query differ with the launch shape */
     int64_t aps;       /* departures (round-based modes) or AP records (Algorithm 6)
                           examined by the lookups */
     int64_t relaxed;   /* relaxations that lowered e[v] (Algorithm 3): candidates below
@@ -441,8 +446,9 @@ int eat_query_batch(const eat_net *net, const int32_t *sources, const int32_t *t
  *                the query arrays are host memory (then staged and copied back).
  * Asynchronous on `stream` when every buffer is device memory, else returns
  * after the rows are in arr_out.  One launch serves all queries: networks whose
- * arrival row fits half an SM's shared memory keep it there, larger ones use
- * their output row.  Other arguments as eat_query_batch.
+ * arrival row fits the share of an SM's shared memory that the launch's blocks leave
+ * each other (all of it for small batches, down to a fifth for large ones) keep it there,
+ * larger ones use their output row.  Other arguments as eat_query_batch.
  */
 #define EAT_MAX_NETS 128
 int eat_query_batch_multi(const eat_net *const *nets, int32_t n_nets, const int32_t *net_idx,
@@ -640,7 +646,7 @@ void eat_server_destroy(eat_server *sv);
  *     (rounded up) for its frontier queue, plus n_stops / 4 bytes when the frontier
  *     bitmaps live in global memory (networks beyond about 900,000 stops), or
  *     16 * n_stops bytes in the paired mode (two queries per block); with a
- *     horizon, 16 * n_stops + n_stops / 8 bytes; the
+ *     horizon 16 * n_stops + n_stops / 8 bytes are set aside for it; the
  *     round-free mode needs none.  So the network may have at most 2,000,000 stops
  *     (about 1,000,000 with a horizon), and on large networks fewer blocks run at
  *     once while the other queries wait in the same launch.  Larger networks are

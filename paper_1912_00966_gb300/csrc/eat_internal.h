@@ -73,7 +73,8 @@ constexpr int32_t kInlineAps = 4;
 // Against one 16-byte record and one 32-byte entry per (type, cluster) this reads 24 bytes
 // per edge, where an edge has two (city) or three (large) types of which half have no
 // departure left: a large query of a 1,024-query step looks up 65,000 edges instead of
-// 194,000 types, and the table takes 2.0 GB instead of 5.1 GB.
+// 194,000 types.  The table takes 2.0 GB beside the 5.1 GB of per-type entries, which the other
+// modes read.
 constexpr int32_t kNoDeparture = 0xffff;
 constexpr int32_t kEdgeOverflow = 15;
 constexpr int32_t kMaxPackedStops = 1 << 24;

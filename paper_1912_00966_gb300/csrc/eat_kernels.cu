@@ -28,7 +28,8 @@
 // and several blocks per SM also the arrival it was queued with), and the next round
 // gives each queued stop a sub-warp (Section II-F's virtual warps) whose lanes take its
 // edges.  Per lane: the queue entry and e[u] (the same for the sub-warp), the edge's 8-byte
-// record, then the 16-byte entry of e[u]'s slot beside e[v].  Queue entries past the shared
+// record, then the 16-byte entry of e[u]'s slot beside e[v].  A stop of many more edges than
+// its lanes (a hub) is shared by the block's warps.  Queue entries past the shared
 // buffer spill to global memory.
 //
 // Horizon (qa.horizon > 0, an option; not in the paper): Algorithms 4-5 expand every
@@ -389,9 +390,9 @@ eat_cta_kernel(const __grid_constant__ EdgeTable<NETS> nets, const QueryArgs qa)
             };
 
             // A hub, a stop of more edges than its sub-warp of 2^pl lanes takes in four passes, is
-            // listed in pieces of whole warps, as many as the block has at most, behind the
-            // spilled stops (whose buffer holds every stop twice over the rounds); the warps
-            // share the pieces once the queue is done.  One sub-warp alone kept the round
+            // listed in pieces of whole warps, as many as the block has at most, from the end of
+            // the buffer that holds last round's spilled stops (n - qcap of its vmax words); the
+            // warps share the pieces once the queue is done.  One sub-warp alone kept the round
             // waiting: 10 hubs of 2,000 spokes, one query 574 -> 60 us, 37 queries 716 -> 67;
             // 100 of 200 302 -> 91 and 375 -> 113.
             const int32_t pieces = (qa.vmax - max(n - qcap, 0)) >> 1;     // room for them
