@@ -574,7 +574,12 @@ static int make_plan_core(const eat_net *const *nets, int n_nets, int32_t n, con
     const size_t beside = kSmemBesideL1 / (size_t)blocks - 1024;
     const size_t room = b0 + qbytes * qleast + qpad <= beside ? beside : std::min(limit, d.smem_per_sm / (size_t)blocks - d.reserve);
     size_t cap = room > b0 + qpad ? (room - b0 - qpad) / qbytes : 0;
-    cap = std::min({cap, (size_t)std::max(vmax, 1), p.mem == 0 ? kQueueMost / 2 : kQueueMost});
+    // Alone on its SM beside shared rows, a network of wide levels queues more stops in shared
+    // memory (a queue of 512 spilled most of a round: 1,000 hubs of 20 spokes, 1 / 152 queries
+    // 93 -> 84 / 207 -> 178 us, 20,000 stops joined at random 136 -> 115 / 233 -> 207; with two
+    // blocks per SM it takes from L1: 100 hubs of 200, 160 queries 130 -> 171).
+    const size_t queue_most = p.mem != 0 ? kQueueMost : level > 512 && n <= d.sms ? 2 * kQueueMost : kQueueMost / 2;
+    cap = std::min({cap, (size_t)std::max(vmax, 1), queue_most});
     if (cap >= 64) cap &= ~(size_t)31;
     p.qcap = (int32_t)std::max(cap, qleast);
     p.smem_mask_off = p.mem == 0 ? (int32_t)(arr_bytes / 4) : 0;   // mem 3: after the query's own row
