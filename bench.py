@@ -61,8 +61,8 @@ BYTES = {"vertices": 12, "lookups": 28, "relaxed": 12}
 # cluster width, so that another kernel or launch shape reports null until it is
 # profiled again.
 NCU_TRAFFIC_PER_QUERY = {
-    "large": ("b5fafcd224b20f19", "eat_cta_kernel", 512, 7200, 600, 8606264768 / 1024),
-    "city": ("b5fafcd224b20f19", "eat_cta_kernel", 512, 14400, 600, 49174323 / 256),
+    "large": ("d87cc4c0d59e8183", "eat_cta_kernel", 512, 7200, 600, 8607145536 / 1024),
+    "city": ("d87cc4c0d59e8183", "eat_cta_kernel", 512, 14400, 600, 49245824 / 256),
 }
 KERNEL_OF_MODE = {1: "eat_cta_kernel", 2: "eat_cluster_kernel", 3: "eat_async_kernel",
                   4: "eat_pair_kernel", 5: "eat_cta_kernel"}
